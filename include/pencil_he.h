@@ -86,10 +86,12 @@ int pencil_ctx_primes(const PencilCtx* ctx, uint64_t* primes, uint64_t* psis);
  * multiply-accumulate reading operands straight from L2: 2, 4 or 8; or 0: the
  * shared-memory staged kernel (each CTA stages one input block of 32 slots for
  * a 64-pair output block; each operand word read once per CTA).
- * PENCIL_TUNE_MAC_STAGING (columns 2, 4, 8): 0 = every thread copies its own
- * operand words a few input blocks ahead (cp.async ring); 1 = one producer
- * warp per CTA copies whole 1 KB operand rows with bulk asynchronous copies
- * (cp.async.bulk + mbarrier), the other warps only multiply.
+ * PENCIL_TUNE_MAC_STAGING (columns 2, 4, 8): 0 = integer multiply-adds, every
+ * thread copies its own operand words a few input blocks ahead (cp.async ring);
+ * 1 (default) = exact base-256 digit products on the tensor cores where they are
+ * the faster form for the product's sizes and the primes allow them (2^b - c with
+ * c < 2^(b-32)), else integer multiply-adds with one producer warp per CTA copying
+ * whole 1 KB operand rows (cp.async.bulk + mbarrier).
  * PENCIL_TUNE_NTT_ARITH: butterfly arithmetic of the NTT kernels: 0 = Shoup
  * products with Harvey's lazy butterflies (any prime); 1 = pseudo-Mersenne
  * products (y w = y0 w + y1 (2^32 w mod q), folded with 2^60 = c and

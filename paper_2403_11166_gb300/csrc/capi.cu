@@ -342,6 +342,16 @@ extern "C" int pencil_ctx_create(const PencilParams* params, int device, PencilC
     lc.nqtil = mulmod(lc.ninv, lc.qtil, q);
     lc.nqtils = shoup(lc.nqtil, q);
     lc.a_max = (u64)((((u128)1) << 64) / q * q - 1);
+    lc.sb = 32 - (u32)__builtin_clzll(q);
+    lc.cb = (1ull << (64 - __builtin_clzll(q))) - q;
+    {   // bias of one combination of diagonals (digits.cuh): 0x33000000 sum_{j < 7} 2^(16 j)
+      u64 bias = 0, w = 0x33000000ull % q;
+      for (int i = 0; i < 7; ++i) {
+        bias = (bias + w) % q;
+        w = mulmod(w, (1ull << 16) % q, q);
+      }
+      lc.digit_bias = bias ? q - bias : 0;
+    }
     {
       const u64 w1 = powmod(psi_inv, brv(1u, p.log_n), q);   // the last inverse stage's twiddle
       const u64 ks[2] = {lc.ninv, lc.nqtil};
@@ -367,6 +377,12 @@ extern "C" int pencil_ctx_create(const PencilParams* params, int device, PencilC
     if (qs[j] >= (1ull << 60) || qs[j] <= (1ull << 59) + (1ull << 33) || d.limb[j].c60 >= (1ull << 28) ||
         d.limb[j].c64 >= (1ull << 28))
       d.mac_split = 0;   // (q > 2^59 + 2^33: the accumulator's final value, below 2^60 + 2^33, is below 2 q)
+  d.mac_mma = 1;
+  for (int j = 0; j < d.L; ++j) {
+    const LimbConst& lc = d.limb[j];
+    if (qs[j] < (1ull << 39) || lc.cb >> lc.sb || lc.c64 >> 32) d.mac_mma = 0;
+  }
+  if (cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) d.sms = 152;
   cudaError_t e1 = cudaMalloc(&ctx->tw_fwd, tf.size() * sizeof(ulonglong2));
   cudaError_t e2 = cudaMalloc(&ctx->tw_inv, ti.size() * sizeof(ulonglong2));
   cudaError_t e3 = cudaMalloc(&ctx->status, sizeof(int));
@@ -1092,6 +1108,13 @@ static int alg1_prepare(PencilCtx* ctx, const PencilPlan* P, const u64* x0, cons
 
 // Alg. 1 steps 2-3 on the received ciphertexts: ct_out[m, n] = sum_k
 // (ct_in[m, k] + NTT(Delta x0)[m, k]) pt[k, n] - NTT(Delta s)[m, n], one launch.
+// -(bias of all the combinations of diagonals of one output) mod q_j (digits.cuh)
+static void mac_mma_start(const PencilCtx* ctx, MacParams& M, bool dual) {
+  const u64 combos = (u64)mac_mma_combinations(M.K, dual);
+  for (int j = 0; j < ctx->dev.L; ++j)
+    M.start[j] = mulmod(combos % ctx->primes[j], ctx->dev.limb[j].digit_bias, ctx->primes[j]);
+}
+
 static int alg1_apply(PencilCtx* ctx, const PencilPlan* P, const u64* ct_in, const u64* pt, u64* ct_out, char* ws,
                       cudaStream_t s) {
   const Alg1Ws w = alg1_ws(P, ws);
@@ -1113,6 +1136,7 @@ static int alg1_apply(PencilCtx* ctx, const PencilPlan* P, const u64* ct_in, con
   M.K = (int)P->c.K();
   M.NC = P->c.NC;
   M.lanes = (int)lnw;
+  mac_mma_start(ctx, M, false);
   {
     PROF(ctx, PENCIL_K_MAC, s);
     CUDA_TRY(launch_mac(ctx->dev, M, false, s));
@@ -1251,6 +1275,7 @@ extern "C" int he_linear_backward(PencilCtx* ctx, const PencilPlan* Pd, const Pe
     M.K = (int)Pw->c.K();
     M.NC = Pw->c.NC;
     M.lanes = (int)lnw;
+    mac_mma_start(ctx, M, true);
     {
       PROF(ctx, PENCIL_K_MAC_DUAL, s);
       CUDA_TRY(launch_mac(ctx->dev, M, true, s));
@@ -1727,7 +1752,7 @@ extern "C" int pencil_batch_commit(PencilBatch* B, const PencilSecretKey* sk, vo
   std::vector<CombineP> comb(nl);
   std::vector<MacParams> mac(nl);
   std::vector<int2> it_pt, it_in, it_out, it_sh, it_prep;
-  std::vector<int4> it_mac;
+  std::vector<int4> it_mma, it_mac;   // blocks of digit products, tiles of integer ones
   bool has_dual = false;
   auto add_encode = [&](const Packing& pk, const Accessor& ac, const void* src, u64* dst, long long count) {
     ModeEncode::Params e;
@@ -1823,12 +1848,18 @@ extern "C" int pencil_batch_commit(PencilBatch* B, const PencilSecretKey* sk, vo
     for (long long i = 0; i < P->ct_out; ++i) it_out.push_back(make_int2(l, (int)i));
     for (long long i = 0; i < prep[l].n_in + P->ct_out; ++i) it_prep.push_back(make_int2(l, (int)i));
     for (long long c = 0; c < (P->out_elems + 1023) / 1024; ++c) it_sh.push_back(make_int2(l, (int)c));
-    const int lane_blocks = (int)((lnw + 127) / 128);
-    for (long long m = 0; m < P->c.M(); ++m)
-      for (int n0 = 0; n0 < P->c.NC; n0 += nt)
-        for (int lb = 0; lb < lane_blocks; ++lb) it_mac.push_back(make_int4(l, (int)m, n0, lb));
+    if (mac_mma_wins(ctx->dev, mac[l], wg)) {
+      mac_mma_start(ctx, mac[l], wg);
+      for (long long m = 0; m < P->c.M(); m += PENCIL_BATCH_MMA_ROWS)
+        for (int n0 = 0; n0 < P->c.NC; n0 += PENCIL_BATCH_MMA_COLS) it_mma.push_back(make_int4(l, (int)m, n0, 0));
+    } else {
+      for (long long m = 0; m < P->c.M(); ++m)
+        for (int n0 = 0; n0 < P->c.NC; n0 += nt) it_mac.push_back(make_int4(l, (int)m, n0, 0));
+    }
   }
   if (!ctx->dev.mac_split) return PENCIL_E_UNIMPL;
+  const long long n_mma = (long long)it_mma.size();
+  it_mac.insert(it_mac.begin(), it_mma.begin(), it_mma.end());
   std::vector<char> blob;
   size_t at = 0, o_enc, o_encr, o_prep, o_dec, o_samp, o_mpol, o_mosh, o_comb, o_mac, o_pt, o_in, o_out, o_sh,
          o_iprep, o_imac, o_words;
@@ -1879,7 +1910,8 @@ extern "C" int pencil_batch_commit(PencilBatch* B, const PencilSecretKey* sk, vo
   D.items_share = reinterpret_cast<const int2*>(d + o_sh);
   D.n_share = (long long)it_sh.size();
   D.items_mac = reinterpret_cast<const int4*>(d + o_imac);
-  D.n_mac = (long long)it_mac.size();
+  D.n_mma = n_mma;
+  D.n_split = (long long)it_mac.size() - n_mma;
   D.ready = reinterpret_cast<u64*>(d + o_words);
   D.step = D.ready + nl;
   D.abort_flag = reinterpret_cast<int*>(D.ready + nl + 1);

@@ -29,6 +29,10 @@ struct LimbConst {
   // the one twiddle of that stage; kappa = N^{-1} (sc_ninv) or N^{-1} qtil (sc_nqtil).
   u64 sc_ninv[4];
   u64 sc_nqtil[4];
+  // q = 2^b - cb (digits.cuh; used when DevCtx::mac_mma): cb < 2^(b-32), sb = b - 32
+  u64 cb;
+  u32 sb;
+  u64 digit_bias;    // -(bias of one combination of diagonals) mod q
 };
 
 struct DevCtx {
@@ -48,6 +52,8 @@ struct DevCtx {
   int mac_split;             // 1: every q_j in (2^59 + 2^33, 2^60) with 2^60, 2^64 mod q_j < 2^28 (30-bit split MAC)
   int mac_nt;                // output columns per thread of the split MAC: 2, 4 or 8
   int mac_staging;           // operand staging of the split MAC: 0 per-thread cp.async ring, 1 bulk copies
+  int sms;                   // multiprocessors of the device
+  int mac_mma;               // 1: every q_j = 2^b - c with c < 2^(b-32), 2^64 mod q_j < 2^32 (digit products, digits.cuh)
   u64 q_mod_t;               // (q_total mod t): messages are scaled as round(q_total m / t)
   int flood_bits;            // 0, or the flooding noise of returned ciphertexts: uniform in [-2^b, 2^b)
 };

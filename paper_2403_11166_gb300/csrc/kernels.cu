@@ -7,6 +7,7 @@
 #include <cstdio>
 
 #include "kernels.h"
+#include "mac_mma.cuh"
 
 namespace pencil {
 
@@ -715,7 +716,28 @@ static cudaError_t launch_mac_bulk(const DevCtx& ctx, const MacParams& P0, bool 
   return cudaSuccess;
 }
 
+// Digit products on the tensor cores (mac_mma.cu) against the integer multiply-add
+// kernels, by modelled time of one slot's block in common units.  A tensor-core tile
+// is 16 columns n x 4 rows m (Alg. 2: 8 rows of one component) whatever part of it
+// exists and pays its combination once per chunk of 16 (8) input blocks; the integer
+// kernels pay per existing (m, n) pair and input block.  Fitted to launches on GB300
+// at L N = 24576 (us; tensor cores / k_mac_bulk): M = 30, NC = 64: K = 3 605 / 510,
+// 5 657 / 651, 6 657 / 768, 16 875 / 1542, 32 1582 / 2871; M = 10, NC = 16: K = 6
+// 74 / 72, 8 75 / 84, 16 91 / 138; M = 4, NC = 4: K = 16 36 / 25, 32 65 / 42; M = 2,
+// NC = 64: K = 16 150 / 114.  Two 54-bit primes at N = 4096 (k_mac): M = 10, NC = 16:
+// K = 1 24 / 22, 2 24 / 28, 16 38 / 129.
+bool mac_mma_wins(const DevCtx& ctx, const MacParams& P, bool dual) {
+  if (!ctx.mac_mma || ctx.mac_nt == 0 || ctx.mac_staging != 1) return false;   // not available, or tuned away
+  const double rows = P.M - P.m_base, K = P.K, nt = (P.NC + 15) / 16, pairs = rows * P.NC / 64.0;
+  if (dual)
+    return 2.0 * ((P.M - P.m_base + 7) / 8) * nt * 22.0 * ((P.K + 7) / 8) <
+           pairs * (ctx.mac_split ? 11.0 + 6.0 * K : 15.0 + 13.0 * K);
+  const double unit = P.K <= 16 ? 19.0 + 0.7 * K : 26.0 * ((P.K + 15) / 16);
+  return ((P.M - P.m_base + 3) / 4) * nt * unit < pairs * (ctx.mac_split ? 11.0 + 2.65 * K : 15.0 + 6.6 * K);
+}
+
 cudaError_t launch_mac(const DevCtx& ctx, const MacParams& P0, bool dual, cudaStream_t s) {
+  if (mac_mma_wins(ctx, P0, dual)) return launch_mac_mma(ctx, P0, dual, s);
   if (ctx.mac_split && ctx.mac_nt == 0) return launch_mac_smem(ctx, P0, dual, s);
   if (ctx.mac_split && ctx.mac_staging == 1) {
     switch (ctx.mac_nt) {
@@ -1212,7 +1234,7 @@ cudaError_t launch_lincomb(const LincombP& P, u64 t_mask, cudaStream_t s) {
 // Many linear layers (Alg. 1 forward) with a fixed launch sequence: every stage
 // of every layer runs in one multi-plan launch over (layer, polynomial) items,
 // and the ct x pt products of all layers run in ONE persistent launch over a
-// (layer, m, n-tile, lane-block) work list.  Nothing is allocated or copied at
+// (layer, output block) x slot block work list.  Nothing is allocated or copied at
 // run time, so the sequence can be captured in a CUDA graph; a device step
 // counter re-keys the randomness of every replay.  The persistent
 // multiply-accumulate consumes a layer's inputs only after that layer's ready
@@ -1313,48 +1335,76 @@ __device__ __forceinline__ bool wait_ready(const u64* ready, int layer, u64 want
   return v != 0;
 }
 
-// HAS_DUAL: the batch holds Alg. 2 layers (MacParams::pa set), whose tiles take
-// two products per input block; the ring is then sized for them.
+// Digit products (mac_mma.cuh) of blocks items[0, n_mma) for every 4 slots, then the
+// integer form (mac_split_tile) of tiles items[n_mma, n_mma + n_split) for every 128:
+// each layer is in the form that is faster for its sizes (mac_mma_wins).  HAS_DUAL:
+// the batch holds Alg. 2 layers (MacParams::pa set), two products per input block.
+// 96 uneven layers forward (70 000 products): the whole pass 15.98 ms with the
+// integer form alone (this launch 6.29 ms of it), 13.50 ms with both.
 template <int NT, bool HAS_DUAL>
-__global__ void __launch_bounds__(128) k_mac_persistent(DevCtx ctx, const MacParams* __restrict__ Ps,
-                                                        const int4* __restrict__ items, long long n_items,
-                                                        const u64* ready, const u64* step, int* abort_flag) {
-  extern __shared__ u64 ring[];
+__global__ void __launch_bounds__(MMA_THREADS, NT == 8 ? 2 : 4) k_mac_persistent(const __grid_constant__ DevCtx ctx,
+                                                                   const MacParams* __restrict__ Ps,
+                                                                   const int4* __restrict__ items, long long n_mma,
+                                                                   long long n_split, const u64* ready,
+                                                                   const u64* step, int* abort_flag) {
+  extern __shared__ __align__(16) u64 ring[];
+  constexpr int MT = PENCIL_BATCH_MMA_ROWS, NC = PENCIL_BATCH_MMA_COLS;
   const u64 want = (step ? *step : 0ull) + 1;
-  for (long long i = blockIdx.x; i < n_items; i += gridDim.x) {
-    const int4 it = items[i];   // (layer, m, n0, lane block)
+  const long long lanes = (long long)ctx.L * ctx.n;
+  const long long w1 = n_mma * (lanes / MMA_LANES), total = w1 + n_split * (lanes / MMA_THREADS);
+  for (long long i = blockIdx.x; i < total; i += gridDim.x) {
+    const bool mma = i < w1;
+    const long long j = mma ? i : i - w1, n = mma ? n_mma : n_split, lb = j / n;
+    const int4 it = items[(mma ? 0 : n_mma) + (j - lb * n)];
     if (!wait_ready(ready, it.x, want, ctx.status, abort_flag)) return;
     const MacParams& P = Ps[it.x];
-    const int lane = it.w * blockDim.x + threadIdx.x;
-    if (lane >= P.lanes) continue;
-    if constexpr (HAS_DUAL) {
-      if (P.pa) {
-        mac_split_tile<NT, true>(ctx, P, it.y, it.z, lane, ring, threadIdx.x);
-        continue;
+    if (mma) {
+      if constexpr (HAS_DUAL) {
+        if (P.pa) {
+          mac_mma_block<true, MT, NC>(ctx, P, it.y, it.z, (int)lb * MMA_LANES, ring);
+          continue;
+        }
       }
+      mac_mma_block<false, MT, NC>(ctx, P, it.y, it.z, (int)lb * MMA_LANES, ring);
+    } else {
+      const int lane = (int)lb * MMA_THREADS + threadIdx.x;
+      if constexpr (HAS_DUAL) {
+        if (P.pa) {
+          mac_split_tile<NT, true>(ctx, P, it.y, it.z, lane, ring, threadIdx.x);
+          continue;
+        }
+      }
+      mac_split_tile<NT, false>(ctx, P, it.y, it.z, lane, ring, threadIdx.x);
     }
-    mac_split_tile<NT, false>(ctx, P, it.y, it.z, lane, ring, threadIdx.x);
   }
 }
 
 template <int NT, bool HAS_DUAL>
+static constexpr size_t mac_persistent_smem() {
+  constexpr int MT = PENCIL_BATCH_MMA_ROWS, NC = PENCIL_BATCH_MMA_COLS;
+  constexpr size_t a = MacRing<NT, HAS_DUAL>::bytes(MMA_THREADS), b = MmaTile<false, MT, NC>::bytes(2),
+                   c = HAS_DUAL ? MmaTile<true, MT, NC>::bytes(2) : 0;
+  return a > b ? (a > c ? a : c) : (b > c ? b : c);
+}
+
+template <int NT, bool HAS_DUAL>
 static cudaError_t launch_mac_persistent(const DevCtx& ctx, const BatchDev& B, unsigned grid, cudaStream_t s) {
-  constexpr size_t smem = MacRing<NT, HAS_DUAL>::bytes(128);
+  constexpr size_t smem = mac_persistent_smem<NT, HAS_DUAL>();
   const cudaError_t e =
       cudaFuncSetAttribute(k_mac_persistent<NT, HAS_DUAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_mac_persistent<NT, HAS_DUAL><<<grid, 128, smem, s>>>(ctx, B.mac, B.items_mac, B.n_mac, B.ready, B.step,
-                                                         B.abort_flag);
+  k_mac_persistent<NT, HAS_DUAL><<<grid, MMA_THREADS, smem, s>>>(ctx, B.mac, B.items_mac, B.n_mma, B.n_split, B.ready,
+                                                                 B.step, B.abort_flag);
   return cudaGetLastError();
 }
 
 template <int NT, bool HAS_DUAL>
 static cudaError_t mac_persistent_occupancy(int* per) {
-  constexpr size_t smem = MacRing<NT, HAS_DUAL>::bytes(128);
+  constexpr size_t smem = mac_persistent_smem<NT, HAS_DUAL>();
   const cudaError_t e =
       cudaFuncSetAttribute(k_mac_persistent<NT, HAS_DUAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per, k_mac_persistent<NT, HAS_DUAL>, 128, smem);
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per, k_mac_persistent<NT, HAS_DUAL>, MMA_THREADS, smem);
 }
 
 // ------------------------------------------------------------------ launchers
@@ -1384,8 +1434,9 @@ cudaError_t launch_batch_forward(const DevCtx& ctx, const BatchDev& B, cudaStrea
   }
   k_signal<<<blocks_for(B.n_layers, 128), 128, 0, s>>>(B.ready, B.n_layers, B.withhold, B.step);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if (B.n_mac) {
-    const unsigned grid = (unsigned)std::min<long long>(B.n_mac, (long long)B.mac_blocks);
+  const long long work = B.n_mma * ((long long)ctx.L * n / MMA_LANES) + B.n_split * ((long long)ctx.L * n / MMA_THREADS);
+  if (work) {
+    const unsigned grid = (unsigned)std::min<long long>(work, (long long)B.mac_blocks);
     if (B.has_dual) {
       e = B.mac_nt == 2   ? launch_mac_persistent<2, true>(ctx, B, grid, s)
           : B.mac_nt == 8 ? launch_mac_persistent<8, true>(ctx, B, grid, s)

@@ -28,6 +28,7 @@ struct MacParams {
   int M, K, NC;
   int lanes;
   int m_base;
+  u64 start[PENCIL_MAX_LIMBS];   // digit products: -(bias of all combinations of diagonals) mod q_j (mac_mma_start)
 };
 
 #define PENCIL_LINCOMB_MAX_TERMS 64
@@ -43,6 +44,15 @@ struct LincombP {
 cudaError_t launch_lincomb(const LincombP& P, u64 t_mask, cudaStream_t s);
 
 cudaError_t upload_cdt();
+// Tensor-core form (contexts with mac_mma); P.start from mac_mma_combinations(K, dual) times digit_bias.
+cudaError_t launch_mac_mma(const DevCtx& ctx, const MacParams& P, bool dual, cudaStream_t s);
+// Combinations of diagonals per output: one per 16 input blocks (Alg. 2: per 8).
+inline int mac_mma_combinations(int K, bool dual) { return dual ? (K + 7) / 8 : (K + 15) / 16; }
+// Whether the digit products are the faster form of this product (see kernels.cu).
+bool mac_mma_wins(const DevCtx& ctx, const MacParams& P, bool dual);
+// Rows and columns of a block of the persistent kernel's digit products.
+#define PENCIL_BATCH_MMA_ROWS 8
+#define PENCIL_BATCH_MMA_COLS 16
 cudaError_t launch_mac(const DevCtx& ctx, const MacParams& P, bool dual, cudaStream_t s);
 cudaError_t launch_sample_err(u64 seed, int first, int count, int n, int8_t* out, cudaStream_t s,
                               u64 dom = PENCIL_DOM_E);
@@ -117,10 +127,10 @@ struct BatchDev {
   long long n_prep;
   const int2* items_share;
   long long n_share;
-  const int4* items_mac;
-  long long n_mac;
+  const int4* items_mac;  // (layer, m0, n0, 0): n_mma blocks of digit products, then n_split tiles of integer ones
+  long long n_mma, n_split;
   int mac_blocks;
-  int mac_nt;          // output columns per thread of the persistent multiply-accumulate: 2, 4 or 8
+  int mac_nt;          // output columns per thread of the integer tiles: 2, 4 or 8
   int has_dual;        // some layer is an Alg. 2 weight gradient (two products per input block)
   u64* ready;          // [n_layers]
   u64* step;           // replay counter
