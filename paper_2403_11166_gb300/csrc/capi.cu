@@ -1389,7 +1389,7 @@ extern "C" int pencil_ring_linear(PencilCtx* ctx, const PencilPlan* P, const uin
   R.outs = (long long)P->g.B * P->g.Co * R.Ho * R.Wo;
   R.t_mask = ctx->dev.t_mask;
   PROF(ctx, PENCIL_K_RING, s);
-  CUDA_TRY(launch_ring(R, s));
+  CUDA_TRY(launch_ring(R, ctx->dev.sms, s));
   return PENCIL_OK;
 }
 

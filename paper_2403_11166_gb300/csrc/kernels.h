@@ -77,7 +77,9 @@ struct RingParams {
   long long outs;     // B * Co * Ho * Wo
   u64 t_mask;
 };
-cudaError_t launch_ring(const RingParams& P, cudaStream_t s);
+cudaError_t launch_ring(const RingParams& P, int sms, cudaStream_t s);
+// Tensor-core form (ring_mma.cu).
+cudaError_t launch_ring_mma(const RingParams& P, int sms, cudaStream_t s);
 cudaError_t launch_bias_grad(const u64* g, int B, int Co, long long hw, u64 t_mask, u64* out, cudaStream_t s);
 
 // ---- batched layers: per-layer parameters of the non-NTT stages
