@@ -94,10 +94,12 @@ int pencil_ctx_primes(const PencilCtx* ctx, uint64_t* primes, uint64_t* psis);
  * whole 1 KB operand rows (cp.async.bulk + mbarrier).
  * PENCIL_TUNE_NTT_ARITH: butterfly arithmetic of the NTT kernels: 0 = Shoup
  * products with Harvey's lazy butterflies (any prime); 1 = pseudo-Mersenne
- * products (y w = y0 w + y1 (2^32 w mod q), folded with 2^60 = c and
- * 2^64 = 16 c mod q) with lazily growing values, for contexts whose primes are
- * all q = 2^60 - c with c < 2^24 (every 60-bit parameter set; the default
- * there), PENCIL_E_PARAMS otherwise. */
+ * products of signed lazily growing values (q = 2^b - c: the high word of a split
+ * product is the quotient), the default for contexts whose primes are all q =
+ * 2^60 - c with c < 2^24 (every 60-bit parameter set), PENCIL_E_PARAMS otherwise.
+ * Contexts of shorter pseudo-Mersenne primes (2^b - c, c < 2^(b-33); e.g. two
+ * 54-bit primes) run the same products whatever the knob, which reads 0 there.
+ */
 enum {
   PENCIL_TUNE_NTT_LOG_RADIX = 0,
   PENCIL_TUNE_MAC_COLUMNS = 1,

@@ -94,6 +94,20 @@ static u64 min_root_2n(u64 q, u64 two_n) {
 
 static u64 shoup(u64 w, u64 q) { return (u64)(((u128)w << 64) / q); }
 
+// Split twiddle of mul_split (common.cuh), q = 2^b - c with b = bit length of q: the
+// centred representatives of w and w 2^32 mod q, each as (low b - 32 bits, signed rest).
+static uint4 split_twiddle(u64 w, u64 q) {
+  const int sh = 32 - __builtin_clzll(q);
+  u32 out[4];
+  const u64 v[2] = {w, (u64)(((u128)w << 32) % q)};
+  for (int i = 0; i < 2; ++i) {
+    const i64 x = v[i] > q / 2 ? (i64)v[i] - (i64)q : (i64)v[i];
+    out[2 * i] = (u32)((u64)x & ((1ull << sh) - 1));
+    out[2 * i + 1] = (u32)(int32_t)(x >> sh);
+  }
+  return make_uint4(out[0], out[1], out[2], out[3]);
+}
+
 static unsigned brv(unsigned x, int bits) {
   unsigned r = 0;
   for (int i = 0; i < bits; ++i) {
@@ -157,8 +171,9 @@ struct PencilCtx {
   DevCtx dev;
   ulonglong2* tw_fwd = nullptr;
   ulonglong2* tw_inv = nullptr;
-  ulonglong2* tw_fwd_f = nullptr;   // fold tables (w, w 2^32 mod q), when every prime allows them
-  ulonglong2* tw_inv_f = nullptr;
+  uint4* tw_fwd_f = nullptr;        // split tables (mul_split), when every prime allows them
+  uint4* tw_inv_f = nullptr;
+  bool arith_knob = false;          // PENCIL_TUNE_NTT_ARITH is open (every prime 2^60 - c)
   int* status = nullptr;
   void* noalloc_addr = nullptr;     // device address of encrypt_share_noalloc's static scratch (this context's)
 };
@@ -301,10 +316,17 @@ extern "C" int pencil_ctx_create(const PencilParams* params, int device, PencilC
   d.t_bits = p.t_bits;
   d.t_mask = (1ull << p.t_bits) - 1;
   std::vector<ulonglong2> tf((size_t)d.L * n), ti((size_t)d.L * n);
-  // pseudo-Mersenne fold butterflies need q_j = 2^60 - c with c < 2^24 for every limb
-  bool fold_ok = true;
-  for (u64 q : qs) fold_ok = fold_ok && q < (1ull << 60) && q > (1ull << 60) - (1ull << 24);
-  std::vector<ulonglong2> tff(fold_ok ? (size_t)d.L * n : 0), tif(fold_ok ? (size_t)d.L * n : 0);
+  // split butterflies (mul_split) need q_j = 2^b - c with c < 2^24 (b = 59, 60) or
+  // c < 2^(b-33) for every limb; the arithmetic knob is open for b = 60 only
+  bool fold_ok = true, fold60 = true;
+  for (u64 q : qs) {
+    const int b = 64 - __builtin_clzll(q);
+    const u64 c = (1ull << b) - q;
+    fold_ok = fold_ok && b >= 40 && c < (b >= 59 ? 1ull << 24 : 1ull << (b - 33));
+    fold60 = fold60 && b == 60 && c < (1ull << 24);
+  }
+  ctx->arith_knob = fold60;
+  std::vector<uint4> tff(fold_ok ? (size_t)d.L * n : 0), tif(fold_ok ? (size_t)d.L * n : 0);
   for (int j = 0; j < d.L; ++j) {
     const u64 q = qs[j];
     const u64 psi = min_root_2n(q, 2ull * n);
@@ -316,8 +338,8 @@ extern "C" int pencil_ctx_create(const PencilParams* params, int device, PencilC
       tf[(size_t)j * n + k] = make_ulonglong2(w, shoup(w, q));
       ti[(size_t)j * n + k] = make_ulonglong2(wi, shoup(wi, q));
       if (fold_ok) {
-        tff[(size_t)j * n + k] = make_ulonglong2(w, (u64)((((u128)w) << 32) % q));
-        tif[(size_t)j * n + k] = make_ulonglong2(wi, (u64)((((u128)wi) << 32) % q));
+        tff[(size_t)j * n + k] = split_twiddle(w, q);
+        tif[(size_t)j * n + k] = split_twiddle(wi, q);
       }
     }
     LimbConst& lc = d.limb[j];
@@ -355,13 +377,10 @@ extern "C" int pencil_ctx_create(const PencilParams* params, int device, PencilC
     {
       const u64 w1 = powmod(psi_inv, brv(1u, p.log_n), q);   // the last inverse stage's twiddle
       const u64 ks[2] = {lc.ninv, lc.nqtil};
-      u64* dst[2] = {lc.sc_ninv, lc.sc_nqtil};
-      for (int i = 0; i < 2; ++i) {
-        const u64 wk = mulmod(w1, ks[i], q);
-        dst[i][0] = ks[i];
-        dst[i][1] = (u64)((((u128)ks[i]) << 32) % q);
-        dst[i][2] = wk;
-        dst[i][3] = (u64)((((u128)wk) << 32) % q);
+      uint4* dst[2] = {lc.sc_ninv, lc.sc_nqtil};
+      for (int i = 0; fold_ok && i < 2; ++i) {
+        dst[i][0] = split_twiddle(ks[i], q);
+        dst[i][1] = split_twiddle(mulmod(w1, ks[i], q), q);
       }
     }
   }
@@ -386,17 +405,17 @@ extern "C" int pencil_ctx_create(const PencilParams* params, int device, PencilC
   cudaError_t e1 = cudaMalloc(&ctx->tw_fwd, tf.size() * sizeof(ulonglong2));
   cudaError_t e2 = cudaMalloc(&ctx->tw_inv, ti.size() * sizeof(ulonglong2));
   cudaError_t e3 = cudaMalloc(&ctx->status, sizeof(int));
-  cudaError_t e4 = fold_ok ? cudaMalloc(&ctx->tw_fwd_f, tff.size() * sizeof(ulonglong2)) : cudaSuccess;
-  cudaError_t e5 = fold_ok ? cudaMalloc(&ctx->tw_inv_f, tif.size() * sizeof(ulonglong2)) : cudaSuccess;
+  cudaError_t e4 = fold_ok ? cudaMalloc(&ctx->tw_fwd_f, tff.size() * sizeof(uint4)) : cudaSuccess;
+  cudaError_t e5 = fold_ok ? cudaMalloc(&ctx->tw_inv_f, tif.size() * sizeof(uint4)) : cudaSuccess;
   if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess || e4 != cudaSuccess || e5 != cudaSuccess) {
     pencil_ctx_destroy(ctx);
     return PENCIL_E_CUDA;
   }
   if (cudaMemcpy(ctx->tw_fwd, tf.data(), tf.size() * sizeof(ulonglong2), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(ctx->tw_inv, ti.data(), ti.size() * sizeof(ulonglong2), cudaMemcpyHostToDevice) != cudaSuccess ||
-      (fold_ok && cudaMemcpy(ctx->tw_fwd_f, tff.data(), tff.size() * sizeof(ulonglong2), cudaMemcpyHostToDevice) !=
+      (fold_ok && cudaMemcpy(ctx->tw_fwd_f, tff.data(), tff.size() * sizeof(uint4), cudaMemcpyHostToDevice) !=
                       cudaSuccess) ||
-      (fold_ok && cudaMemcpy(ctx->tw_inv_f, tif.data(), tif.size() * sizeof(ulonglong2), cudaMemcpyHostToDevice) !=
+      (fold_ok && cudaMemcpy(ctx->tw_inv_f, tif.data(), tif.size() * sizeof(uint4), cudaMemcpyHostToDevice) !=
                       cudaSuccess) ||
       cudaMemset(ctx->status, 0, sizeof(int)) != cudaSuccess || upload_cdt() != cudaSuccess) {
     pencil_ctx_destroy(ctx);
@@ -407,7 +426,7 @@ extern "C" int pencil_ctx_create(const PencilParams* params, int device, PencilC
   d.tw_fwd_f = ctx->tw_fwd_f;
   d.tw_inv_f = ctx->tw_inv_f;
   d.ntt_arith = fold_ok ? 1 : 0;
-  if (fold_ok) d.ntt_loge = 4;   // fold engine: radix 2^4 at every N (N = 16384: 1024-thread CTAs, measured faster)
+  if (fold_ok) d.ntt_loge = 4;   // split engine: radix 2^4 at every N (N = 16384: 1024-thread CTAs, measured faster)
   d.status = ctx->status;
   *out = ctx;
   return PENCIL_OK;
@@ -458,8 +477,8 @@ extern "C" int pencil_ctx_tune(PencilCtx* ctx, int32_t knob, int32_t value) {
   }
   if (knob == PENCIL_TUNE_NTT_ARITH) {
     if (value != 0 && value != 1) return PENCIL_E_ARG;
-    if (value == 1 && !ctx->tw_fwd_f) return PENCIL_E_PARAMS;   // some prime is not 2^60 - c, c < 2^24
-    ctx->dev.ntt_arith = value;
+    if (value == 1 && !ctx->arith_knob) return PENCIL_E_PARAMS;   // some prime is not 2^60 - c, c < 2^24
+    if (ctx->arith_knob) ctx->dev.ntt_arith = value;
     return PENCIL_OK;
   }
   return PENCIL_E_ARG;
@@ -487,7 +506,7 @@ extern "C" int pencil_ctx_get_tune(const PencilCtx* ctx, int32_t knob, int32_t* 
     return PENCIL_OK;
   }
   if (knob == PENCIL_TUNE_NTT_ARITH) {
-    *value = ctx->dev.ntt_arith;
+    *value = ctx->arith_knob ? ctx->dev.ntt_arith : 0;
     return PENCIL_OK;
   }
   if (knob == PENCIL_TUNE_MAC_STAGING) {

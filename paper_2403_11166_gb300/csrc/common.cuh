@@ -24,12 +24,12 @@ struct LimbConst {
   u64 c60, c64;      // 2^60 mod q and 2^64 mod q                 (split multiply-accumulate folds)
   u64 nqtil, nqtils; // N^{-1} qtil mod q_j                       (INTT scaling folded into the CRT factor)
   u64 a_max;         // floor(2^64 / q) q - 1: the largest 64-bit word accepted for a uniform residue
-  // Final scaling kappa of an inverse transform merged into its last stage (fold
-  // engine): {kappa, kappa 2^32, w1 kappa, w1 kappa 2^32} mod q, w1 = psi^-brv(1)
-  // the one twiddle of that stage; kappa = N^{-1} (sc_ninv) or N^{-1} qtil (sc_nqtil).
-  u64 sc_ninv[4];
-  u64 sc_nqtil[4];
-  // q = 2^b - cb (digits.cuh; used when DevCtx::mac_mma): cb < 2^(b-32), sb = b - 32
+  // Final scaling kappa of an inverse transform merged into its last stage (split
+  // engine): the split twiddles (mul_split) kappa and w1 kappa, w1 = psi^-brv(1) the
+  // one twiddle of that stage; kappa = N^{-1} (sc_ninv) or N^{-1} qtil (sc_nqtil).
+  uint4 sc_ninv[2];
+  uint4 sc_nqtil[2];
+  // q = 2^b - cb, sb = b - 32 (mul_split; digits.cuh)
   u64 cb;
   u32 sb;
   u64 digit_bias;    // -(bias of one combination of diagonals) mod q
@@ -45,9 +45,9 @@ struct DevCtx {
   LimbConst limb[PENCIL_MAX_LIMBS];
   const ulonglong2* tw_fwd;  // [L][N] (psi^brv(k), Shoup companion)
   const ulonglong2* tw_inv;  // [L][N] (psi^-brv(k), Shoup companion)
-  int ntt_arith;             // butterflies of the NTT kernels: 0 Shoup / Harvey, 1 pseudo-Mersenne folds
-  const ulonglong2* tw_fwd_f;  // [L][N] (psi^brv(k), psi^brv(k) 2^32 mod q)   (null unless every
-  const ulonglong2* tw_inv_f;  // [L][N] (psi^-brv(k), psi^-brv(k) 2^32 mod q)  q_j = 2^60 - c, c < 2^24)
+  int ntt_arith;             // butterflies of the NTT kernels: 0 Shoup / Harvey, 1 signed split products
+  const uint4* tw_fwd_f;     // [L][N] split psi^brv(k) (mul_split)    (null unless every
+  const uint4* tw_inv_f;     // [L][N] split psi^-brv(k)                q_j allows them)
   int* status;               // device status word (atomicOr of error bits)
   int mac_split;             // 1: every q_j in (2^59 + 2^33, 2^60) with 2^60, 2^64 mod q_j < 2^28 (30-bit split MAC)
   int mac_nt;                // output columns per thread of the split MAC: 2, 4 or 8
@@ -201,104 +201,97 @@ __device__ __forceinline__ void gs_butterfly(u64& x, u64& y, u64 w, u64 ws, u64 
 }
 
 // ------------------------------------------------------------------ pseudo-Mersenne twiddle products
-// For q = 2^60 - c with c < 2^24 (every prime of the 60-bit parameter sets):
-// 2^60 = c60 = c and 2^64 = c64 = 16 c (mod q).  Beside each twiddle w the table
-// holds w32 = w 2^32 mod q, so that for y = y1 2^32 + y0 (any y < 2^64)
-//   y w = y0 w + y1 w32 (mod q),
-// a sum S < 2^93 of four 32x32->64 partial products (no quotient estimate).  With
-// S = sh 2^64 + sm 2^60 + sl (sh <= 2^29 + 1, sm < 16, sl < 2^60) the folds
-//   S = sl + sm c60 + sh c64 (mod q) < 2^60 + 2^57 + 2^30 < 1.13 q
-// leave a lazy residue; the product is six 32x32->64 multiply-adds and seven
-// 32-bit ALU operations, against six such products, four 32-bit multiply-adds
-// and the correction of a Shoup product (measured with pencil_mul_probe's
-// counters: a Shoup product occupies the multiply pipe 34 cycles per warp).
-// Written as one PTX block so that every 64-bit addend of a 32x32->64
-// multiply-add is a register pair that a previous multiply produced (addends
-// assembled from 32-bit halves cost register moves: measured 30.6 -> 25.0
-// instructions per warp of butterflies in the N = 8192 forward transform).
-//   h = y1 w32h + y0 wh (< 2^61),  l = y0 wl,  m = y1 w32l,
-//   S = l + m + 2^32 h = u 2^64 + t 2^32 + s0   (one 32-bit carry chain),
-//   sm = t >> 28, sl = (t mod 2^28) 2^32 + s0, sh = u.
-__device__ __forceinline__ u64 mul_fold(u64 y, u64 w, u64 w32, u32 c60, u32 c64) {
+// For q = 2^b - c (c < 2^24 for b = 59, 60, c < 2^(b-33) below) and signed lazy values
+// |y| < 8 2^b.  A twiddle w is kept as its centred representative and that of
+// w 2^32 mod q, each split at bit sh = b - 32: w = w1 2^sh + w0 with 0 <= w0 < 2^sh
+// and w1 a signed 32-bit word.  With y = y1 2^32 + y0, y0 the SIGNED low word (y1 takes
+// its carry), and v the split of w 2^32:
+//   H = y0 w1 + y1 v1,  L = y0 w0 + y1 v0     (|H| < 2^63, four signed 32x32->64),
+//   y w = L + H 2^sh = L + lo32(H) 2^sh + hi32(H) 2^b = L + lo32(H) 2^sh + hi32(H) c  (mod q):
+// the high word of H is the quotient and its low word sits at bit sh, so nothing is
+// split by shifts and masks and no quotient is estimated: five wide multiply-adds, two
+// shifts, three additions.  The value is signed, for y in [-A, B] (units of 2^b)
+// between -(1/2 + A/16 + 1/32) and 3/2 + B/16 + 1/32.  (The unsigned form it replaces
+// split w at bit 32 and needed fourteen instructions; measured in registers, a forward
+// butterfly with its share of the folds takes 30.0 cycles per warp against 36.7; the low
+// word's shift as a sixth wide multiply-add 32.5.)
+struct FoldC {
+  u32 c, sh, sr, m;   // c, b - 32, 64 - b, 2^(b-32) - 1
+  __device__ __forceinline__ explicit FoldC(const LimbConst& lc)
+      : c((u32)lc.cb), sh(lc.sb), sr(32u - lc.sb), m((1u << lc.sb) - 1u) {}
+};
+
+// base + y w (mod q), lazily.
+__device__ __forceinline__ u64 mul_split(u64 base, u64 y, const uint4 w, const FoldC& f) {
   u64 r;
   asm("{\n\t"
-      ".reg .u64 h, l, m, p;\n\t"
-      ".reg .u32 y0, y1, w0, w1, v0, v1, l0, l1, m0, m1, h0, h1, s0, t, u, sm, tl;\n\t"
-      "mov.b64 {y0, y1}, %1;\n\t"
-      "mov.b64 {w0, w1}, %2;\n\t"
-      "mov.b64 {v0, v1}, %3;\n\t"
-      "mul.wide.u32 h, y1, v1;\n\t"
-      "mad.wide.u32 h, y0, w1, h;\n\t"
-      "mul.wide.u32 l, y0, w0;\n\t"
-      "mul.wide.u32 m, y1, v0;\n\t"
-      "mov.b64 {l0, l1}, l;\n\t"
-      "mov.b64 {m0, m1}, m;\n\t"
+      ".reg .u32 y0, y1, s, h0, h1, a, b;\n\t"
+      ".reg .u64 l, h, g;\n\t"
+      "mov.b64 {y0, y1}, %2;\n\t"
+      "shr.u32 s, y0, 31;\n\t"
+      "add.u32 y1, y1, s;\n\t"
+      "mul.wide.s32 h, y0, %4;\n\t"
+      "mad.wide.s32 h, y1, %6, h;\n\t"
+      "mad.wide.s32 l, y0, %3, %1;\n\t"
+      "mad.wide.s32 l, y1, %5, l;\n\t"
       "mov.b64 {h0, h1}, h;\n\t"
-      "add.cc.u32 s0, l0, m0;\n\t"
-      "addc.cc.u32 t, l1, m1;\n\t"
-      "addc.u32 u, h1, 0;\n\t"
-      "add.cc.u32 t, t, h0;\n\t"
-      "addc.u32 u, u, 0;\n\t"
-      "shr.u32 sm, t, 28;\n\t"
-      "and.b32 tl, t, 0x0FFFFFFF;\n\t"
-      "mad.lo.cc.u32 s0, sm, %4, s0;\n\t"
-      "addc.u32 tl, tl, 0;\n\t"
-      "mov.b64 p, {s0, tl};\n\t"
-      "mad.wide.u32 %0, u, %5, p;\n\t"
+      "mad.wide.s32 l, h1, %7, l;\n\t"
+      "shl.b32 a, h0, %8;\n\t"
+      "shr.u32 b, h0, %9;\n\t"
+      "mov.b64 g, {a, b};\n\t"
+      "add.u64 %0, l, g;\n\t"
       "}"
       : "=l"(r)
-      : "l"(y), "l"(w), "l"(w32), "r"(c60), "r"(c64));
+      : "l"(base), "l"(y), "r"(w.x), "r"(w.y), "r"(w.z), "r"(w.w), "r"(f.c), "r"(f.sh), "r"(f.sr));
   return r;
 }
 
-// The same product in plain C (the reference form of the PTX above; the
-// multiply probe times both).
-__device__ __forceinline__ u64 mul_fold_c(u64 y, u64 w, u64 w32, u32 c60, u32 c64) {
-  const u32 y0 = (u32)y, y1 = (u32)(y >> 32);
-  // S = y0 wl + y1 w32l + 2^32 (y0 wh + y1 w32h)   (l, h: low and high 32-bit halves)
-  const u64 p1 = (u64)y1 * (u32)w32;                           // y1 w32l
-  const u64 p0 = (u64)y0 * (u32)w + (u32)p1;                   // y0 wl + lo(p1) < 2^64 - 2^32
-  u64 m = (u64)y1 * (u32)(w32 >> 32) + (p1 >> 32);             // < 2^60 + 2^32
-  m = (u64)y0 * (u32)(w >> 32) + m;                            // < 2^61 + 2^32
-  m += p0 >> 32;                                               // S = m 2^32 + lo(p0), m < 2^61 + 2^33
-  const u32 ml = (u32)m;
-  const u64 t = (u64)(ml >> 28) * c60 + (((u64)(ml & 0x0FFFFFFFu) << 32) | (u32)p0);   // sl + sm c60
-  return (u64)(u32)(m >> 32) * c64 + t;                                                 // + sh c64
-}
-
-// v mod q, lazily: any v < 2^64 -> (v mod 2^60) + (v >> 60) c60 < 2^60 + 2^32 (< 2 q).
-// (v >> 60) c60 < 2^32 (c60 < 2^28): a 32-bit multiply-add with carry, not a
-// 32x32->64 one (which holds the multiply pipe twice as long).
-__device__ __forceinline__ u64 fold60(u64 v, u32 c60) {
+// Signed lazy value, |v| < 2^63 -> (v mod 2^b) + floor(v / 2^b) c, within 2^-7 of [0, 2^b].
+__device__ __forceinline__ u64 fold_s(u64 v, const FoldC& f) {
   u64 r;
   asm("{\n\t"
-      ".reg .u32 v0, v1, s, h;\n\t"
+      ".reg .u32 v0, v1, s, h;\n\t.reg .u64 p;\n\t"
       "mov.b64 {v0, v1}, %1;\n\t"
-      "shr.u32 s, v1, 28;\n\t"
-      "and.b32 h, v1, 0x0FFFFFFF;\n\t"
-      "mad.lo.cc.u32 v0, s, %2, v0;\n\t"
-      "addc.u32 h, h, 0;\n\t"
-      "mov.b64 %0, {v0, h};\n\t"
+      "shr.s32 s, v1, %3;\n\t"
+      "and.b32 h, v1, %4;\n\t"
+      "mov.b64 p, {v0, h};\n\t"
+      "mad.wide.s32 %0, s, %2, p;\n\t"
       "}"
       : "=l"(r)
-      : "l"(v), "r"(c60));
+      : "l"(v), "r"(f.c), "r"(f.sh), "r"(f.m));
   return r;
 }
 
-// Cooley-Tukey butterfly with a lazy pseudo-Mersenne product: x, y < B q ->
-// x + w y < (B + 1.13) q, x - w y + 2 q < (B + 2) q (no correction step).
-__device__ __forceinline__ void ct_fold(u64& x, u64& y, const ulonglong2 w, u32 c60, u32 c64, u64 q2) {
-  const u64 t = mul_fold(y, w.x, w.y, c60, c64);
-  y = x + q2 - t;
+// The same for an unsigned value below 2^64: below 2^b + 2^(64-b) c < 2 q.
+__device__ __forceinline__ u64 fold_u(u64 v, const FoldC& f) {
+  u64 r;
+  asm("{\n\t"
+      ".reg .u32 v0, v1, s, h;\n\t.reg .u64 p;\n\t"
+      "mov.b64 {v0, v1}, %1;\n\t"
+      "shr.u32 s, v1, %3;\n\t"
+      "and.b32 h, v1, %4;\n\t"
+      "mov.b64 p, {v0, h};\n\t"
+      "mad.wide.u32 %0, s, %2, p;\n\t"
+      "}"
+      : "=l"(r)
+      : "l"(v), "r"(f.c), "r"(f.sh), "r"(f.m));
+  return r;
+}
+
+// Cooley-Tukey butterfly on signed lazy values: x + w y, x - w y.  From [0, 1] (units
+// of 2^b) four stages stay inside (-6.96, 7.96): one fold per round of at most four.
+__device__ __forceinline__ void ct_split(u64& x, u64& y, const uint4 w, const FoldC& f) {
+  const u64 t = mul_split(0, y, w, f);
+  y = x - t;
   x = x + t;
 }
 
-// Gentleman-Sande butterfly: x, y < B q <= cq, cq + B q < 2^64 ->
-// x + y < 2 B q, (x - y + cq) w < 1.13 q.
-__device__ __forceinline__ void gs_fold(u64& x, u64& y, const ulonglong2 w, u32 c60, u32 c64, u64 cq) {
-  const u64 d = x + cq - y;
+// Gentleman-Sande butterfly: x + y, (x - y) w.  From [-0.87, 1.87], two stages with the
+// second one's sums folded stay inside (-3.5, 7.5) and return to that range.
+__device__ __forceinline__ void gs_split(u64& x, u64& y, const uint4 w, const FoldC& f) {
+  const u64 d = x - y;
   x = x + y;
-  y = mul_fold(d, w.x, w.y, c60, c64);
+  y = mul_split(0, d, w, f);
 }
 
 // [0, 8q) -> [0, q)

@@ -236,15 +236,18 @@ __device__ __forceinline__ void ntt_inv_run(const DevCtx& ctx, const typename Mo
 }
 
 // ------------------------------------------------------------------ pseudo-Mersenne engine
-// The same transforms for primes q = 2^60 - c (c < 2^24) with ct_fold / gs_fold
-// butterflies (common.cuh): no correction step inside a butterfly; values grow
-// lazily and are folded (fold60) only where the bound requires it:
-//  * forward: a stage adds less than 2q to the bound, so the registers are
-//    folded once per round of at most 5 stages (bound < 11.01 q < 2^64) and
-//    brought to [0, q) (fold, one conditional subtraction) before the epilogue;
-//  * inverse: a stage doubles the bound of its sums, so the sums of every
-//    second stage (counted from the first inverse stage) are folded; inputs
-//    stay below 2.26 q and the subtraction constant is 2q or 4q.
+// The same transforms for primes q = 2^b - c with signed split products (mul_split,
+// common.cuh): no correction step inside a butterfly and no added multiple of q;
+// signed values grow lazily and are folded only where the bound requires it
+// (units of 2^b):
+//  * forward: from [0, 1], k = 1 .. 4 stages stay inside -(1.59, 3.27, 5.06, 6.96) ..
+//    (2.59, 4.27, 6.06, 7.96), so the registers are folded once per round of at most
+//    four stages (rounds of five fold after their second stage too); before the last
+//    fold 4 q (at most two stages) or 8 q is added, so that it is unsigned and one
+//    conditional subtraction is canonical;
+//  * inverse: a stage doubles the range of its sums, so the sums of every second
+//    stage (counted from the first inverse stage) are folded; the last stage's
+//    products (its scaling) start from 2 q, which makes them positive.
 // Shared memory holds the N words with two spare words after every 32
 // (slot ph(x)): every round's accesses are conflict-free and a thread's words of
 // one round sit at compile-time offsets from one base address.  The last
@@ -324,29 +327,30 @@ struct FRound {
   }
   // Stage J of the round (global stage S0 + J), forward.
   template <int J>
-  static __device__ __forceinline__ void fwd_stage(u64 (&v)[E], const ulonglong2* __restrict__ tw, int tau, u32 c60,
-                                                   u32 c64, u64 q2) {
+  static __device__ __forceinline__ void fwd_stage(u64 (&v)[E], const uint4* __restrict__ tw, int tau, const FoldC& f) {
     constexpr int half = 1 << (K - 1 - J);
 #pragma unroll
     for (int gg = 0; gg < G; ++gg) {
       const int B = grp(tau, gg) >> LOGD;
 #pragma unroll
       for (int i = 0; i < (1 << J); ++i) {
-        const ulonglong2 w = __ldg(tw + (1 << (S0 + J)) + (B << J) + i);
+        const uint4 w = __ldg(tw + (1 << (S0 + J)) + (B << J) + i);
 #pragma unroll
         for (int r = 0; r < half; ++r) {
           const int l = gg * (1 << K) + i * 2 * half + r;
-          ct_fold(v[l], v[l + half], w, c60, c64, q2);
+          ct_split(v[l], v[l + half], w, f);
         }
       }
     }
+    if constexpr (K == 5 && J == 1) {   // five stages from [0, 1] would leave 64 bits
+#pragma unroll
+      for (int l = 0; l < E; ++l) v[l] = fold_s(v[l], f);
+    }
   }
-  // Stage J of the round, inverse; `step` = its position in the inverse order
-  // (LOGN - 1 - (S0 + J)): even steps subtract against 2q, odd ones against 4q
-  // and fold their sums.
+  // Stage J of the round, inverse; the stages at odd positions of the inverse order
+  // (LOGN - 1 - (S0 + J)) fold their sums.
   template <int J>
-  static __device__ __forceinline__ void inv_stage(u64 (&v)[E], const ulonglong2* __restrict__ tw, int tau, u32 c60,
-                                                   u32 c64, u64 q2, u64 q4) {
+  static __device__ __forceinline__ void inv_stage(u64 (&v)[E], const uint4* __restrict__ tw, int tau, const FoldC& f) {
     constexpr int half = 1 << (K - 1 - J);
     constexpr bool odd = ((LOGN - 1 - (S0 + J)) & 1) != 0;
 #pragma unroll
@@ -354,63 +358,58 @@ struct FRound {
       const int B = grp(tau, gg) >> LOGD;
 #pragma unroll
       for (int i = 0; i < (1 << J); ++i) {
-        const ulonglong2 w = __ldg(tw + (1 << (S0 + J)) + (B << J) + i);
+        const uint4 w = __ldg(tw + (1 << (S0 + J)) + (B << J) + i);
 #pragma unroll
         for (int r = 0; r < half; ++r) {
           const int l = gg * (1 << K) + i * 2 * half + r;
-          gs_fold(v[l], v[l + half], w, c60, c64, odd ? q4 : q2);
-          if constexpr (odd) v[l] = fold60(v[l], c60);
+          gs_split(v[l], v[l + half], w, f);
+          if constexpr (odd) v[l] = fold_s(v[l], f);
         }
       }
     }
   }
   template <int... J>
   static __device__ __forceinline__ void fwd_seq(std::integer_sequence<int, J...>, u64 (&v)[E],
-                                                 const ulonglong2* tw, int tau, u32 c60, u32 c64, u64 q2) {
-    (fwd_stage<J>(v, tw, tau, c60, c64, q2), ...);
+                                                 const uint4* tw, int tau, const FoldC& f) {
+    (fwd_stage<J>(v, tw, tau, f), ...);
   }
   // Round 0 of the inverse with the transform's final scaling kappa merged into
   // its last stage (global stage 0, whose butterflies all use w1 = tw[1]):
-  //   x' = (x + y) kappa,  y' = (x - y + cq) (w1 kappa),  both < 1.13 q,
+  //   x' = (x + y) kappa + 2 q,  y' = (x - y) (w1 kappa) + 2 q,  both in (0.9 q, 4.1 q),
   // N / 2 products instead of the stage's N / 2 and the N of a separate scaling.
-  // sc = {kappa, kappa 2^32, w1 kappa, w1 kappa 2^32} mod q.
-  static __device__ __forceinline__ void inv_scaled(u64 (&v)[E], const ulonglong2* tw, int tau, u32 c60, u32 c64,
-                                                    u64 q2, u64 q4, const u64* sc) {
+  // sc = split twiddles {kappa, w1 kappa}.
+  static __device__ __forceinline__ void inv_scaled(u64 (&v)[E], const uint4* tw, int tau, const FoldC& f, u64 q2,
+                                                    const uint4* sc) {
     static_assert(S0 == 0 && G == 1 && K == LOGE, "the first round, full");
-    inv_seq(std::make_integer_sequence<int, K - 1>{}, v, tw, tau, c60, c64, q2, q4, 1);
-    constexpr bool odd = ((LOGN - 1) & 1) != 0;   // the subtraction constant of inverse step LOGN - 1
-    const u64 cq = odd ? q4 : q2;
-    const u64 k = sc[0], k32 = sc[1], wk = sc[2], wk32 = sc[3];
+    inv_seq(std::make_integer_sequence<int, K - 1>{}, v, tw, tau, f, 1);
+    const uint4 k = sc[0], wk = sc[1];
 #pragma unroll
     for (int r = 0; r < E / 2; ++r) {
       const u64 x = v[r], y = v[r + E / 2];
-      v[r] = mul_fold(x + y, k, k32, c60, c64);
-      v[r + E / 2] = mul_fold(x + cq - y, wk, wk32, c60, c64);
+      v[r] = mul_split(q2, x + y, k, f);
+      v[r + E / 2] = mul_split(q2, x - y, wk, f);
     }
   }
   // Stages K - 1 .. 0 (inverse order), or K - 1 .. 1 with sizeof...(J) = K - 1.
   template <int... J>
   static __device__ __forceinline__ void inv_seq(std::integer_sequence<int, J...>, u64 (&v)[E],
-                                                 const ulonglong2* tw, int tau, u32 c60, u32 c64, u64 q2, u64 q4,
-                                                 int = 0) {
-    (inv_stage<K - 1 - J>(v, tw, tau, c60, c64, q2, q4), ...);
+                                                 const uint4* tw, int tau, const FoldC& f, int = 0) {
+    (inv_stage<K - 1 - J>(v, tw, tau, f), ...);
   }
-  static __device__ __forceinline__ void fwd(u64 (&v)[E], const ulonglong2* tw, int tau, u32 c60, u32 c64, u64 q2) {
-    fwd_seq(std::make_integer_sequence<int, K>{}, v, tw, tau, c60, c64, q2);
+  static __device__ __forceinline__ void fwd(u64 (&v)[E], const uint4* tw, int tau, const FoldC& f) {
+    fwd_seq(std::make_integer_sequence<int, K>{}, v, tw, tau, f);
   }
   // Stages j0 .. K - 1 only (j0 uniform across the CTA).
   template <int... J>
   static __device__ __forceinline__ void fwd_from_seq(std::integer_sequence<int, J...>, int j0, u64 (&v)[E],
-                                                      const ulonglong2* tw, int tau, u32 c60, u32 c64, u64 q2) {
-    ((J >= j0 ? fwd_stage<J>(v, tw, tau, c60, c64, q2) : void()), ...);
+                                                      const uint4* tw, int tau, const FoldC& f) {
+    ((J >= j0 ? fwd_stage<J>(v, tw, tau, f) : void()), ...);
   }
-  static __device__ __forceinline__ void fwd_from(int j0, u64 (&v)[E], const ulonglong2* tw, int tau, u32 c60,
-                                                  u32 c64, u64 q2) {
-    fwd_from_seq(std::make_integer_sequence<int, K>{}, j0, v, tw, tau, c60, c64, q2);
+  static __device__ __forceinline__ void fwd_from(int j0, u64 (&v)[E], const uint4* tw, int tau, const FoldC& f) {
+    fwd_from_seq(std::make_integer_sequence<int, K>{}, j0, v, tw, tau, f);
   }
-  static __device__ __forceinline__ void inv(u64 (&v)[E], const ulonglong2* tw, int tau, u32 c60, u32 c64, u64 q2,
-                                             u64 q4) {
-    inv_seq(std::make_integer_sequence<int, K>{}, v, tw, tau, c60, c64, q2, q4);
+  static __device__ __forceinline__ void inv(u64 (&v)[E], const uint4* tw, int tau, const FoldC& f) {
+    inv_seq(std::make_integer_sequence<int, K>{}, v, tw, tau, f);
   }
 };
 
@@ -419,17 +418,16 @@ struct FRound {
 // shared memory.  Each round folds its words and leaves them in shared memory.
 template <int LOGN, int LOGE, int S0>
 struct FFwdRounds {
-  static __device__ __forceinline__ void run(u64 (&v)[1 << LOGE], u64* sm, const ulonglong2* tw, int tau, u32 c60,
-                                             u32 c64, u64 q2) {
+  static __device__ __forceinline__ void run(u64 (&v)[1 << LOGE], u64* sm, const uint4* tw, int tau, const FoldC& f) {
     using Rd = FRound<LOGN, LOGE, S0>;
     if constexpr (S0 > 0) Rd::load(v, sm, tau);
-    Rd::fwd(v, tw, tau, c60, c64, q2);
+    Rd::fwd(v, tw, tau, f);
 #pragma unroll
-    for (int l = 0; l < (1 << LOGE); ++l) v[l] = fold60(v[l], c60);
+    for (int l = 0; l < (1 << LOGE); ++l) v[l] = fold_s(v[l], f);
     if constexpr (S0 > 0) phase_sync<Rd::kLocal>();   // every reader of these slots is done
     Rd::store(v, sm, tau);
     phase_sync<Rd::kLocal>();   // the following rounds are warp-local once this one is
-    if constexpr (S0 + LOGE < FCfg<LOGN, LOGE>::SL) FFwdRounds<LOGN, LOGE, S0 + LOGE>::run(v, sm, tw, tau, c60, c64, q2);
+    if constexpr (S0 + LOGE < FCfg<LOGN, LOGE>::SL) FFwdRounds<LOGN, LOGE, S0 + LOGE>::run(v, sm, tw, tau, f);
   }
 };
 
@@ -437,19 +435,18 @@ struct FFwdRounds {
 // return v holds the coefficients tau + l T.
 template <int LOGN, int LOGE, int S0>
 struct FInvRounds {
-  static __device__ __forceinline__ void run(u64 (&v)[1 << LOGE], u64* sm, const ulonglong2* tw, int tau, u32 c60,
-                                             u32 c64, u64 q2, u64 q4, const u64* sc) {
+  static __device__ __forceinline__ void run(u64 (&v)[1 << LOGE], u64* sm, const uint4* tw, int tau, const FoldC& f, u64 q2, const uint4* sc) {
     using Rd = FRound<LOGN, LOGE, S0>;
     Rd::load(v, sm, tau);
     if constexpr (S0 == 0)
-      Rd::inv_scaled(v, tw, tau, c60, c64, q2, q4, sc);
+      Rd::inv_scaled(v, tw, tau, f, q2, sc);
     else
-      Rd::inv(v, tw, tau, c60, c64, q2, q4);
+      Rd::inv(v, tw, tau, f);
     if constexpr (S0 > 0) {
       phase_sync<Rd::kLocal>();
       Rd::store(v, sm, tau);
       phase_sync<Rd::kLocal && FRound<LOGN, LOGE, S0 - LOGE>::kLocal>();
-      FInvRounds<LOGN, LOGE, S0 - LOGE>::run(v, sm, tw, tau, c60, c64, q2, q4, sc);
+      FInvRounds<LOGN, LOGE, S0 - LOGE>::run(v, sm, tw, tau, f, q2, sc);
     }
   }
 };
@@ -457,8 +454,7 @@ struct FInvRounds {
 // The last forward round's KL stages on one group of W = 2^KL consecutive slots
 // (group index g: positions g W .. g W + W - 1), then canonical values.
 template <int LOGN, int LOGE>
-__device__ __forceinline__ void fold_last_fwd(u64* u, const ulonglong2* __restrict__ tw, int g, u32 c60, u32 c64,
-                                              u64 q, u64 q2) {
+__device__ __forceinline__ void fold_last_fwd(u64* u, const uint4* __restrict__ tw, int g, const FoldC& f, u64 q, u64 off) {
   using C = FCfg<LOGN, LOGE>;
   constexpr int W = 1 << C::KL;
 #pragma unroll
@@ -466,20 +462,19 @@ __device__ __forceinline__ void fold_last_fwd(u64* u, const ulonglong2* __restri
     const int half = W >> (J + 1);
 #pragma unroll
     for (int i = 0; i < (1 << J); ++i) {
-      const ulonglong2 w = __ldg(tw + (1 << (C::SL + J)) + (g << J) + i);
+      const uint4 w = __ldg(tw + (1 << (C::SL + J)) + (g << J) + i);
 #pragma unroll
-      for (int r = 0; r < half; ++r) ct_fold(u[i * 2 * half + r], u[i * 2 * half + r + half], w, c60, c64, q2);
+      for (int r = 0; r < half; ++r) ct_split(u[i * 2 * half + r], u[i * 2 * half + r + half], w, f);
     }
   }
 #pragma unroll
-  for (int i = 0; i < W; ++i) u[i] = csub(fold60(u[i], c60), q);
+  for (int i = 0; i < W; ++i) u[i] = csub(fold_u(u[i] + off, f), q);
 }
 
 // The first inverse round's KL stages (inverse steps 0 .. KL - 1) on one group.
 template <int LOGN, int LOGE>
 __device__ __forceinline__ void fold_first_inv(u64 (&u)[1 << FCfg<LOGN, LOGE>::KL],
-                                               const ulonglong2* __restrict__ tw, int g, u32 c60, u32 c64, u64 q2,
-                                               u64 q4) {
+                                               const uint4* __restrict__ tw, int g, const FoldC& f) {
   using C = FCfg<LOGN, LOGE>;
   constexpr int W = 1 << C::KL;
 #pragma unroll
@@ -488,12 +483,12 @@ __device__ __forceinline__ void fold_first_inv(u64 (&u)[1 << FCfg<LOGN, LOGE>::K
     const bool odd = ((LOGN - 1 - (C::SL + J)) & 1) != 0;
 #pragma unroll
     for (int i = 0; i < (1 << J); ++i) {
-      const ulonglong2 w = __ldg(tw + (1 << (C::SL + J)) + (g << J) + i);
+      const uint4 w = __ldg(tw + (1 << (C::SL + J)) + (g << J) + i);
 #pragma unroll
       for (int r = 0; r < half; ++r) {
         u64& x = u[i * 2 * half + r];
-        gs_fold(x, u[i * 2 * half + r + half], w, c60, c64, odd ? q4 : q2);
-        if (odd) x = fold60(x, c60);
+        gs_split(x, u[i * 2 * half + r + half], w, f);
+        if (odd) x = fold_s(x, f);
       }
     }
   }
@@ -512,13 +507,12 @@ struct SparseInput<M, std::void_t<decltype(M::kSparse)>> : std::bool_constant<M:
 // stages only copy.  Round 0 (LOGE stages) is therefore skipped whole, and so
 // are the first j stages of round 1 where sup <= T / 2^j; round 1 then starts
 // from word x = p[x mod (N / 2^(LOGE + j))], read from the T prologue values in
-// shared memory (one gather per thread instead of E).  The values and their
-// bounds are those the skipped butterflies leave (ct_fold(a, 0) = (a, a + 2q)
-// only widens the bound).  Leaves round 1's words, folded, in shared memory.
+// shared memory (one gather per thread instead of E).  The values are those the
+// skipped butterflies leave (ct_split(a, 0) = (a, a)).  Leaves round 1's words, folded, in shared memory.
 template <int LOGN, int LOGE, class Mode>
 __device__ __forceinline__ void fold_sparse_head(const DevCtx& ctx, const typename Mode::Params& P,
                                                  const LimbConst& lc, int poly, int limb, int sup, u64 (&v)[1 << LOGE],
-                                                 u64* sm, const ulonglong2* tw, int tau, u32 c60, u32 c64, u64 q2) {
+                                                 u64* sm, const uint4* tw, int tau, const FoldC& f) {
   using C = FCfg<LOGN, LOGE>;
   using R1 = FRound<LOGN, LOGE, LOGE>;
   static_assert(R1::K == LOGE && R1::G == 1, "round 1 must be a full round");
@@ -531,13 +525,13 @@ __device__ __forceinline__ void fold_sparse_head(const DevCtx& ctx, const typena
   const u64* b = sm + ph(tau & (D1 - 1));
 #pragma unroll
   for (int l = 0; l < C::E; ++l) v[l] = b[ph(D1 * (l & m))];
-  R1::fwd_from(j, v, tw, tau, c60, c64, q2);
+  R1::fwd_from(j, v, tw, tau, f);
 #pragma unroll
-  for (int l = 0; l < C::E; ++l) v[l] = fold60(v[l], c60);
+  for (int l = 0; l < C::E; ++l) v[l] = fold_s(v[l], f);
   __syncthreads();   // every thread has read the prologue values
   R1::store(v, sm, tau);
   phase_sync<R1::kLocal>();
-  if constexpr (2 * LOGE < C::SL) FFwdRounds<LOGN, LOGE, 2 * LOGE>::run(v, sm, tw, tau, c60, c64, q2);
+  if constexpr (2 * LOGE < C::SL) FFwdRounds<LOGN, LOGE, 2 * LOGE>::run(v, sm, tw, tau, f);
 }
 
 template <int LOGN, int LOGE, class Mode>
@@ -546,16 +540,16 @@ __device__ __forceinline__ void ntt_fwd_run_fold(const DevCtx& ctx, const typena
   using C = FCfg<LOGN, LOGE>;
   const int tau = threadIdx.x;
   const LimbConst& lc = ctx.limb[limb];
-  const u64 q = lc.q, q2 = 2 * q;
-  const u32 c60 = (u32)lc.c60, c64 = (u32)lc.c64;
-  const ulonglong2* tw = ctx.tw_fwd_f + (size_t)limb * C::N;
+  const u64 q = lc.q;
+  const FoldC f(lc);
+  const uint4* tw = ctx.tw_fwd_f + (size_t)limb * C::N;
   u64 v[C::E];
   bool dense = true;
   if constexpr (SparseInput<Mode>::value && C::R >= 3) {
     const int sup = Mode::support(P);
     if (sup <= C::T) {
       dense = false;
-      fold_sparse_head<LOGN, LOGE, Mode>(ctx, P, lc, poly, limb, sup, v, sm, tw, tau, c60, c64, q2);
+      fold_sparse_head<LOGN, LOGE, Mode>(ctx, P, lc, poly, limb, sup, v, sm, tw, tau, f);
     }
   }
   if (dense) {
@@ -572,7 +566,7 @@ __device__ __forceinline__ void ntt_fwd_run_fold(const DevCtx& ctx, const typena
       for (int l = 0; l < C::E; ++l) v[l] = Mode::template load<C::N>(ctx, P, lc, poly, limb, tau + l * C::T);
     }
     // (round 0 stores each thread's words at the slots it read them from: no barrier needed here)
-    FFwdRounds<LOGN, LOGE, 0>::run(v, sm, tw, tau, c60, c64, q2);
+    FFwdRounds<LOGN, LOGE, 0>::run(v, sm, tw, tau, f);
   }
   if constexpr (C::FUSE) {
     // groups of GW consecutive slots per iteration: the last round's groups of
@@ -593,7 +587,7 @@ __device__ __forceinline__ void ntt_fwd_run_fold(const DevCtx& ctx, const typena
         u[2 * i + 1] = x.y;
       }
 #pragma unroll
-      for (int s = 0; s < GW / W; ++s) fold_last_fwd<LOGN, LOGE>(u + s * W, tw, k * (GW / W) + s, c60, c64, q, q2);
+      for (int s = 0; s < GW / W; ++s) fold_last_fwd<LOGN, LOGE>(u + s * W, tw, k * (GW / W) + s, f, q, 4 * q);
       if constexpr (Mode::kQuad) {
 #pragma unroll
         for (int i = 0; i < GW / 4; ++i) Mode::template store4<C::N>(ctx, P, lc, poly, limb, k * GW + 4 * i, u + 4 * i);
@@ -606,9 +600,9 @@ __device__ __forceinline__ void ntt_fwd_run_fold(const DevCtx& ctx, const typena
   } else {
     using Rd = FRound<LOGN, LOGE, C::SL>;
     Rd::load(v, sm, tau);
-    Rd::fwd(v, tw, tau, c60, c64, q2);
+    Rd::fwd(v, tw, tau, f);
 #pragma unroll
-    for (int l = 0; l < C::E; ++l) v[l] = csub(fold60(v[l], c60), q);
+    for (int l = 0; l < C::E; ++l) v[l] = csub(fold_u(v[l] + 8 * q, f), q);
     static_assert(Rd::kLocal, "the last round is warp-local");
     __syncwarp();
     Rd::store(v, sm, tau);
@@ -641,10 +635,10 @@ __device__ __forceinline__ void ntt_inv_run_fold(const DevCtx& ctx, const typena
   using C = FCfg<LOGN, LOGE>;
   const int tau = threadIdx.x;
   const LimbConst& lc = ctx.limb[limb];
-  const u64 q = lc.q, q2 = 2 * q, q4 = 4 * q;
-  const u32 c60 = (u32)lc.c60, c64 = (u32)lc.c64;
-  const ulonglong2* tw = ctx.tw_inv_f + (size_t)limb * C::N;
-  const u64* sc = Mode::kInvScale == InvScale::kNinv ? lc.sc_ninv : lc.sc_nqtil;
+  const u64 q = lc.q, q2 = 2 * q;
+  const FoldC f(lc);
+  const uint4* tw = ctx.tw_inv_f + (size_t)limb * C::N;
+  const uint4* sc = Mode::kInvScale == InvScale::kNinv ? lc.sc_ninv : lc.sc_nqtil;
   u64 v[C::E];
   if constexpr (C::FUSE) {
     constexpr int W = 1 << C::KL;
@@ -656,14 +650,14 @@ __device__ __forceinline__ void ntt_inv_run_fold(const DevCtx& ctx, const typena
       u64 u[W];
 #pragma unroll
       for (int i = 0; i < W; ++i) u[i] = Mode::template load<C::N>(ctx, P, lc, poly, limb, g * W + i);
-      fold_first_inv<LOGN, LOGE>(u, tw, g, c60, c64, q2, q4);
+      fold_first_inv<LOGN, LOGE>(u, tw, g, f);
       ulonglong2* b = reinterpret_cast<ulonglong2*>(sm + ph(g * W));
 #pragma unroll
       for (int i = 0; i < W / 2; ++i) b[i] = make_ulonglong2(u[2 * i], u[2 * i + 1]);
     }
     if constexpr (C::SL > 0) {
       phase_sync<FRound<LOGN, LOGE, C::SL - LOGE>::kLocal>();
-      FInvRounds<LOGN, LOGE, C::SL - LOGE>::run(v, sm, tw, tau, c60, c64, q2, q4, sc);
+      FInvRounds<LOGN, LOGE, C::SL - LOGE>::run(v, sm, tw, tau, f, q2, sc);
     } else {
       __syncthreads();
     }
@@ -678,12 +672,13 @@ __device__ __forceinline__ void ntt_inv_run_fold(const DevCtx& ctx, const typena
     }
     static_assert(FRound<LOGN, LOGE, C::SL>::kLocal, "the last round is warp-local");
     __syncwarp();
-    FInvRounds<LOGN, LOGE, C::SL>::run(v, sm, tw, tau, c60, c64, q2, q4, sc);
+    FInvRounds<LOGN, LOGE, C::SL>::run(v, sm, tw, tau, f, q2, sc);
   }
-  // v < 1.13 q, already scaled by the mode's kappa in the last stage
+  // v in (0.9 q, 4.1 q), already scaled by the mode's kappa in the last stage
   if constexpr (ClusterLimbs<Mode>::value) __syncthreads();   // the last round's reads are done
 #pragma unroll
-  for (int l = 0; l < C::E; ++l) Mode::template store<C::N>(ctx, P, lc, poly, limb, tau + l * C::T, csub(v[l], q));
+  for (int l = 0; l < C::E; ++l)
+    Mode::template store<C::N>(ctx, P, lc, poly, limb, tau + l * C::T, csub(fold_u(v[l], f), q));
 }
 
 // Launch shape of either engine.
