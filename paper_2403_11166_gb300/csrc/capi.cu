@@ -180,12 +180,12 @@ struct PencilCtx {
 
 struct PencilSecretKey {
   PencilCtx* ctx;
-  ulonglong2* sk = nullptr;
+  ulonglong2* sk = nullptr;   // [L][N] (value, Shoup companion), then [L][N] split twiddles (uint4)
 };
 
 struct PencilPublicKey {
   PencilCtx* ctx;
-  ulonglong2* key = nullptr;   // [2][L][N] (value, Shoup companion), then N bytes of scratch
+  ulonglong2* key = nullptr;   // [2][L][N] (value, Shoup companion), [2][L][N] split twiddles, N bytes of scratch
 };
 
 struct Geom {
@@ -211,7 +211,7 @@ struct PencilPlan {
   Accessor acc_v, acc_w, acc_y;  // ptr filled per call
   long long hw;                  // output spatial size (bias broadcast)
   int co_out;                    // output channel count seen by the bias
-  u64* d_tab = nullptr;          // [3][N]: v, w, y tables
+  ulonglong2* d_tab = nullptr;   // [3][N]: v, w, y tables (Packing)
   int4* d_org = nullptr;         // origins: v [ct_in], w [pt], y [ct_out]
   Packing pk_v, pk_w, pk_y;
   long long ws_encrypt, ws_forward, ws_backward, ws_decrypt, ws_encrypt_pk;
@@ -351,6 +351,7 @@ extern "C" int pencil_ctx_create(const PencilParams* params, int device, PencilC
     lc.ninvs = shoup(lc.ninv, q);
     lc.delta = delta_mod(qs, p.t_bits, q);
     lc.deltas = shoup(lc.delta, q);
+    lc.delta_sp = split_twiddle(lc.delta, q);
     u64 qt = 1;
     for (int i = 0; i < d.L; ++i)
       if (i != j) qt = mulmod(qt, qs[i] % q, q);
@@ -388,6 +389,7 @@ extern "C" int pencil_ctx_create(const PencilParams* params, int device, PencilC
     u64 qt = 1;
     for (int j = 0; j < d.L; ++j) qt *= qs[j];
     d.q_mod_t = qt & d.t_mask;
+    d.q_frac = d.q_mod_t << (64 - p.t_bits);
   }
   d.mac_nt = 4;
   d.mac_staging = 1;   // measured: bulk copies by a producer warp, 4 columns per thread
@@ -536,7 +538,7 @@ extern "C" int pencil_keygen(PencilCtx* ctx, uint64_t seed, PencilSecretKey** ou
   PencilSecretKey* sk = new (std::nothrow) PencilSecretKey();
   if (!sk) return PENCIL_E_CUDA;
   sk->ctx = ctx;
-  if (cudaMalloc(&sk->sk, (size_t)ctx->dev.L * ctx->n * sizeof(ulonglong2)) != cudaSuccess) {
+  if (cudaMalloc(&sk->sk, 2ull * ctx->dev.L * ctx->n * sizeof(ulonglong2)) != cudaSuccess) {
     delete sk;
     return PENCIL_E_CUDA;
   }
@@ -567,7 +569,7 @@ extern "C" int pencil_pk_keygen(PencilCtx* ctx, const PencilSecretKey* sk, uint6
   PencilPublicKey* pk = new (std::nothrow) PencilPublicKey();
   if (!pk) return PENCIL_E_CUDA;
   pk->ctx = ctx;
-  const size_t key_bytes = 2ull * ctx->dev.L * ctx->n * sizeof(ulonglong2);
+  const size_t key_bytes = 4ull * ctx->dev.L * ctx->n * sizeof(ulonglong2);
   if (cudaMalloc(&pk->key, key_bytes + ctx->n) != cudaSuccess) {
     delete pk;
     return PENCIL_E_CUDA;
@@ -825,7 +827,7 @@ extern "C" int pencil_plan_linear(PencilCtx* ctx, const PencilLayerDesc* layer, 
   const int h = p.th + p.kth - 1, w = p.tw + p.ktw - 1;
   const long long O = (long long)(p.cib - 1) * h * w + (long long)(p.kth - 1) * w + p.ktw - 1;
   const long long blk = (long long)p.cob * p.cib * h * w;
-  std::vector<u64> tab(3 * (size_t)n, PENCIL_TAB_NONE);
+  std::vector<u64> tab(3 * (size_t)n, PENCIL_TAB_NONE);   // fields below N <= 2^14
   for (int b = 0; b < p.bb; ++b)
     for (int ch = 0; ch < p.cib; ++ch)
       for (int i = 0; i < h; ++i)
@@ -860,9 +862,19 @@ extern "C" int pencil_plan_linear(PencilCtx* ctx, const PencilLayerDesc* layer, 
     for (int nn = 0; nn < c.NC; ++nn) org[o++] = make_int4(mb * p.bb, nn * p.cob, mh * p.th, mw * p.tw);
   }
   DeviceGuard guard(ctx->device);
-  if (cudaMalloc(&P->d_tab, tab.size() * sizeof(u64)) != cudaSuccess ||
+  // beside the coordinates, the byte offset they give in the operand's tensor
+  std::vector<ulonglong2> tab2(tab.size());
+  for (size_t i = 0; i < tab.size(); ++i) {
+    const Accessor& ac = i < (size_t)n ? P->acc_v : i < 2 * (size_t)n ? P->acc_w : P->acc_y;
+    const u64 x = tab[i];
+    const i64 off = x == PENCIL_TAB_NONE ? 0
+                                         : 8 * ((i64)(x & 0xffff) * ac.s0 + (i64)((x >> 16) & 0xffff) * ac.s1 +
+                                                (i64)((x >> 32) & 0xffff) * ac.s2 + (i64)(x >> 48) * ac.s3);
+    tab2[i] = make_ulonglong2(x, (u64)off);
+  }
+  if (cudaMalloc(&P->d_tab, tab2.size() * sizeof(ulonglong2)) != cudaSuccess ||
       cudaMalloc(&P->d_org, org.size() * sizeof(int4)) != cudaSuccess ||
-      cudaMemcpy(P->d_tab, tab.data(), tab.size() * sizeof(u64), cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemcpy(P->d_tab, tab2.data(), tab2.size() * sizeof(ulonglong2), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(P->d_org, org.data(), org.size() * sizeof(int4), cudaMemcpyHostToDevice) != cudaSuccess) {
     pencil_plan_destroy(P);
     return PENCIL_E_CUDA;

@@ -19,6 +19,7 @@ struct LimbConst {
   u64 r64, r64s;     // 2^64 mod q and its Shoup companion
   u64 ninv, ninvs;   // N^{-1} mod q                              (INTT scaling)
   u64 delta, deltas; // floor(q_total / t) mod q                  (BFV Delta)
+  uint4 delta_sp;    // its split twiddle (mul_split)
   u64 qtil, qtils;   // (q_total / q_j)^{-1} mod q_j              (CRT)
   u64 th_hi, th_lo;  // floor(2^(128 + t_bits) / q_j), 128 bits   (t / q_j in 0.128 fixed point)
   u64 c60, c64;      // 2^60 mod q and 2^64 mod q                 (split multiply-accumulate folds)
@@ -55,6 +56,7 @@ struct DevCtx {
   int sms;                   // multiprocessors of the device
   int mac_mma;               // 1: every q_j = 2^b - c with c < 2^(b-32), 2^64 mod q_j < 2^32 (digit products, digits.cuh)
   u64 q_mod_t;               // (q_total mod t): messages are scaled as round(q_total m / t)
+  u64 q_frac;                // q_mod_t 2^(64 - t_bits): (q_total mod t) / t as a 64-bit fraction
   int flood_bits;            // 0, or the flooding noise of returned ciphertexts: uniform in [-2^b, 2^b)
 };
 
@@ -68,19 +70,21 @@ struct Accessor {
   int pr, ps, hr, wr;
 };
 
-// Packing of one operand position class (inputs, kernels or outputs):
-// tab[e] = local (a, b, r, s) of coefficient e packed as 4 x 16 bits, or
-// all-ones when coefficient e carries nothing; org[idx] = the block origin of
-// polynomial idx; bound = the geometry extent of (a, b, r, s); support = 1 +
-// the highest e with an entry (coefficients from support on are always zero).
+// Packing of one operand position class (inputs, kernels or outputs) with the strides
+// of that operand's tensor: tab[e] = (x) local (a, b, r, s) of coefficient e packed as
+// 4 x 16 bits, each below 2^14 (blocks hold at most N <= 2^14 elements), or 0x7fff in
+// every field when coefficient e carries nothing, and (y) its offset in bytes from the
+// block's first element; org[idx] = the block origin of polynomial idx; bound = the
+// geometry extent of (a, b, r, s); support = 1 + the highest e with an entry
+// (coefficients from support on are always zero).
 struct Packing {
-  const u64* tab;
+  const ulonglong2* tab;
   const int4* org;
   int4 bound;
   int support;
 };
 
-#define PENCIL_TAB_NONE 0xFFFFFFFFFFFFFFFFull
+#define PENCIL_TAB_NONE 0x7FFF7FFF7FFF7FFFull
 
 // ------------------------------------------------------------------ 64-bit modular arithmetic
 __device__ __forceinline__ u64 mulhi64(u64 a, u64 b) { return __umul64hi(a, b); }
@@ -163,15 +167,15 @@ __host__ __device__ __forceinline__ void gs_bf4(u64& x, u64& y, u64 w, u64 ws, u
 
 __device__ __forceinline__ u64 add_mod(u64 a, u64 b, u64 q) { return csub(a + b, q); }
 
-// round(q_total m / t) mod q_j for m in [0, t): Delta m + floor(((q_total mod t) m + t / 2) / t),
-// the BFV message scaling (t = 2^t_bits, so the division is a shift of the
-// 128-bit product; the quotient is below t < q_j).
+// round((q_total mod t) m / t) for m in [0, t): the part of the BFV message scaling
+// round(q_total m / t) = Delta m + this that does not depend on the limb (below t < q_j).
+// q_frac m / 2^64 is exact, so rounding adds the top fraction bit.
+__device__ __forceinline__ u64 scale_extra(u64 m, const DevCtx& c) {
+  return __umul64hi(c.q_frac, m) + ((c.q_frac * m) >> 63);
+}
+// round(q_total m / t) mod q_j, canonical.
 __device__ __forceinline__ u64 scale_msg(u64 m, const LimbConst& lc, const DevCtx& c) {
-  const u64 lo = c.q_mod_t * m, hi = __umul64hi(c.q_mod_t, m);
-  const u64 slo = lo + (1ull << (c.t_bits - 1));
-  const u64 shi = hi + (slo < lo ? 1ull : 0ull);
-  const u64 extra = (shi << (64 - c.t_bits)) | (slo >> c.t_bits);
-  return add_mod(mul_shoup(m, lc.delta, lc.deltas, lc.q), extra, lc.q);
+  return add_mod(mul_shoup(m, lc.delta, lc.deltas, lc.q), scale_extra(m, c), lc.q);
 }
 __device__ __forceinline__ u64 sub_mod(u64 a, u64 b, u64 q) { return a >= b ? a - b : a + q - b; }
 
@@ -353,33 +357,59 @@ __device__ __forceinline__ u64 philox_word(const Philox4& w, int i) {
   return i == 0 ? w.v[0] : i == 1 ? w.v[1] : i == 2 ? w.v[2] : w.v[3];
 }
 
-// Uniform residue mod q_j of coefficient `coef` from its 64-bit Philox word w
-// (the encryption mask a, the public key's a): w is accepted when w <= a_max
-// (below the largest multiple of q_j under 2^64) and reduced; a rejected word is
-// replaced by word 0 of the block at counter (coef, ct, limb, r), r = 1, 2, ...
-// (probability below 2^-32 per word for the primes used; the loop stops after 64
-// replacements, which for primes above 2^40 never happens in practice).
-__device__ __forceinline__ u64 uniform_mod_q(u64 w, int coef, int ct, int limb, u64 seed, u64 dom,
-                                             const LimbConst& lc) {
+// 64-bit word of coefficient `coef` whose residue mod q_j is uniform (the encryption
+// mask a, the public key's a), from its Philox word w: w is accepted when w <= a_max
+// (below the largest multiple of q_j under 2^64); a rejected word is replaced by word 0
+// of the block at counter (coef, ct, limb, r), r = 1, 2, ... (probability below 2^-32
+// per word for the primes used; the loop stops after 64 replacements, which for primes
+// above 2^40 never happens in practice).
+__device__ __forceinline__ u64 uniform_word(u64 w, int coef, int ct, int limb, u64 seed, u64 dom,
+                                            const LimbConst& lc) {
   for (u64 r = 1; w > lc.a_max && r <= 64; ++r) w = philox4x64((u64)coef, (u64)ct, (u64)limb, r, seed, dom).v[0];
-  return reduce64(w, lc);
+  return w;
 }
 
 // ------------------------------------------------------------------ packing gathers
-__device__ __forceinline__ u64 gather(const Packing& pk, const Accessor& ac, int idx, int e) {
-  u64 ent = __ldg(pk.tab + e);
-  if (ent == PENCIL_TAB_NONE) return 0;
-  int4 o = __ldg(pk.org + idx);
-  int a = o.x + (int)(ent & 0xffff);
-  int b = o.y + (int)((ent >> 16) & 0xffff);
-  int r = o.z + (int)((ent >> 32) & 0xffff);
-  int s = o.w + (int)(ent >> 48);
-  if (a >= pk.bound.x || b >= pk.bound.y || r >= pk.bound.z || s >= pk.bound.w) return 0;
-  r -= ac.pr;
-  s -= ac.ps;
-  if ((unsigned)r >= (unsigned)ac.hr || (unsigned)s >= (unsigned)ac.wr) return 0;
-  return __ldg(ac.ptr + ac.base + a * ac.s0 + b * ac.s1 + r * ac.s2 + s * ac.s3);
-}
+// One polynomial's view of its operand: address of its block's first element (or, with
+// a null tensor, that element's index times 8) and the extent of its valid local
+// coordinates, packed so that one 64-bit subtraction tests all four upper bounds and one
+// 32-bit addition the two lower ones: with 16-bit fields c <= 0x7fff, bit 15 of
+// (0x8000 + max) - c is set iff c <= max and bit 15 of c + (0x8000 - min) iff c >= min.
+// Set up once per polynomial; an element then costs a 16-byte table load, six integer
+// operations and a 64-bit addition (the origin, four compares, two range checks and four
+// 64-bit strided products it replaces were about half of the fused transforms'
+// prologues: ModeMoPrep at N = 8192 260 thread instructions per coefficient, 175 of them
+// the transform).
+struct Window {
+  const char* base;
+  u32 tl, th, lh;
+  __device__ __forceinline__ Window(const Packing& pk, const Accessor& ac, int idx, const void* ptr) {
+    const int4 o = __ldg(pk.org + idx);
+    base = reinterpret_cast<const char*>(ptr) +
+           8 * (ac.base + o.x * ac.s0 + o.y * ac.s1 + (i64)(o.z - ac.pr) * ac.s2 + (i64)(o.w - ac.ps) * ac.s3);
+    tl = top(pk.bound.x - o.x) | (top(pk.bound.y - o.y) << 16);
+    th = top(min(pk.bound.z, ac.hr + ac.pr) - o.z) | (top(min(pk.bound.w, ac.wr + ac.ps) - o.w) << 16);
+    lh = low(ac.pr - o.z) | (low(ac.ps - o.w) << 16);
+  }
+  __device__ __forceinline__ Window(const char* b, u32 l, u32 h, u32 m) : base(b), tl(l), th(h), lh(m) {}
+  static __device__ __forceinline__ u32 top(int extent) { return 0x7FFFu + (u32)min(max(extent, 0), 0x4000); }
+  static __device__ __forceinline__ u32 low(int first) { return 0x8000u - (u32)min(max(first, 0), 0x7FFF); }
+  __device__ __forceinline__ bool has(const ulonglong2& ent) const {
+    const u32 cl = (u32)ent.x, ch = (u32)(ent.x >> 32);
+    return ((tl - cl) & (th - ch) & (ch + lh) & 0x80008000u) == 0x80008000u;
+  }
+  __device__ __forceinline__ const char* at(const ulonglong2& ent) const { return base + (i64)ent.y; }
+  // element of coefficient e (0 where the coefficient carries nothing)
+  __device__ __forceinline__ u64 get(const Packing& pk, int e) const {
+    const ulonglong2 ent = __ldg(pk.tab + e);
+    return has(ent) ? __ldg(reinterpret_cast<const u64*>(at(ent))) : 0ull;
+  }
+  // element index of coefficient e in the operand's tensor (null ptr), or -1
+  __device__ __forceinline__ i64 index(const Packing& pk, int e) const {
+    const ulonglong2 ent = __ldg(pk.tab + e);
+    return has(ent) ? (i64)at(ent) >> 3 : -1;
+  }
+};
 
 // Decryption's CRT step: with y_j = x_j (q/q_j)^{-1} mod q_j,
 //   t x / q = sum_j y_j t / q_j - v t  (v integer),
@@ -409,17 +439,4 @@ __device__ __forceinline__ u64 crt_round(const CrtSum& s, u64 t_mask, int check,
   const u64 r_lo = s.lo + (1ull << 63);
   const u64 r_hi = s.hi + (r_lo < s.lo ? 1ull : 0ull);
   return r_hi & t_mask;
-}
-
-// Output flat index of coefficient e of output polynomial idx, or -1.
-__device__ __forceinline__ i64 out_index(const Packing& pk, const Accessor& ac, int idx, int e) {
-  u64 ent = __ldg(pk.tab + e);
-  if (ent == PENCIL_TAB_NONE) return -1;
-  int4 o = __ldg(pk.org + idx);
-  int a = o.x + (int)(ent & 0xffff);
-  int b = o.y + (int)((ent >> 16) & 0xffff);
-  int r = o.z + (int)((ent >> 32) & 0xffff);
-  int s = o.w + (int)(ent >> 48);
-  if (a >= pk.bound.x || b >= pk.bound.y || r >= pk.bound.z || s >= pk.bound.w) return -1;
-  return ac.base + a * ac.s0 + b * ac.s1 + r * ac.s2 + s * ac.s3;
 }

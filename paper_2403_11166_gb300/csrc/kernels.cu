@@ -847,9 +847,10 @@ __device__ __forceinline__ void mask_poly_block(const DevCtx& ctx, const Packing
                                                 int ct, int blk, u64* out_ct) {
   i64 flat[4];
   bool any_pad = false;
+  const Window win(pk, ac, ct, nullptr);
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    flat[i] = out_index(pk, ac, ct, 4 * blk + i);
+    flat[i] = win.index(pk, 4 * blk + i);
     any_pad |= flat[i] < 0;
   }
   Philox4 pad = {{0, 0, 0, 0}};
@@ -929,7 +930,7 @@ __device__ __forceinline__ void decrypt_combine_one(const DevCtx& ctx, const Pac
                                                     const u64* yres, int ct, int e, int check, u64* y1,
                                                     const u64* c0c = nullptr, long long out_elems = 0) {
   const int n = ctx.n;
-  const i64 flat = out_index(pk, ac, ct, e);
+  const i64 flat = Window(pk, ac, ct, nullptr).index(pk, e);
   if (flat < 0) return;
   CrtSum sum{0, 0};
   for (int j = 0; j < ctx.L; ++j) {

@@ -168,6 +168,7 @@ __device__ __forceinline__ void ntt_fwd_run(const DevCtx& ctx, const typename Mo
   using C = NttCfg<LOGN, LOGE>;
   const int tau = threadIdx.x;
   const LimbConst& lc = ctx.limb[limb];
+  const typename Mode::Pre pre(ctx, P, poly);
   const u64 q = lc.q, q2 = 2 * q;
   const ulonglong2* tw = ctx.tw_fwd + (size_t)limb * C::N;
   u64 v[C::E];
@@ -178,14 +179,14 @@ __device__ __forceinline__ void ntt_fwd_run(const DevCtx& ctx, const typename Mo
 #pragma unroll(Mode::kLoadUnroll)
     for (int l = 0; l < C::E; ++l) {
       const int e = tau + l * C::T;
-      sm[sidx<LOGN>(e)] = Mode::template load<C::N>(ctx, P, lc, poly, limb, e);
+      sm[sidx<LOGN>(e)] = Mode::template load<C::N, false>(ctx, P, pre, lc, poly, limb, e);
     }
 #pragma unroll
     for (int l = 0; l < C::E; ++l) v[l] = sm[sidx<LOGN>(tau + l * C::T)];
     __syncthreads();
   } else {
 #pragma unroll
-    for (int l = 0; l < C::E; ++l) v[l] = Mode::template load<C::N>(ctx, P, lc, poly, limb, tau + l * C::T);
+    for (int l = 0; l < C::E; ++l) v[l] = Mode::template load<C::N, false>(ctx, P, pre, lc, poly, limb, tau + l * C::T);
   }
   FwdRounds<LOGN, C::LOGE, 0>::run(v, sm, tw, tau, q, q2);
   if constexpr (Mode::kQuad) {
@@ -195,7 +196,7 @@ __device__ __forceinline__ void ntt_fwd_run(const DevCtx& ctx, const typename Mo
       u64 x[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) x[i] = canon4(sm[sidx<LOGN>(e + i)], q, q2);
-      Mode::template store4<C::N>(ctx, P, lc, poly, limb, e, x);
+      Mode::template store4<C::N, false>(ctx, P, lc, poly, limb, e, x);
     }
   } else {
 #pragma unroll(Mode::kEpilogueUnroll)
@@ -203,7 +204,7 @@ __device__ __forceinline__ void ntt_fwd_run(const DevCtx& ctx, const typename Mo
       const int e = 2 * (tau + l * C::T);
       const u64 x0 = canon4(sm[sidx<LOGN>(e)], q, q2);
       const u64 x1 = canon4(sm[sidx<LOGN>(e + 1)], q, q2);
-      Mode::template store2<C::N>(ctx, P, lc, poly, limb, e, x0, x1);
+      Mode::template store2<C::N, false>(ctx, P, lc, poly, limb, e, x0, x1);
     }
   }
 }
@@ -216,13 +217,14 @@ __device__ __forceinline__ void ntt_inv_run(const DevCtx& ctx, const typename Mo
   using C = NttCfg<LOGN, LOGE>;
   const int tau = threadIdx.x;
   const LimbConst& lc = ctx.limb[limb];
+  const typename Mode::Pre pre(ctx, P, poly);
   const u64 q = lc.q, q2 = 2 * q;
   const ulonglong2* tw = ctx.tw_inv + (size_t)limb * C::N;
   u64 v[C::E];
 #pragma unroll(Mode::kLoadUnroll)
   for (int l = 0; l < C::E; ++l) {
     const int e = tau + l * C::T;
-    sm[sidx<LOGN>(e)] = Mode::template load<C::N>(ctx, P, lc, poly, limb, e);
+    sm[sidx<LOGN>(e)] = Mode::template load<C::N, false>(ctx, P, pre, lc, poly, limb, e);
   }
   __syncthreads();
   InvRounds<LOGN, C::LOGE, C::LAST_S0>::run(v, sm, tw, tau, q, q2);
@@ -511,12 +513,13 @@ struct SparseInput<M, std::void_t<decltype(M::kSparse)>> : std::bool_constant<M:
 // skipped butterflies leave (ct_split(a, 0) = (a, a)).  Leaves round 1's words, folded, in shared memory.
 template <int LOGN, int LOGE, class Mode>
 __device__ __forceinline__ void fold_sparse_head(const DevCtx& ctx, const typename Mode::Params& P,
-                                                 const LimbConst& lc, int poly, int limb, int sup, u64 (&v)[1 << LOGE],
+                                                 const typename Mode::Pre& pre, const LimbConst& lc, int poly, int limb, int sup,
+                                                 u64 (&v)[1 << LOGE],
                                                  u64* sm, const uint4* tw, int tau, const FoldC& f) {
   using C = FCfg<LOGN, LOGE>;
   using R1 = FRound<LOGN, LOGE, LOGE>;
   static_assert(R1::K == LOGE && R1::G == 1, "round 1 must be a full round");
-  sm[ph(tau)] = tau < sup ? Mode::template load<C::N>(ctx, P, lc, poly, limb, tau) : 0ull;
+  sm[ph(tau)] = tau < sup ? Mode::template load<C::N, true>(ctx, P, pre, lc, poly, limb, tau) : 0ull;
   int j = 0;
   while (j < LOGE && sup <= (C::T >> (j + 1))) ++j;
   __syncthreads();
@@ -540,6 +543,7 @@ __device__ __forceinline__ void ntt_fwd_run_fold(const DevCtx& ctx, const typena
   using C = FCfg<LOGN, LOGE>;
   const int tau = threadIdx.x;
   const LimbConst& lc = ctx.limb[limb];
+  const typename Mode::Pre pre(ctx, P, poly);
   const u64 q = lc.q;
   const FoldC f(lc);
   const uint4* tw = ctx.tw_fwd_f + (size_t)limb * C::N;
@@ -549,7 +553,7 @@ __device__ __forceinline__ void ntt_fwd_run_fold(const DevCtx& ctx, const typena
     const int sup = Mode::support(P);
     if (sup <= C::T) {
       dense = false;
-      fold_sparse_head<LOGN, LOGE, Mode>(ctx, P, lc, poly, limb, sup, v, sm, tw, tau, f);
+      fold_sparse_head<LOGN, LOGE, Mode>(ctx, P, pre, lc, poly, limb, sup, v, sm, tw, tau, f);
     }
   }
   if (dense) {
@@ -557,13 +561,13 @@ __device__ __forceinline__ void ntt_fwd_run_fold(const DevCtx& ctx, const typena
 #pragma unroll(Mode::kLoadUnroll)
       for (int l = 0; l < C::E; ++l) {
         const int e = tau + l * C::T;
-        sm[ph(e)] = Mode::template load<C::N>(ctx, P, lc, poly, limb, e);
+        sm[ph(e)] = Mode::template load<C::N, true>(ctx, P, pre, lc, poly, limb, e);
       }
 #pragma unroll
       for (int l = 0; l < C::E; ++l) v[l] = sm[ph(tau + l * C::T)];
     } else {
 #pragma unroll
-      for (int l = 0; l < C::E; ++l) v[l] = Mode::template load<C::N>(ctx, P, lc, poly, limb, tau + l * C::T);
+      for (int l = 0; l < C::E; ++l) v[l] = Mode::template load<C::N, true>(ctx, P, pre, lc, poly, limb, tau + l * C::T);
     }
     // (round 0 stores each thread's words at the slots it read them from: no barrier needed here)
     FFwdRounds<LOGN, LOGE, 0>::run(v, sm, tw, tau, f);
@@ -590,11 +594,11 @@ __device__ __forceinline__ void ntt_fwd_run_fold(const DevCtx& ctx, const typena
       for (int s = 0; s < GW / W; ++s) fold_last_fwd<LOGN, LOGE>(u + s * W, tw, k * (GW / W) + s, f, q, 4 * q);
       if constexpr (Mode::kQuad) {
 #pragma unroll
-        for (int i = 0; i < GW / 4; ++i) Mode::template store4<C::N>(ctx, P, lc, poly, limb, k * GW + 4 * i, u + 4 * i);
+        for (int i = 0; i < GW / 4; ++i) Mode::template store4<C::N, true>(ctx, P, lc, poly, limb, k * GW + 4 * i, u + 4 * i);
       } else {
 #pragma unroll
         for (int i = 0; i < GW / 2; ++i)
-          Mode::template store2<C::N>(ctx, P, lc, poly, limb, k * GW + 2 * i, u[2 * i], u[2 * i + 1]);
+          Mode::template store2<C::N, true>(ctx, P, lc, poly, limb, k * GW + 2 * i, u[2 * i], u[2 * i + 1]);
       }
     }
   } else {
@@ -616,14 +620,14 @@ __device__ __forceinline__ void ntt_fwd_run_fold(const DevCtx& ctx, const typena
         const ulonglong2* b = reinterpret_cast<const ulonglong2*>(sm + ph(e));
         const ulonglong2 x01 = b[0], x23 = b[1];
         u64 x[4] = {x01.x, x01.y, x23.x, x23.y};
-        Mode::template store4<C::N>(ctx, P, lc, poly, limb, e, x);
+        Mode::template store4<C::N, true>(ctx, P, lc, poly, limb, e, x);
       }
     } else {
 #pragma unroll(Mode::kEpilogueUnroll)
       for (int l = 0; l < C::E / 2; ++l) {
         const int e = wbase + 2 * (lane + 32 * l);
         const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(sm + ph(e));
-        Mode::template store2<C::N>(ctx, P, lc, poly, limb, e, x.x, x.y);
+        Mode::template store2<C::N, true>(ctx, P, lc, poly, limb, e, x.x, x.y);
       }
     }
   }
@@ -635,6 +639,7 @@ __device__ __forceinline__ void ntt_inv_run_fold(const DevCtx& ctx, const typena
   using C = FCfg<LOGN, LOGE>;
   const int tau = threadIdx.x;
   const LimbConst& lc = ctx.limb[limb];
+  const typename Mode::Pre pre(ctx, P, poly);
   const u64 q = lc.q, q2 = 2 * q;
   const FoldC f(lc);
   const uint4* tw = ctx.tw_inv_f + (size_t)limb * C::N;
@@ -649,7 +654,7 @@ __device__ __forceinline__ void ntt_inv_run_fold(const DevCtx& ctx, const typena
       const int g = gbase + 32 * j;
       u64 u[W];
 #pragma unroll
-      for (int i = 0; i < W; ++i) u[i] = Mode::template load<C::N>(ctx, P, lc, poly, limb, g * W + i);
+      for (int i = 0; i < W; ++i) u[i] = Mode::template load<C::N, true>(ctx, P, pre, lc, poly, limb, g * W + i);
       fold_first_inv<LOGN, LOGE>(u, tw, g, f);
       ulonglong2* b = reinterpret_cast<ulonglong2*>(sm + ph(g * W));
 #pragma unroll
@@ -668,7 +673,7 @@ __device__ __forceinline__ void ntt_inv_run_fold(const DevCtx& ctx, const typena
 #pragma unroll(Mode::kLoadUnroll)
     for (int l = 0; l < C::E; ++l) {
       const int e = wbase + 32 * l;
-      sm[ph(e)] = Mode::template load<C::N>(ctx, P, lc, poly, limb, e);
+      sm[ph(e)] = Mode::template load<C::N, true>(ctx, P, pre, lc, poly, limb, e);
     }
     static_assert(FRound<LOGN, LOGE, C::SL>::kLocal, "the last round is warp-local");
     __syncwarp();
@@ -777,6 +782,20 @@ __device__ __forceinline__ size_t ct_off(int poly, int comp, int limb, int L, in
   return (((size_t)poly * 2 + comp) * L + limb) * n;
 }
 
+// What a mode keeps per polynomial for its prologue (Mode::Pre).
+struct NoPre {
+  template <class P>
+  __device__ __forceinline__ NoPre(const DevCtx&, const P&, int) {}
+};
+struct WindowPre {
+  Window win;
+  template <class P>
+  __device__ __forceinline__ WindowPre(const DevCtx&, const P& p, int poly) : win(p.pk, p.ac, poly, p.ac.ptr) {}
+};
+
+// The split engine (SPLIT) takes prologue values as signed lazy residues in about
+// [-1/2, 1] (units of 2^b), the Shoup engine canonical ones.
+
 // In-place transform of [count][L][N] polynomials.
 struct ModeRaw {
   static constexpr InvScale kInvScale = InvScale::kNinv;
@@ -789,9 +808,10 @@ struct ModeRaw {
     u64* polys;
     int ahead = 0;   // CTAs ahead whose input each CTA asks L2 to fetch (0: none)
   };
+  using Pre = NoPre;
   static __device__ __forceinline__ void rebase(Params&, u64) {}
-  template <int N>
-  static __device__ __forceinline__ u64 load(const DevCtx& c, const Params& P, const LimbConst&, int poly, int limb,
+  template <int N, bool SPLIT>
+  static __device__ __forceinline__ u64 load(const DevCtx& c, const Params& P, const Pre& pre, const LimbConst&, int poly, int limb,
                                              int e) {
     return P.polys[limb_off(poly, limb, c.L, N) + e];
   }
@@ -801,7 +821,7 @@ struct ModeRaw {
                  "r"((u32)(N * sizeof(u64)))
                  : "memory");
   }
-  template <int N>
+  template <int N, bool SPLIT>
   static __device__ __forceinline__ void store2(const DevCtx& c, const Params& P, const LimbConst&, int poly,
                                                 int limb, int e, u64 x0, u64 x1) {
     *reinterpret_cast<ulonglong2*>(P.polys + limb_off(poly, limb, c.L, N) + e) = make_ulonglong2(x0, x1);
@@ -825,30 +845,43 @@ struct ModeEncrypt {
     Packing pk;
     Accessor ac;
     const int8_t* err;        // [count][N]
-    const ulonglong2* sk;     // [L][N] (s_hat, companion)
+    const ulonglong2* sk;     // [L][N] (s_hat, companion), [L][N] split s_hat
     u64* ct;                  // [count][2][L][N]
     u64 seed;
   };
   // seed of replay `step` (batched graphs): seed + step * 2^32
+  using Pre = WindowPre;
   static __device__ __forceinline__ void rebase(Params& P, u64 step) { P.seed += step << 32; }
-  template <int N>
-  static __device__ __forceinline__ u64 load(const DevCtx& c, const Params& P, const LimbConst& lc, int poly, int,
+  template <int N, bool SPLIT>
+  static __device__ __forceinline__ u64 load(const DevCtx& c, const Params& P, const Pre& pre, const LimbConst& lc, int poly, int,
                                              int e) {
-    const u64 m = gather(P.pk, P.ac, poly, e) & c.t_mask;
-    const u64 r = scale_msg(m, lc, c);
+    const u64 m = pre.win.get(P.pk, e) & c.t_mask;
     const int ee = P.err[(size_t)poly * N + e];
+    if constexpr (SPLIT) {
+      const FoldC f(lc);
+      return fold_s(mul_split(scale_extra(m, c) + (i64)ee, m, lc.delta_sp, f), f);
+    }
+    const u64 r = scale_msg(m, lc, c);
     return ee >= 0 ? add_mod(r, (u64)ee, lc.q) : sub_mod(r, (u64)(-ee), lc.q);
   }
-  template <int N>
+  template <int N, bool SPLIT>
   static __device__ __forceinline__ void store4(const DevCtx& c, const Params& P, const LimbConst& lc, int poly,
                                                 int limb, int e, const u64* x) {
     const Philox4 w = philox4x64((u64)(e >> 2), (u64)poly, (u64)limb, 0ull, P.seed, PENCIL_DOM_A);
     u64 a[4], c0[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      a[i] = uniform_mod_q(w.v[i], e + i, poly, limb, P.seed, PENCIL_DOM_A, lc);
-      const ulonglong2 s = __ldg(P.sk + (size_t)limb * N + e + i);
-      c0[i] = sub_mod(x[i], mul_shoup(a[i], s.x, s.y, lc.q), lc.q);
+      const u64 word = uniform_word(w.v[i], e + i, poly, limb, P.seed, PENCIL_DOM_A, lc);
+      if constexpr (SPLIT) {
+        const FoldC f(lc);
+        a[i] = csub(fold_u(word, f), lc.q);
+        const uint4 s = __ldg(reinterpret_cast<const uint4*>(P.sk) + (size_t)(c.L + limb) * N + e + i);
+        c0[i] = csub(fold_u(x[i] + 2 * lc.q - mul_split(0, a[i], s, f), f), lc.q);
+      } else {
+        a[i] = reduce64(word, lc);
+        const ulonglong2 s = __ldg(P.sk + (size_t)limb * N + e + i);
+        c0[i] = sub_mod(x[i], mul_shoup(a[i], s.x, s.y, lc.q), lc.q);
+      }
     }
     ulonglong2* d0 = reinterpret_cast<ulonglong2*>(P.ct + ct_off(poly, 0, limb, c.L, N) + e);
     ulonglong2* d1 = reinterpret_cast<ulonglong2*>(P.ct + ct_off(poly, 1, limb, c.L, N) + e);
@@ -873,15 +906,17 @@ struct ModeEncode {
     u64* pt;   // [count][L][N]
   };
   static __device__ __forceinline__ int support(const Params& P) { return P.pk.support; }
+  using Pre = WindowPre;
   static __device__ __forceinline__ void rebase(Params&, u64) {}
-  template <int N>
-  static __device__ __forceinline__ u64 load(const DevCtx& c, const Params& P, const LimbConst& lc, int poly, int,
+  template <int N, bool SPLIT>
+  static __device__ __forceinline__ u64 load(const DevCtx& c, const Params& P, const Pre& pre, const LimbConst& lc, int poly, int,
                                              int e) {
-    const u64 v = gather(P.pk, P.ac, poly, e) & c.t_mask;
+    const u64 v = pre.win.get(P.pk, e) & c.t_mask;
     const u64 half = (c.t_mask >> 1) + 1;
+    if constexpr (SPLIT) return v >= half ? v - (c.t_mask + 1) : v;
     return v >= half ? lc.q - ((c.t_mask + 1) - v) : v;
   }
-  template <int N>
+  template <int N, bool SPLIT>
   static __device__ __forceinline__ void store2(const DevCtx& c, const Params& P, const LimbConst&, int poly,
                                                 int limb, int e, u64 x0, u64 x1) {
     *reinterpret_cast<ulonglong2*>(P.pt + limb_off(poly, limb, c.L, N) + e) = make_ulonglong2(x0, x1);
@@ -906,21 +941,44 @@ struct ModeMoPrep {
     u64* out_mask;      // [count - n_in][L][N]
     u64 seed;           // mask seed (key of the flooding stream)
   };
+  // input polynomials' window (the mask polynomials have none)
+  struct Pre {
+    const char* base = nullptr;
+    u32 tl = 0, th = 0, lh = 0;
+    __device__ __forceinline__ Pre(const DevCtx&, const Params& P, int poly) {
+      if (poly >= P.n_in) return;
+      const Window w(P.pk, P.ac, poly, P.ac.ptr);
+      base = w.base;
+      tl = w.tl;
+      th = w.th;
+      lh = w.lh;
+    }
+  };
   static __device__ __forceinline__ void rebase(Params& P, u64 step) { P.seed += step << 32; }   // as the mask's
-  template <int N>
-  static __device__ __forceinline__ u64 load(const DevCtx& c, const Params& P, const LimbConst& lc, int poly, int,
+  template <int N, bool SPLIT>
+  static __device__ __forceinline__ u64 load(const DevCtx& c, const Params& P, const Pre& pre, const LimbConst& lc, int poly, int,
                                              int e) {
-    if (poly < P.n_in) return scale_msg(gather(P.pk, P.ac, poly, e) & c.t_mask, lc, c);
-    const int idx = poly - P.n_in;
-    const u64 r = scale_msg(P.mpoly[(size_t)idx * N + e], lc, c);
-    if (!c.flood_bits) return r;
-    // flooding noise f (uniform in [-2^b, 2^b)) of returned ciphertext idx: Delta s - f
-    const u64 w = philox_word(philox4x64((u64)(e >> 2), (u64)idx, 0ull, 0ull, P.seed, PENCIL_DOM_FLOOD), e & 3) &
-                  ((2ull << c.flood_bits) - 1);
-    const u64 half = 1ull << c.flood_bits;
-    return w >= half ? sub_mod(r, reduce64(w - half, lc), lc.q) : add_mod(r, reduce64(half - w, lc), lc.q);
+    i64 add = 0;   // flooding noise f (uniform in [-2^b, 2^b)) of returned ciphertext idx: Delta s - f
+    u64 m;
+    if (poly < P.n_in) {
+      m = Window(pre.base, pre.tl, pre.th, pre.lh).get(P.pk, e) & c.t_mask;
+    } else {
+      const int idx = poly - P.n_in;
+      m = P.mpoly[(size_t)idx * N + e];
+      if (c.flood_bits) {
+        const u64 w = philox_word(philox4x64((u64)(e >> 2), (u64)idx, 0ull, 0ull, P.seed, PENCIL_DOM_FLOOD), e & 3) &
+                      ((2ull << c.flood_bits) - 1);
+        add = (i64)((1ull << c.flood_bits) - w);
+      }
+    }
+    if constexpr (SPLIT) {   // |add| <= 2^62: inside the signed range with the product
+      const FoldC f(lc);
+      return fold_s(mul_split(scale_extra(m, c) + add, m, lc.delta_sp, f), f);
+    }
+    const u64 r = scale_msg(m, lc, c);
+    return add >= 0 ? add_mod(r, reduce64((u64)add, lc), lc.q) : sub_mod(r, reduce64((u64)-add, lc), lc.q);
   }
-  template <int N>
+  template <int N, bool SPLIT>
   static __device__ __forceinline__ void store2(const DevCtx& c, const Params& P, const LimbConst&, int poly,
                                                 int limb, int e, u64 x0, u64 x1) {
     u64* dst = poly < P.n_in ? P.out_in + limb_off(poly, limb, c.L, N)
@@ -933,7 +991,18 @@ __device__ __forceinline__ u64 shoup_companion(u64 w, u64 q) {
   return (u64)((((unsigned __int128)w) << 64) / q);
 }
 
-// DO key generation: ternary s, NTT, stored with Shoup companions.
+// Word `at` of a key of `rows` x n values in both product forms: with its Shoup
+// companion, and as a split twiddle behind all of those (mul_split).
+__device__ __forceinline__ void put_key(ulonglong2* key, int rows, size_t at, int n, u64 x, const LimbConst& lc) {
+  key[at] = make_ulonglong2(x, shoup_companion(x, lc.q));
+  const u64 half = lc.q >> 1, y = reduce128(x >> 32, x << 32, lc);
+  const i64 a = x > half ? (i64)(x - lc.q) : (i64)x, b = y > half ? (i64)(y - lc.q) : (i64)y;
+  const u64 m = (1ull << lc.sb) - 1ull;
+  reinterpret_cast<uint4*>(key)[(size_t)rows * n + at] =
+      make_uint4((u32)((u64)a & m), (u32)(a >> lc.sb), (u32)((u64)b & m), (u32)(b >> lc.sb));
+}
+
+// DO key generation: ternary s, NTT, stored for both product forms.
 struct ModeKeygen {
   static constexpr bool kHeavyLoad = true;
   static constexpr bool kQuad = false;
@@ -941,20 +1010,21 @@ struct ModeKeygen {
   static constexpr int kEpilogueUnroll = 1;
   struct Params {
     u64 seed;
-    ulonglong2* sk;   // [L][N]
+    ulonglong2* sk;   // [L][N] with companions, then [L][N] split
   };
+  using Pre = NoPre;
   static __device__ __forceinline__ void rebase(Params&, u64) {}
-  template <int N>
-  static __device__ __forceinline__ u64 load(const DevCtx&, const Params& P, const LimbConst& lc, int, int, int e) {
+  template <int N, bool SPLIT>
+  static __device__ __forceinline__ u64 load(const DevCtx&, const Params& P, const Pre& pre, const LimbConst& lc, int, int, int e) {
     const Philox4 w = philox4x64((u64)(e >> 2), 0ull, 0ull, 0ull, P.seed, PENCIL_DOM_SECRET);
     const u64 r = w.v[e & 3] % 3ull;
     return r == 0 ? lc.q - 1 : r - 1;
   }
-  template <int N>
-  static __device__ __forceinline__ void store2(const DevCtx&, const Params& P, const LimbConst& lc, int, int limb,
+  template <int N, bool SPLIT>
+  static __device__ __forceinline__ void store2(const DevCtx& c, const Params& P, const LimbConst& lc, int, int limb,
                                                 int e, u64 x0, u64 x1) {
-    P.sk[(size_t)limb * N + e] = make_ulonglong2(x0, shoup_companion(x0, lc.q));
-    P.sk[(size_t)limb * N + e + 1] = make_ulonglong2(x1, shoup_companion(x1, lc.q));
+    put_key(P.sk, c.L, limb * N + e, N, x0, lc);
+    put_key(P.sk, c.L, limb * N + e + 1, N, x1, lc);
   }
 };
 
@@ -973,25 +1043,26 @@ struct ModePkKeygen {
   struct Params {
     const int8_t* err;       // [N]
     const ulonglong2* sk;    // [L][N]
-    ulonglong2* key;         // [2][L][N]
+    ulonglong2* key;         // [2][L][N] with companions, then [2][L][N] split
     u64 seed;
   };
+  using Pre = NoPre;
   static __device__ __forceinline__ void rebase(Params&, u64) {}
-  template <int N>
-  static __device__ __forceinline__ u64 load(const DevCtx&, const Params& P, const LimbConst& lc, int, int, int e) {
+  template <int N, bool SPLIT>
+  static __device__ __forceinline__ u64 load(const DevCtx&, const Params& P, const Pre& pre, const LimbConst& lc, int, int, int e) {
     return lift_small(P.err[e], lc.q);
   }
-  template <int N>
+  template <int N, bool SPLIT>
   static __device__ __forceinline__ void store4(const DevCtx& c, const Params& P, const LimbConst& lc, int, int limb,
                                                 int e, const u64* x) {
     const Philox4 w = philox4x64((u64)(e >> 2), 0ull, (u64)limb, 0ull, P.seed, PENCIL_DOM_PK_A);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const u64 a = uniform_mod_q(w.v[i], e + i, 0, limb, P.seed, PENCIL_DOM_PK_A, lc);
+      const u64 a = reduce64(uniform_word(w.v[i], e + i, 0, limb, P.seed, PENCIL_DOM_PK_A, lc), lc);
       const ulonglong2 s = __ldg(P.sk + (size_t)limb * N + e + i);
       const u64 p0 = neg_mod(add_mod(mul_shoup(a, s.x, s.y, lc.q), x[i], lc.q), lc.q);
-      P.key[(size_t)limb * N + e + i] = make_ulonglong2(p0, shoup_companion(p0, lc.q));
-      P.key[(size_t)(c.L + limb) * N + e + i] = make_ulonglong2(a, shoup_companion(a, lc.q));
+      put_key(P.key, 2 * c.L, (size_t)limb * N + e + i, N, p0, lc);
+      put_key(P.key, 2 * c.L, (size_t)(c.L + limb) * N + e + i, N, a, lc);
     }
   }
 };
@@ -1006,13 +1077,16 @@ struct ModePkU {
     const int8_t* u;   // [ct][N]
     u64* u_hat;        // [ct][L][N]
   };
+  using Pre = NoPre;
   static __device__ __forceinline__ void rebase(Params&, u64) {}
-  template <int N>
-  static __device__ __forceinline__ u64 load(const DevCtx&, const Params& P, const LimbConst& lc, int poly, int,
+  template <int N, bool SPLIT>
+  static __device__ __forceinline__ u64 load(const DevCtx&, const Params& P, const Pre& pre, const LimbConst& lc, int poly, int,
                                              int e) {
-    return lift_small(P.u[(size_t)poly * N + e], lc.q);
+    const int v = P.u[(size_t)poly * N + e];
+    if constexpr (SPLIT) return (u64)(i64)v;
+    return lift_small(v, lc.q);
   }
-  template <int N>
+  template <int N, bool SPLIT>
   static __device__ __forceinline__ void store2(const DevCtx& c, const Params& P, const LimbConst&, int poly,
                                                 int limb, int e, u64 x0, u64 x1) {
     *reinterpret_cast<ulonglong2*>(P.u_hat + limb_off(poly, limb, c.L, N) + e) = make_ulonglong2(x0, x1);
@@ -1034,28 +1108,49 @@ struct ModeEncryptPk {
     const int8_t* e1;          // [ct][N]
     const int8_t* e2;          // [ct][N]
     const u64* u_hat;          // [ct][L][N]
-    const ulonglong2* key;     // [2][L][N]
+    const ulonglong2* key;     // [2][L][N] with companions, then [2][L][N] split
     u64* ct;                   // [ct][2][L][N]
   };
+  struct Pre {
+    Window win;
+    __device__ __forceinline__ Pre(const DevCtx&, const Params& P, int poly) : win(P.pk, P.ac, poly >> 1, P.ac.ptr) {}
+  };
   static __device__ __forceinline__ void rebase(Params&, u64) {}
-  template <int N>
-  static __device__ __forceinline__ u64 load(const DevCtx& c, const Params& P, const LimbConst& lc, int poly, int,
+  template <int N, bool SPLIT>
+  static __device__ __forceinline__ u64 load(const DevCtx& c, const Params& P, const Pre& pre, const LimbConst& lc, int poly, int,
                                              int e) {
     const int ct = poly >> 1;
-    if (poly & 1) return lift_small(P.e2[(size_t)ct * N + e], lc.q);
-    const u64 r = scale_msg(gather(P.pk, P.ac, ct, e) & c.t_mask, lc, c);
+    if (poly & 1) {
+      const int e2 = P.e2[(size_t)ct * N + e];
+      if constexpr (SPLIT) return (u64)(i64)e2;
+      return lift_small(e2, lc.q);
+    }
+    const u64 m = pre.win.get(P.pk, e) & c.t_mask;
     const int ee = P.e1[(size_t)ct * N + e];
+    if constexpr (SPLIT) {
+      const FoldC f(lc);
+      return fold_s(mul_split(scale_extra(m, c) + (i64)ee, m, lc.delta_sp, f), f);
+    }
+    const u64 r = scale_msg(m, lc, c);
     return ee >= 0 ? add_mod(r, (u64)ee, lc.q) : sub_mod(r, (u64)(-ee), lc.q);
   }
-  template <int N>
+  template <int N, bool SPLIT>
   static __device__ __forceinline__ void store2(const DevCtx& c, const Params& P, const LimbConst& lc, int poly,
                                                 int limb, int e, u64 x0, u64 x1) {
     const int ct = poly >> 1, comp = poly & 1;
     const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(P.u_hat + limb_off(ct, limb, c.L, N) + e);
-    const ulonglong2 k0 = __ldg(P.key + (size_t)(comp * c.L + limb) * N + e);
-    const ulonglong2 k1 = __ldg(P.key + (size_t)(comp * c.L + limb) * N + e + 1);
-    const u64 y0 = add_mod(x0, mul_shoup(u.x, k0.x, k0.y, lc.q), lc.q);
-    const u64 y1 = add_mod(x1, mul_shoup(u.y, k1.x, k1.y, lc.q), lc.q);
+    const size_t at = (size_t)(comp * c.L + limb) * N + e;
+    u64 y0, y1;
+    if constexpr (SPLIT) {
+      const FoldC f(lc);
+      const uint4* key = reinterpret_cast<const uint4*>(P.key) + 2 * (size_t)c.L * N + at;
+      y0 = csub(fold_u(mul_split(x0 + lc.q, u.x, __ldg(key), f), f), lc.q);
+      y1 = csub(fold_u(mul_split(x1 + lc.q, u.y, __ldg(key + 1), f), f), lc.q);
+    } else {
+      const ulonglong2 k0 = __ldg(P.key + at), k1 = __ldg(P.key + at + 1);
+      y0 = add_mod(x0, mul_shoup(u.x, k0.x, k0.y, lc.q), lc.q);
+      y1 = add_mod(x1, mul_shoup(u.y, k1.x, k1.y, lc.q), lc.q);
+    }
     *reinterpret_cast<ulonglong2*>(P.ct + ct_off(ct, comp, limb, c.L, N) + e) = make_ulonglong2(y0, y1);
   }
 };
@@ -1072,15 +1167,22 @@ struct ModeDecrypt {
   static constexpr int kEpilogueUnroll = 16;
   struct Params {
     const u64* ct;          // [count][2][L][N]
-    const ulonglong2* sk;   // [L][N]
+    const ulonglong2* sk;   // [L][N] with companions, then [L][N] split
     u64* out;               // [count][L][N]
     int skip_c0;
   };
+  using Pre = NoPre;
   static __device__ __forceinline__ void rebase(Params&, u64) {}
-  template <int N>
-  static __device__ __forceinline__ u64 load(const DevCtx& c, const Params& P, const LimbConst& lc, int poly,
+  template <int N, bool SPLIT>
+  static __device__ __forceinline__ u64 load(const DevCtx& c, const Params& P, const Pre& pre, const LimbConst& lc, int poly,
                                              int limb, int e) {
     const u64 c1 = __ldg(P.ct + ct_off(poly, 1, limb, c.L, N) + e);
+    if constexpr (SPLIT) {   // c0 + c1 s in [-0.6, 2.6], folded; c1 s alone is in range
+      const FoldC f(lc);
+      const uint4 s = __ldg(reinterpret_cast<const uint4*>(P.sk) + (size_t)(c.L + limb) * N + e);
+      if (P.skip_c0) return mul_split(0, c1, s, f);
+      return fold_s(mul_split(__ldg(P.ct + ct_off(poly, 0, limb, c.L, N) + e), c1, s, f), f);
+    }
     const ulonglong2 s = __ldg(P.sk + (size_t)limb * N + e);
     const u64 c1s = mul_shoup(c1, s.x, s.y, lc.q);
     if (P.skip_c0) return c1s;
@@ -1115,11 +1217,12 @@ struct ModeDecryptFused {
     u64* y1;
     int check;
   };
+  using Pre = NoPre;
   static __device__ __forceinline__ void rebase(Params&, u64) {}
-  template <int N>
-  static __device__ __forceinline__ u64 load(const DevCtx& c, const Params& P, const LimbConst& lc, int poly,
+  template <int N, bool SPLIT>
+  static __device__ __forceinline__ u64 load(const DevCtx& c, const Params& P, const Pre& pre, const LimbConst& lc, int poly,
                                              int limb, int e) {
-    return ModeDecrypt::template load<N>(c, P.d, lc, poly, limb, e);
+    return ModeDecrypt::template load<N, SPLIT>(c, P.d, pre, lc, poly, limb, e);
   }
   template <int N>
   static __device__ __forceinline__ void store(const DevCtx&, const Params&, const LimbConst& lc, int, int, int e,
@@ -1134,6 +1237,7 @@ struct ModeDecryptFused {
     cl.sync();   // every limb's residues are in its CTA's shared memory
     const int T = (int)blockDim.x;
     const int L = c.L;
+    const Window win(P.pk, P.ac, poly, P.y1);
     const ulonglong2* res[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j)
@@ -1141,8 +1245,9 @@ struct ModeDecryptFused {
     // coefficient pairs (2 p, 2 p + 1): 16-byte remote loads
 #pragma unroll 2
     for (int p = (int)blockIdx.y * T + (int)threadIdx.x; p < N / 2; p += L * T) {
-      const i64 f0 = out_index(P.pk, P.ac, poly, 2 * p), f1 = out_index(P.pk, P.ac, poly, 2 * p + 1);
-      if (f0 < 0 && f1 < 0) continue;
+      const ulonglong2 e0 = __ldg(P.pk.tab + 2 * p), e1 = __ldg(P.pk.tab + 2 * p + 1);
+      const bool h0 = win.has(e0), h1 = win.has(e1);
+      if (!h0 && !h1) continue;
       CrtSum s0{0, 0}, s1{0, 0};
 #pragma unroll
       for (int j = 0; j < 8; ++j)
@@ -1151,8 +1256,8 @@ struct ModeDecryptFused {
           crt_add(s0, y.x, c.limb[j]);
           crt_add(s1, y.y, c.limb[j]);
         }
-      if (f0 >= 0) P.y1[f0] = crt_round(s0, c.t_mask, P.check, c.status);
-      if (f1 >= 0) P.y1[f1] = crt_round(s1, c.t_mask, P.check, c.status);
+      if (h0) *reinterpret_cast<u64*>(const_cast<char*>(win.at(e0))) = crt_round(s0, c.t_mask, P.check, c.status);
+      if (h1) *reinterpret_cast<u64*>(const_cast<char*>(win.at(e1))) = crt_round(s1, c.t_mask, P.check, c.status);
     }
     cl.sync();   // the other CTAs have finished reading this one's shared memory
   }
@@ -1174,16 +1279,17 @@ struct ModeCompact {
     u64* c0c;               // [L][out_elems]
     long long out_elems;
   };
+  using Pre = NoPre;
   static __device__ __forceinline__ void rebase(Params&, u64) {}
-  template <int N>
-  static __device__ __forceinline__ u64 load(const DevCtx& c, const Params& P, const LimbConst&, int poly, int limb,
+  template <int N, bool SPLIT>
+  static __device__ __forceinline__ u64 load(const DevCtx& c, const Params& P, const Pre& pre, const LimbConst&, int poly, int limb,
                                              int e) {
     return __ldg(P.ct + ct_off(poly, 0, limb, c.L, N) + e);
   }
   template <int N>
   static __device__ __forceinline__ void store(const DevCtx&, const Params& P, const LimbConst& lc, int poly,
                                                int limb, int e, u64 x) {
-    const i64 flat = out_index(P.pk, P.ac, poly, e);
+    const i64 flat = Window(P.pk, P.ac, poly, nullptr).index(P.pk, e);
     if (flat >= 0) P.c0c[(size_t)limb * P.out_elems + flat] = x;   // x = N^{-1} INTT, canonical
   }
 };
