@@ -782,27 +782,32 @@ cudaError_t launch_mac(const DevCtx& ctx, const MacParams& P0, bool dual, cudaSt
 // w = Philox(key (seed, 3), counter (i/4, ct, 0, 0)) word i%4.
 __device__ __forceinline__ int8_t cdt_sample(u64 w) {
   const u64 u = w & 0x7FFFFFFFFFFFFFFFull;
+  const u32 uh = (u32)(u >> 32);
+  // the thresholds' high words decide unless the last one passed equals u's
+  // (probability below 2^-26; they ascend, so no other can)
   int mag = 0;
 #pragma unroll
-  for (int j = 0; j < PENCIL_CDT_LEN; ++j) mag += (u >= c_cdt[j]) ? 1 : 0;
+  for (int j = 0; j < PENCIL_CDT_LEN; ++j) mag += uh >= (u32)(c_cdt[j] >> 32) ? 1 : 0;
+  if (mag && (u32)(c_cdt[mag - 1] >> 32) == uh) {
+    mag = 0;
+#pragma unroll 1
+    for (int j = 0; j < PENCIL_CDT_LEN; ++j) mag += u >= c_cdt[j] ? 1 : 0;
+  }
   return (int8_t)((w >> 63) ? -mag : mag);
 }
 
-__global__ void k_sample_err(u64 seed, int first, int count, int n, int8_t* out, u64 dom) {
-  const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const int per = n >> 2;
-  if (id >= (long long)count * per) return;
-  const int ct = first + (int)(id / per);
-  const int blk = (int)(id % per);
+__global__ void __launch_bounds__(256) k_sample_err(u64 seed, int first, int log_n, int8_t* out, u64 dom) {
+  const int lg = log_n - 10, ct = first + (int)(blockIdx.x >> lg);
+  const int blk = ((int)(blockIdx.x & ((1u << lg) - 1u)) << 8) + threadIdx.x;
   const Philox4 w = philox4x64((u64)blk, (u64)ct, 0ull, 0ull, seed, dom);
-  reinterpret_cast<char4*>(out + (size_t)ct * n)[blk] =
+  reinterpret_cast<char4*>(out + ((size_t)ct << log_n))[blk] =
       make_char4(cdt_sample(w.v[0]), cdt_sample(w.v[1]), cdt_sample(w.v[2]), cdt_sample(w.v[3]));
 }
 
 cudaError_t launch_sample_err(u64 seed, int first, int count, int n, int8_t* out, cudaStream_t s, u64 dom) {
   const long long total = (long long)count * (n >> 2);
   if (total == 0) return cudaSuccess;
-  k_sample_err<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(seed, first, count, n, out, dom);
+  k_sample_err<<<(unsigned)(total / 256), 256, 0, s>>>(seed, first, 31 - __builtin_clz((unsigned)n), out, dom);
   return cudaGetLastError();
 }
 
@@ -838,57 +843,54 @@ cudaError_t launch_sample_pk(u64 seed, int first, int count, int n, int8_t* e1, 
 // Mask polynomial of each output ciphertext: at coefficients carrying output
 // element `flat`, Philox(key (seed, 4), counter (flat/4, 0, 0, 0)) word flat%4;
 // elsewhere Philox(key (seed, 5), counter (i/4, ct, 0, 0)) word i%4; mod t.
-// Coefficients 4 blk .. 4 blk + 3 of the mask polynomial of output ciphertext ct.
-// Coefficients 4 blk .. 4 blk + 3 of output polynomial ct.  Consecutive
-// coefficients usually carry consecutive outputs, so one Philox block of the
-// element stream is reused while flat / 4 stays the same; the padding stream
-// is drawn only if some coefficient carries no output.
-__device__ __forceinline__ void mask_poly_block(const DevCtx& ctx, const Packing& pk, const Accessor& ac, u64 seed,
+// Coefficients 4 blk .. 4 blk + 3 of output polynomial ct.  The padding stream's block is
+// drawn where some coefficient carries no output; then each pass evaluates one block of
+// the element stream for every coefficient that draws from it, so a warp takes as many
+// passes as its worst thread has different blocks: one or two, where one per coefficient
+// took four (rows of outputs start at any flat % 4; 1920 polynomials of 28 x 19 tiles at
+// N = 8192: 239 us with four).
+__device__ __forceinline__ void mask_poly_block(const DevCtx& ctx, const Packing& pk, const Window& win, u64 seed,
                                                 int ct, int blk, u64* out_ct) {
   i64 flat[4];
-  bool any_pad = false;
-  const Window win(pk, ac, ct, nullptr);
+  u32 todo = 0;
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     flat[i] = win.index(pk, 4 * blk + i);
-    any_pad |= flat[i] < 0;
+    todo |= flat[i] >= 0 ? 1u << i : 0u;
   }
-  Philox4 pad = {{0, 0, 0, 0}};
-  if (any_pad) pad = philox4x64((u64)blk, (u64)ct, 0ull, 0ull, seed, PENCIL_DOM_MASK_PAD);
-  Philox4 el = {{0, 0, 0, 0}};
-  i64 cur = -1;
-  u64 r[4];
+  Philox4 r = {{0, 0, 0, 0}};
+  if (todo != 15u) r = philox4x64((u64)blk, (u64)ct, 0ull, 0ull, seed, PENCIL_DOM_MASK_PAD);
+  while (todo) {
+    i64 src = 0;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    u64 w = philox_word(pad, i);
-    if (flat[i] >= 0) {
-      if ((flat[i] >> 2) != cur) {
-        cur = flat[i] >> 2;
-        el = philox4x64((u64)cur, 0ull, 0ull, 0ull, seed, PENCIL_DOM_MASK);
+    for (int i = 3; i >= 0; --i)
+      if (todo >> i & 1u) src = flat[i] >> 2;
+    const Philox4 w = philox4x64((u64)src, 0ull, 0ull, 0ull, seed, PENCIL_DOM_MASK);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if ((todo >> i & 1u) && flat[i] >> 2 == src) {
+        r.v[i] = philox_word(w, (int)(flat[i] & 3));
+        todo &= ~(1u << i);
       }
-      w = philox_word(el, (int)(flat[i] & 3));
-    }
-    r[i] = w & ctx.t_mask;
   }
   ulonglong2* o = reinterpret_cast<ulonglong2*>(out_ct + 4 * blk);
-  o[0] = make_ulonglong2(r[0], r[1]);
-  o[1] = make_ulonglong2(r[2], r[3]);
+  o[0] = make_ulonglong2(r.v[0] & ctx.t_mask, r.v[1] & ctx.t_mask);
+  o[1] = make_ulonglong2(r.v[2] & ctx.t_mask, r.v[3] & ctx.t_mask);
 }
 
-__global__ void k_mask_poly(DevCtx ctx, Packing pk, Accessor ac, u64 seed, int count, u64* out) {
-  const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const int n = ctx.n;
-  const int per = n >> 2;
-  if (id >= (long long)count * per) return;
-  const int ct = (int)(id / per);
-  mask_poly_block(ctx, pk, ac, seed, ct, (int)(id % per), out + (size_t)ct * n);
+// (a CTA of 256 threads stays inside one polynomial: its window is uniform)
+__global__ void __launch_bounds__(256) k_mask_poly(const __grid_constant__ DevCtx ctx, const __grid_constant__ Packing pk,
+                                                   const __grid_constant__ Accessor ac, u64 seed, u64* out) {
+  const int lg = ctx.log_n - 10, ct = blockIdx.x >> lg;
+  const int blk = ((int)(blockIdx.x & ((1u << lg) - 1u)) << 8) + threadIdx.x;
+  mask_poly_block(ctx, pk, Window(pk, ac, ct, nullptr), seed, ct, blk, out + ((size_t)ct << ctx.log_n));
 }
 
 cudaError_t launch_mask_poly(const DevCtx& ctx, const Packing& pk, const Accessor& ac, u64 seed, int count, u64* out,
                              cudaStream_t s) {
   const long long total = (long long)count * (ctx.n >> 2);
   if (total == 0) return cudaSuccess;
-  k_mask_poly<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(ctx, pk, ac, seed, count, out);
+  k_mask_poly<<<(unsigned)(total / 256), 256, 0, s>>>(ctx, pk, ac, seed, out);
   return cudaGetLastError();
 }
 
@@ -898,14 +900,39 @@ __device__ __forceinline__ void mo_share_block(u64 seed, long long count, u64 t_
                                                int co, u64* y0, long long blk) {
   if (blk * 4 >= count) return;
   const Philox4 w = philox4x64((u64)blk, 0ull, 0ull, 0ull, seed, PENCIL_DOM_MASK);
+  u64 v[4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const long long flat = blk * 4 + i;
-    if (flat < count) {
-      u64 v = w.v[i] & t_mask;
-      if (bias) v = (v + __ldg(bias + (flat / hw) % co)) & t_mask;
-      y0[flat] = v;
+  for (int i = 0; i < 4; ++i) v[i] = w.v[i] & t_mask;
+  if (bias) {   // channel of the first element by one division, the others by counting
+    const long long f0 = blk * 4;
+    long long p;
+    int c;
+    if (count >> 31) {
+      const long long row = f0 / hw;
+      p = f0 - row * hw;
+      c = (int)(row % co);
+    } else {
+      const u32 row = (u32)f0 / (u32)hw;
+      p = f0 - (long long)row * hw;
+      c = (int)(row % (u32)co);
     }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      v[i] = (v[i] + __ldg(bias + c)) & t_mask;
+      if (++p == hw) {
+        p = 0;
+        c = c + 1 == co ? 0 : c + 1;
+      }
+    }
+  }
+  u64* dst = y0 + blk * 4;
+  if (blk * 4 + 4 <= count && !(reinterpret_cast<uintptr_t>(dst) & 15)) {
+    reinterpret_cast<ulonglong2*>(dst)[0] = make_ulonglong2(v[0], v[1]);
+    reinterpret_cast<ulonglong2*>(dst)[1] = make_ulonglong2(v[2], v[3]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (blk * 4 + i < count) dst[i] = v[i];
   }
 }
 
@@ -926,11 +953,11 @@ cudaError_t launch_mo_share(u64 seed, long long count, u64 t_mask, const u64* bi
 // y_j = x_j * (q/q_j)^{-1} mod q_j (first half), then crt_add / crt_round.
 // c0c (compact send form, else null): c0 at the output coefficients in
 // coefficient form, [L][out_elems]; added as c0c * qtil to the INTT(c1 s) residues.
-__device__ __forceinline__ void decrypt_combine_one(const DevCtx& ctx, const Packing& pk, const Accessor& ac,
+__device__ __forceinline__ void decrypt_combine_one(const DevCtx& ctx, const Packing& pk, const Window& win,
                                                     const u64* yres, int ct, int e, int check, u64* y1,
                                                     const u64* c0c = nullptr, long long out_elems = 0) {
   const int n = ctx.n;
-  const i64 flat = Window(pk, ac, ct, nullptr).index(pk, e);
+  const i64 flat = win.index(pk, e);
   if (flat < 0) return;
   CrtSum sum{0, 0};
   for (int j = 0; j < ctx.L; ++j) {
@@ -942,12 +969,14 @@ __device__ __forceinline__ void decrypt_combine_one(const DevCtx& ctx, const Pac
   y1[flat] = crt_round(sum, ctx.t_mask, check, ctx.status);
 }
 
-__global__ void k_decrypt_combine(DevCtx ctx, Packing pk, Accessor ac, const u64* yres, int first, int count,
-                                  int check, u64* y1, const u64* c0c, long long out_elems) {
-  const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const int n = ctx.n;
-  if (id >= (long long)count * n) return;
-  decrypt_combine_one(ctx, pk, ac, yres, first + (int)(id / n), (int)(id % n), check, y1, c0c, out_elems);
+__global__ void __launch_bounds__(256) k_decrypt_combine(const __grid_constant__ DevCtx ctx,
+                                                         const __grid_constant__ Packing pk,
+                                                         const __grid_constant__ Accessor ac, const u64* yres,
+                                                         int first, int check, u64* y1, const u64* c0c,
+                                                         long long out_elems) {
+  const int lg = ctx.log_n - 8, ct = first + (int)(blockIdx.x >> lg);
+  const int e = ((int)(blockIdx.x & ((1u << lg) - 1u)) << 8) + threadIdx.x;
+  decrypt_combine_one(ctx, pk, Window(pk, ac, ct, nullptr), yres, ct, e, check, y1, c0c, out_elems);
 }
 
 cudaError_t launch_decrypt_combine(const DevCtx& ctx, const Packing& pk, const Accessor& ac, const u64* yres,
@@ -955,8 +984,7 @@ cudaError_t launch_decrypt_combine(const DevCtx& ctx, const Packing& pk, const A
                                    long long out_elems) {
   const long long total = (long long)count * ctx.n;
   if (total == 0) return cudaSuccess;
-  k_decrypt_combine<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(ctx, pk, ac, yres, first, count, check, y1, c0c,
-                                                                    out_elems);
+  k_decrypt_combine<<<(unsigned)(total / 256), 256, 0, s>>>(ctx, pk, ac, yres, first, check, y1, c0c, out_elems);
   return cudaGetLastError();
 }
 
@@ -1062,30 +1090,65 @@ cudaError_t launch_ring(const RingParams& P, int sms, cudaStream_t s) {
 }
 
 // Bias gradient: out[o] = sum_{b, i, j} g[b, o, i, j] mod t   (g row-major [B][Co][HW]).
+// A cluster of CTAs per channel, each a contiguous part of the B HW elements; the first
+// CTA adds the others' sums from their shared memory.  One CTA per channel left most of
+// the GPU idle on few channels (16 channels x 65 536 elements: 77 us a launch).
+#define BIAS_PARTS 8
 __global__ void __launch_bounds__(256) k_bias_grad(const u64* g, int B, int Co, long long hw, u64 t_mask, u64* out) {
-  const int o = blockIdx.x;
-  const long long R = (long long)B * hw;
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  const int parts = (int)gridDim.x, o = blockIdx.y;
+  const long long R = (long long)B * hw, per = (R + parts - 1) / parts;
+  const long long first = blockIdx.x * per, last = min(R, first + per);
+  const u64* go = g + o * hw;
+  const long long row = (long long)Co * hw;
   u64 acc = 0;
-  for (long long r = threadIdx.x; r < R; r += blockDim.x) {
-    const long long b = r / hw, p = r % hw;
-    acc += __ldg(g + (b * Co + o) * hw + p);
+  if (R >> 31) {
+    for (long long r = first + threadIdx.x; r < last; r += 256) {
+      const long long b = r / hw;
+      acc += __ldg(go + b * row + (r - b * hw));
+    }
+  } else {
+#pragma unroll 4
+    for (u32 r = (u32)first + threadIdx.x; r < (u32)last; r += 256) {
+      const u32 b = r / (u32)hw;
+      acc += __ldg(go + (long long)b * row + (r - b * (u32)hw));
+    }
   }
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
-  __shared__ u64 part[8];
+  __shared__ u64 part[8], total;
   if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = acc;
   __syncthreads();
   if (threadIdx.x == 0) {
     u64 s = 0;
     for (int w = 0; w < 8; ++w) s += part[w];
+    total = s;
+  }
+  cl.sync();
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    u64 s = 0;
+    for (int k = 0; k < parts; ++k) s += *cl.map_shared_rank(&total, k);
     out[o] = s & t_mask;
   }
+  cl.sync();   // the others' shared memory has been read
 }
 
 cudaError_t launch_bias_grad(const u64* g, int B, int Co, long long hw, u64 t_mask, u64* out, cudaStream_t s) {
   if (Co == 0) return cudaSuccess;
-  k_bias_grad<<<Co, 256, 0, s>>>(g, B, Co, hw, t_mask, out);
-  return cudaGetLastError();
+  const unsigned parts = (long long)B * hw > 4096 ? BIAS_PARTS : 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(parts, (unsigned)Co);
+  cfg.blockDim = dim3(256);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = parts;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_bias_grad, g, B, Co, hw, t_mask, out);
 }
 
 // ------------------------------------------------------------------ linear combinations of shares
@@ -1093,26 +1156,66 @@ cudaError_t launch_bias_grad(const u64* g, int B, int Co, long long hw, u64 t_ma
 // shares are linear combinations over Z_t, t = 2^t_bits (u64 wrap-around is
 // exact mod t):  out[e] = addend[e] (+ or -) sum_{i2, i} k[i2 terms + i]
 // src[off + (e / inner) outer + e % inner + i tstride + i2 tstride2].
-__global__ void k_lincomb(LincombP P, u64 t_mask) {
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < P.count; e += stride) {
-    const long long base = P.off + (e / P.inner) * P.outer + e % P.inner;
-    u64 acc = 0;
-    for (int i2 = 0; i2 < P.terms2; ++i2) {
-      const u64* src = P.src + base + i2 * P.tstride2;
-      const u64* k = P.k + i2 * P.terms;
-      for (int i = 0; i < P.terms; ++i) acc += k[i] * __ldg(src + i * P.tstride);
+// Bound by memory (64 terms: 64 words read per word written); a thread takes V
+// consecutive elements (V = 2, 16-byte accesses, when every offset and stride is even
+// and the tensors are 16-byte aligned) with eight terms' loads in flight.
+template <int V>
+__global__ void __launch_bounds__(256) k_lincomb(const __grid_constant__ LincombP P, u64 t_mask) {
+  const long long stride = (long long)gridDim.x * blockDim.x * V;
+  for (long long e = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * V; e < P.count; e += stride) {
+    long long row, at;
+    if ((P.count | P.inner) >> 31) {
+      row = e / P.inner;
+      at = e - row * P.inner;
+    } else {
+      row = (u32)e / (u32)P.inner;
+      at = e - row * P.inner;
     }
-    u64 v = P.addend ? __ldg(P.addend + e) : 0ull;
-    v = P.negate ? v - acc : v + acc;
-    P.out[e] = v & t_mask;
+    const u64* base = P.src + P.off + row * P.outer + at;
+    u64 acc0 = 0, acc1 = 0;
+    for (int i2 = 0; i2 < P.terms2; ++i2) {
+      const u64* src = base + i2 * P.tstride2;
+      const u64* k = P.k + i2 * P.terms;
+#pragma unroll 8
+      for (int i = 0; i < P.terms; ++i) {
+        if constexpr (V == 2) {
+          const ulonglong2 x = __ldg(reinterpret_cast<const ulonglong2*>(src + i * P.tstride));
+          acc0 += k[i] * x.x;
+          acc1 += k[i] * x.y;
+        } else {
+          acc0 += k[i] * __ldg(src + i * P.tstride);
+        }
+      }
+    }
+    if (P.negate) {
+      acc0 = 0 - acc0;
+      acc1 = 0 - acc1;
+    }
+    if constexpr (V == 2) {
+      if (P.addend) {
+        const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(P.addend + e);
+        acc0 += a.x;
+        acc1 += a.y;
+      }
+      *reinterpret_cast<ulonglong2*>(P.out + e) = make_ulonglong2(acc0 & t_mask, acc1 & t_mask);
+    } else {
+      if (P.addend) acc0 += P.addend[e];
+      P.out[e] = acc0 & t_mask;
+    }
   }
 }
 
 cudaError_t launch_lincomb(const LincombP& P, u64 t_mask, cudaStream_t s) {
   if (P.count <= 0) return cudaSuccess;
-  const long long blocks = std::min<long long>((P.count + 255) / 256, 152LL * 16);
-  k_lincomb<<<(unsigned)blocks, 256, 0, s>>>(P, t_mask);
+  const long long all = P.off | P.inner | P.outer | P.count | P.tstride | P.tstride2;
+  const uintptr_t ptrs = reinterpret_cast<uintptr_t>(P.src) | reinterpret_cast<uintptr_t>(P.out) |
+                         reinterpret_cast<uintptr_t>(P.addend);
+  const bool pairs = !(all & 1) && !(ptrs & 15);
+  const long long blocks = std::min<long long>((P.count + (pairs ? 511 : 255)) / (pairs ? 512 : 256), 152LL * 16);
+  if (pairs)
+    k_lincomb<2><<<(unsigned)blocks, 256, 0, s>>>(P, t_mask);
+  else
+    k_lincomb<1><<<(unsigned)blocks, 256, 0, s>>>(P, t_mask);
   return cudaGetLastError();
 }
 
@@ -1128,33 +1231,28 @@ cudaError_t launch_lincomb(const LincombP& P, u64 t_mask, cudaStream_t s) {
 // stages); waits are bounded by clock64 and, on expiry, set PENCIL_E_TIMEOUT in
 // the status word and abort the remaining items instead of reading stale data.
 // ------------------------------------------------------------------ small multi-plan kernels
-__global__ void k_sample_err_multi(const SampleP* __restrict__ Ps, const int2* __restrict__ items, long long n_items,
-                                   int n, const u64* step) {
-  const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const int per = n >> 2;
-  if (id >= n_items * per) return;
-  const int2 it = items[id / per];
-  const int blk = (int)(id % per);
+__global__ void __launch_bounds__(256) k_sample_err_multi(const SampleP* __restrict__ Ps,
+                                                          const int2* __restrict__ items, int log_n,
+                                                          const u64* step) {
+  const int lg = log_n - 10;
+  const int2 it = items[blockIdx.x >> lg];
+  const int blk = ((int)(blockIdx.x & ((1u << lg) - 1u)) << 8) + threadIdx.x;
   const SampleP P = Ps[it.x];
   const u64 seed = P.seed + ((step ? *step : 0ull) << 32);
   const Philox4 w = philox4x64((u64)blk, (u64)it.y, 0ull, 0ull, seed, PENCIL_DOM_E);
-  int8_t v[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) v[i] = cdt_sample(w.v[i]);
-  reinterpret_cast<char4*>(P.err + (size_t)it.y * n)[blk] = make_char4(v[0], v[1], v[2], v[3]);
+  reinterpret_cast<char4*>(P.err + ((size_t)it.y << log_n))[blk] =
+      make_char4(cdt_sample(w.v[0]), cdt_sample(w.v[1]), cdt_sample(w.v[2]), cdt_sample(w.v[3]));
 }
 
-__global__ void k_mask_poly_multi(DevCtx ctx, const MaskPolyP* __restrict__ Ps, const int2* __restrict__ items,
-                                  long long n_items, const u64* step) {
-  const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const int n = ctx.n;
-  const int per = n >> 2;
-  if (id >= n_items * per) return;
-  const int2 it = items[id / per];
-  const int blk = (int)(id % per);
-  const MaskPolyP P = Ps[it.x];
+__global__ void __launch_bounds__(256) k_mask_poly_multi(const __grid_constant__ DevCtx ctx,
+                                                         const MaskPolyP* __restrict__ Ps,
+                                                         const int2* __restrict__ items, const u64* step) {
+  const int lg = ctx.log_n - 10;
+  const int2 it = items[blockIdx.x >> lg];
+  const int blk = ((int)(blockIdx.x & ((1u << lg) - 1u)) << 8) + threadIdx.x;
+  const MaskPolyP& P = Ps[it.x];
   const u64 seed = P.seed + ((step ? *step : 0ull) << 32);
-  mask_poly_block(ctx, P.pk, P.ac, seed, it.y, blk, P.out + (size_t)it.y * n);
+  mask_poly_block(ctx, P.pk, Window(P.pk, P.ac, it.y, nullptr), seed, it.y, blk, P.out + ((size_t)it.y << ctx.log_n));
 }
 
 __global__ void k_mo_share_multi(const MoShareP* __restrict__ Ps, const int2* __restrict__ items, long long n_items,
@@ -1169,14 +1267,14 @@ __global__ void k_mo_share_multi(const MoShareP* __restrict__ Ps, const int2* __
   mo_share_block(seed, P.count, t_mask, P.bias, P.hw, P.co, P.y0, blk);
 }
 
-__global__ void k_combine_multi(DevCtx ctx, const CombineP* __restrict__ Ps, const int2* __restrict__ items,
-                                long long n_items) {
-  const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const int n = ctx.n;
-  if (id >= n_items * n) return;
-  const int2 it = items[id / n];
-  const CombineP P = Ps[it.x];
-  decrypt_combine_one(ctx, P.pk, P.ac, P.yres, it.y, (int)(id % n), 1, P.y1);
+__global__ void __launch_bounds__(256) k_combine_multi(const __grid_constant__ DevCtx ctx,
+                                                       const CombineP* __restrict__ Ps,
+                                                       const int2* __restrict__ items) {
+  const int lg = ctx.log_n - 8;
+  const int2 it = items[blockIdx.x >> lg];
+  const int e = ((int)(blockIdx.x & ((1u << lg) - 1u)) << 8) + threadIdx.x;
+  const CombineP& P = Ps[it.x];
+  decrypt_combine_one(ctx, P.pk, Window(P.pk, P.ac, it.y, nullptr), P.yres, it.y, e, 1, P.y1);
 }
 
 // ready[l] = step + 1 for every layer except one the host asked to withhold
@@ -1233,7 +1331,7 @@ __global__ void __launch_bounds__(MMA_THREADS, NT == 8 ? 2 : 4) k_mac_persistent
                                                                    const int4* __restrict__ items, long long n_mma,
                                                                    long long n_split, const u64* ready,
                                                                    const u64* step, int* abort_flag) {
-  extern __shared__ __align__(16) u64 ring[];
+  extern __shared__ __align__(128) u64 ring[];
   constexpr int MT = PENCIL_BATCH_MMA_ROWS, NC = PENCIL_BATCH_MMA_COLS;
   const u64 want = (step ? *step : 0ull) + 1;
   const long long lanes = (long long)ctx.L * ctx.n;
@@ -1304,14 +1402,13 @@ cudaError_t launch_batch_forward(const DevCtx& ctx, const BatchDev& B, cudaStrea
     if (e != cudaSuccess) return e;
   }
   if (B.n_in) {
-    k_sample_err_multi<<<blocks_for(B.n_in * (n / 4), 256), 256, 0, s>>>(B.sample, B.items_in, B.n_in, n, B.step);
+    k_sample_err_multi<<<blocks_for(B.n_in * (n / 4), 256), 256, 0, s>>>(B.sample, B.items_in, ctx.log_n, B.step);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     e = ntt_multi<ModeEncrypt, false>(ctx, B.encrypt, B.items_in, B.n_in, B.step, s);
     if (e != cudaSuccess) return e;
   }
   if (B.n_out) {   // the MO's mask s, then NTT(Delta x0) and NTT(Delta s) of every layer in one launch
-    k_mask_poly_multi<<<blocks_for(B.n_out * (n / 4), 256), 256, 0, s>>>(ctx, B.maskpoly, B.items_out, B.n_out,
-                                                                            B.step);
+    k_mask_poly_multi<<<blocks_for(B.n_out * (n / 4), 256), 256, 0, s>>>(ctx, B.maskpoly, B.items_out, B.step);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   if (B.n_prep) {
@@ -1342,7 +1439,7 @@ cudaError_t launch_batch_forward(const DevCtx& ctx, const BatchDev& B, cudaStrea
   if (B.n_out) {
     e = ntt_multi<ModeDecrypt, true>(ctx, B.decrypt, B.items_out, B.n_out, B.step, s);
     if (e != cudaSuccess) return e;
-    k_combine_multi<<<blocks_for(B.n_out * n, 256), 256, 0, s>>>(ctx, B.combine, B.items_out, B.n_out);
+    k_combine_multi<<<blocks_for(B.n_out * n, 256), 256, 0, s>>>(ctx, B.combine, B.items_out);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   k_step_advance<<<1, 1, 0, s>>>(B.step);
