@@ -953,20 +953,30 @@ cudaError_t launch_mo_share(u64 seed, long long count, u64 t_mask, const u64* bi
 // y_j = x_j * (q/q_j)^{-1} mod q_j (first half), then crt_add / crt_round.
 // c0c (compact send form, else null): c0 at the output coefficients in
 // coefficient form, [L][out_elems]; added as c0c * qtil to the INTT(c1 s) residues.
-__device__ __forceinline__ void decrypt_combine_one(const DevCtx& ctx, const Packing& pk, const Window& win,
-                                                    const u64* yres, int ct, int e, int check, u64* y1,
-                                                    const u64* c0c = nullptr, long long out_elems = 0) {
-  const int n = ctx.n;
-  const i64 flat = win.index(pk, e);
-  if (flat < 0) return;
-  CrtSum sum{0, 0};
-  for (int j = 0; j < ctx.L; ++j) {
+// Thread = coefficients e, e + 1 (e even) of output polynomial ct; a CTA stays inside
+// one polynomial.
+__device__ __forceinline__ void decrypt_combine_pair(const DevCtx& ctx, const Packing& pk, const Window& win,
+                                                     const u64* yres, int ct, int e, int check, u64* y1,
+                                                     const u64* c0c = nullptr, long long out_elems = 0) {
+  const i64 f0 = win.index(pk, e), f1 = win.index(pk, e + 1);
+  if (f0 < 0 && f1 < 0) return;
+  CrtSum s0{0, 0}, s1{0, 0};
+  const u64* y = yres + (((size_t)ct * ctx.L) << ctx.log_n) + e;
+#pragma unroll
+  for (int j = 0; j < PENCIL_MAX_LIMBS; ++j) {
+    if (j >= ctx.L) break;
     const LimbConst& lc = ctx.limb[j];
-    u64 y = __ldg(yres + ((size_t)ct * ctx.L + j) * n + e);
-    if (c0c) y = add_mod(y, mul_shoup(__ldg(c0c + (size_t)j * out_elems + flat), lc.qtil, lc.qtils, lc.q), lc.q);
-    crt_add(sum, y, lc);
+    ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2*>(y + ((size_t)j << ctx.log_n)));
+    if (c0c) {
+      const u64* c = c0c + (size_t)j * out_elems;
+      if (f0 >= 0) v.x = add_mod(v.x, mul_shoup(__ldg(c + f0), lc.qtil, lc.qtils, lc.q), lc.q);
+      if (f1 >= 0) v.y = add_mod(v.y, mul_shoup(__ldg(c + f1), lc.qtil, lc.qtils, lc.q), lc.q);
+    }
+    crt_add(s0, v.x, lc);
+    crt_add(s1, v.y, lc);
   }
-  y1[flat] = crt_round(sum, ctx.t_mask, check, ctx.status);
+  if (f0 >= 0) y1[f0] = crt_round(s0, ctx.t_mask, check, ctx.status);
+  if (f1 >= 0) y1[f1] = crt_round(s1, ctx.t_mask, check, ctx.status);
 }
 
 __global__ void __launch_bounds__(256) k_decrypt_combine(const __grid_constant__ DevCtx ctx,
@@ -974,9 +984,9 @@ __global__ void __launch_bounds__(256) k_decrypt_combine(const __grid_constant__
                                                          const __grid_constant__ Accessor ac, const u64* yres,
                                                          int first, int check, u64* y1, const u64* c0c,
                                                          long long out_elems) {
-  const int lg = ctx.log_n - 8, ct = first + (int)(blockIdx.x >> lg);
-  const int e = ((int)(blockIdx.x & ((1u << lg) - 1u)) << 8) + threadIdx.x;
-  decrypt_combine_one(ctx, pk, Window(pk, ac, ct, nullptr), yres, ct, e, check, y1, c0c, out_elems);
+  const int lg = ctx.log_n - 9, ct = first + (int)(blockIdx.x >> lg);
+  const int e = ((int)(blockIdx.x & ((1u << lg) - 1u)) << 9) + 2 * (int)threadIdx.x;
+  decrypt_combine_pair(ctx, pk, Window(pk, ac, ct, nullptr), yres, ct, e, check, y1, c0c, out_elems);
 }
 
 cudaError_t launch_decrypt_combine(const DevCtx& ctx, const Packing& pk, const Accessor& ac, const u64* yres,
@@ -984,7 +994,7 @@ cudaError_t launch_decrypt_combine(const DevCtx& ctx, const Packing& pk, const A
                                    long long out_elems) {
   const long long total = (long long)count * ctx.n;
   if (total == 0) return cudaSuccess;
-  k_decrypt_combine<<<(unsigned)(total / 256), 256, 0, s>>>(ctx, pk, ac, yres, first, check, y1, c0c, out_elems);
+  k_decrypt_combine<<<(unsigned)(total / 512), 256, 0, s>>>(ctx, pk, ac, yres, first, check, y1, c0c, out_elems);
   return cudaGetLastError();
 }
 
@@ -1270,11 +1280,11 @@ __global__ void k_mo_share_multi(const MoShareP* __restrict__ Ps, const int2* __
 __global__ void __launch_bounds__(256) k_combine_multi(const __grid_constant__ DevCtx ctx,
                                                        const CombineP* __restrict__ Ps,
                                                        const int2* __restrict__ items) {
-  const int lg = ctx.log_n - 8;
+  const int lg = ctx.log_n - 9;
   const int2 it = items[blockIdx.x >> lg];
-  const int e = ((int)(blockIdx.x & ((1u << lg) - 1u)) << 8) + threadIdx.x;
+  const int e = ((int)(blockIdx.x & ((1u << lg) - 1u)) << 9) + 2 * (int)threadIdx.x;
   const CombineP& P = Ps[it.x];
-  decrypt_combine_one(ctx, P.pk, Window(P.pk, P.ac, it.y, nullptr), P.yres, it.y, e, 1, P.y1);
+  decrypt_combine_pair(ctx, P.pk, Window(P.pk, P.ac, it.y, nullptr), P.yres, it.y, e, 1, P.y1);
 }
 
 // ready[l] = step + 1 for every layer except one the host asked to withhold
@@ -1439,7 +1449,7 @@ cudaError_t launch_batch_forward(const DevCtx& ctx, const BatchDev& B, cudaStrea
   if (B.n_out) {
     e = ntt_multi<ModeDecrypt, true>(ctx, B.decrypt, B.items_out, B.n_out, B.step, s);
     if (e != cudaSuccess) return e;
-    k_combine_multi<<<blocks_for(B.n_out * n, 256), 256, 0, s>>>(ctx, B.combine, B.items_out);
+    k_combine_multi<<<blocks_for(B.n_out * n, 512), 256, 0, s>>>(ctx, B.combine, B.items_out);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   k_step_advance<<<1, 1, 0, s>>>(B.step);

@@ -29,14 +29,6 @@ namespace pencil {
 // decryption (the CRT factor folded in).
 enum class InvScale { kNinv, kNqtil };
 
-// Inverse modes whose store writes shared memory (the run then synchronises the
-// CTA before its stores) and that finish with a step across the L limb CTAs of
-// one polynomial, launched as a thread-block cluster (1, L, 1).
-template <class M, class = void>
-struct ClusterLimbs : std::false_type {};
-template <class M>
-struct ClusterLimbs<M, std::void_t<decltype(M::kClusterLimbs)>> : std::bool_constant<M::kClusterLimbs> {};
-
 // Shared-memory slot of coefficient x: the low four index bits are XOR-ed with
 // (bits 4..7) ^ (bits 5..8).  8-byte accesses are served per half-warp (16
 // threads over the 16 bank pairs); with this swizzle every round's strided
@@ -229,7 +221,6 @@ __device__ __forceinline__ void ntt_inv_run(const DevCtx& ctx, const typename Mo
   __syncthreads();
   InvRounds<LOGN, C::LOGE, C::LAST_S0>::run(v, sm, tw, tau, q, q2);
   // v in [0, 2q); scaled here by the mode's kappa (N^{-1}, possibly with its own constant folded in)
-  if constexpr (ClusterLimbs<Mode>::value) __syncthreads();   // the last round's reads are done
   const bool ninv = Mode::kInvScale == InvScale::kNinv;
   const u64 kap = ninv ? lc.ninv : lc.nqtil, kaps = ninv ? lc.ninvs : lc.nqtils;
 #pragma unroll
@@ -329,14 +320,14 @@ struct FRound {
   }
   // Stage J of the round (global stage S0 + J), forward.
   template <int J>
-  static __device__ __forceinline__ void fwd_stage(u64 (&v)[E], const uint4* __restrict__ tw, int tau, const FoldC& f) {
+  static __device__ __forceinline__ void fwd_stage(u64 (&v)[E], const uint4* __restrict__ tw, int tau, const FoldC& f, int root) {
     constexpr int half = 1 << (K - 1 - J);
 #pragma unroll
     for (int gg = 0; gg < G; ++gg) {
       const int B = grp(tau, gg) >> LOGD;
 #pragma unroll
       for (int i = 0; i < (1 << J); ++i) {
-        const uint4 w = __ldg(tw + (1 << (S0 + J)) + (B << J) + i);
+        const uint4 w = __ldg(tw + (root << (S0 + J)) + (B << J) + i);
 #pragma unroll
         for (int r = 0; r < half; ++r) {
           const int l = gg * (1 << K) + i * 2 * half + r;
@@ -352,7 +343,7 @@ struct FRound {
   // Stage J of the round, inverse; the stages at odd positions of the inverse order
   // (LOGN - 1 - (S0 + J)) fold their sums.
   template <int J>
-  static __device__ __forceinline__ void inv_stage(u64 (&v)[E], const uint4* __restrict__ tw, int tau, const FoldC& f) {
+  static __device__ __forceinline__ void inv_stage(u64 (&v)[E], const uint4* __restrict__ tw, int tau, const FoldC& f, int root) {
     constexpr int half = 1 << (K - 1 - J);
     constexpr bool odd = ((LOGN - 1 - (S0 + J)) & 1) != 0;
 #pragma unroll
@@ -360,7 +351,7 @@ struct FRound {
       const int B = grp(tau, gg) >> LOGD;
 #pragma unroll
       for (int i = 0; i < (1 << J); ++i) {
-        const uint4 w = __ldg(tw + (1 << (S0 + J)) + (B << J) + i);
+        const uint4 w = __ldg(tw + (root << (S0 + J)) + (B << J) + i);
 #pragma unroll
         for (int r = 0; r < half; ++r) {
           const int l = gg * (1 << K) + i * 2 * half + r;
@@ -372,8 +363,8 @@ struct FRound {
   }
   template <int... J>
   static __device__ __forceinline__ void fwd_seq(std::integer_sequence<int, J...>, u64 (&v)[E],
-                                                 const uint4* tw, int tau, const FoldC& f) {
-    (fwd_stage<J>(v, tw, tau, f), ...);
+                                                 const uint4* tw, int tau, const FoldC& f, int root) {
+    (fwd_stage<J>(v, tw, tau, f, root), ...);
   }
   // Round 0 of the inverse with the transform's final scaling kappa merged into
   // its last stage (global stage 0, whose butterflies all use w1 = tw[1]):
@@ -395,23 +386,23 @@ struct FRound {
   // Stages K - 1 .. 0 (inverse order), or K - 1 .. 1 with sizeof...(J) = K - 1.
   template <int... J>
   static __device__ __forceinline__ void inv_seq(std::integer_sequence<int, J...>, u64 (&v)[E],
-                                                 const uint4* tw, int tau, const FoldC& f, int = 0) {
-    (inv_stage<K - 1 - J>(v, tw, tau, f), ...);
+                                                 const uint4* tw, int tau, const FoldC& f, int root) {
+    (inv_stage<K - 1 - J>(v, tw, tau, f, root), ...);
   }
-  static __device__ __forceinline__ void fwd(u64 (&v)[E], const uint4* tw, int tau, const FoldC& f) {
-    fwd_seq(std::make_integer_sequence<int, K>{}, v, tw, tau, f);
+  static __device__ __forceinline__ void fwd(u64 (&v)[E], const uint4* tw, int tau, const FoldC& f, int root) {
+    fwd_seq(std::make_integer_sequence<int, K>{}, v, tw, tau, f, root);
   }
   // Stages j0 .. K - 1 only (j0 uniform across the CTA).
   template <int... J>
   static __device__ __forceinline__ void fwd_from_seq(std::integer_sequence<int, J...>, int j0, u64 (&v)[E],
-                                                      const uint4* tw, int tau, const FoldC& f) {
-    ((J >= j0 ? fwd_stage<J>(v, tw, tau, f) : void()), ...);
+                                                      const uint4* tw, int tau, const FoldC& f, int root) {
+    ((J >= j0 ? fwd_stage<J>(v, tw, tau, f, root) : void()), ...);
   }
-  static __device__ __forceinline__ void fwd_from(int j0, u64 (&v)[E], const uint4* tw, int tau, const FoldC& f) {
-    fwd_from_seq(std::make_integer_sequence<int, K>{}, j0, v, tw, tau, f);
+  static __device__ __forceinline__ void fwd_from(int j0, u64 (&v)[E], const uint4* tw, int tau, const FoldC& f, int root) {
+    fwd_from_seq(std::make_integer_sequence<int, K>{}, j0, v, tw, tau, f, root);
   }
-  static __device__ __forceinline__ void inv(u64 (&v)[E], const uint4* tw, int tau, const FoldC& f) {
-    inv_seq(std::make_integer_sequence<int, K>{}, v, tw, tau, f);
+  static __device__ __forceinline__ void inv(u64 (&v)[E], const uint4* tw, int tau, const FoldC& f, int root) {
+    inv_seq(std::make_integer_sequence<int, K>{}, v, tw, tau, f, root);
   }
 };
 
@@ -420,35 +411,36 @@ struct FRound {
 // shared memory.  Each round folds its words and leaves them in shared memory.
 template <int LOGN, int LOGE, int S0>
 struct FFwdRounds {
-  static __device__ __forceinline__ void run(u64 (&v)[1 << LOGE], u64* sm, const uint4* tw, int tau, const FoldC& f) {
+  static __device__ __forceinline__ void run(u64 (&v)[1 << LOGE], u64* sm, const uint4* tw, int tau, const FoldC& f, int root) {
     using Rd = FRound<LOGN, LOGE, S0>;
     if constexpr (S0 > 0) Rd::load(v, sm, tau);
-    Rd::fwd(v, tw, tau, f);
+    Rd::fwd(v, tw, tau, f, root);
 #pragma unroll
     for (int l = 0; l < (1 << LOGE); ++l) v[l] = fold_s(v[l], f);
     if constexpr (S0 > 0) phase_sync<Rd::kLocal>();   // every reader of these slots is done
     Rd::store(v, sm, tau);
     phase_sync<Rd::kLocal>();   // the following rounds are warp-local once this one is
-    if constexpr (S0 + LOGE < FCfg<LOGN, LOGE>::SL) FFwdRounds<LOGN, LOGE, S0 + LOGE>::run(v, sm, tw, tau, f);
+    if constexpr (S0 + LOGE < FCfg<LOGN, LOGE>::SL) FFwdRounds<LOGN, LOGE, S0 + LOGE>::run(v, sm, tw, tau, f, root);
   }
 };
 
 // Inverse rounds from S0 down to 0 (words in shared memory on entry, synced); on
 // return v holds the coefficients tau + l T.
-template <int LOGN, int LOGE, int S0>
+template <int LOGN, int LOGE, int S0, bool SCALED = true>
 struct FInvRounds {
-  static __device__ __forceinline__ void run(u64 (&v)[1 << LOGE], u64* sm, const uint4* tw, int tau, const FoldC& f, u64 q2, const uint4* sc) {
+  static __device__ __forceinline__ void run(u64 (&v)[1 << LOGE], u64* sm, const uint4* tw, int tau, const FoldC& f,
+                                             u64 q2, const uint4* sc, int root) {
     using Rd = FRound<LOGN, LOGE, S0>;
     Rd::load(v, sm, tau);
-    if constexpr (S0 == 0)
+    if constexpr (S0 == 0 && SCALED)
       Rd::inv_scaled(v, tw, tau, f, q2, sc);
     else
-      Rd::inv(v, tw, tau, f);
+      Rd::inv(v, tw, tau, f, root);
     if constexpr (S0 > 0) {
       phase_sync<Rd::kLocal>();
       Rd::store(v, sm, tau);
       phase_sync<Rd::kLocal && FRound<LOGN, LOGE, S0 - LOGE>::kLocal>();
-      FInvRounds<LOGN, LOGE, S0 - LOGE>::run(v, sm, tw, tau, f, q2, sc);
+      FInvRounds<LOGN, LOGE, S0 - LOGE, SCALED>::run(v, sm, tw, tau, f, q2, sc, root);
     }
   }
 };
@@ -456,7 +448,8 @@ struct FInvRounds {
 // The last forward round's KL stages on one group of W = 2^KL consecutive slots
 // (group index g: positions g W .. g W + W - 1), then canonical values.
 template <int LOGN, int LOGE>
-__device__ __forceinline__ void fold_last_fwd(u64* u, const uint4* __restrict__ tw, int g, const FoldC& f, u64 q, u64 off) {
+__device__ __forceinline__ void fold_last_fwd(u64* u, const uint4* __restrict__ tw, int g, const FoldC& f, u64 q,
+                                              u64 off, int root) {
   using C = FCfg<LOGN, LOGE>;
   constexpr int W = 1 << C::KL;
 #pragma unroll
@@ -464,7 +457,7 @@ __device__ __forceinline__ void fold_last_fwd(u64* u, const uint4* __restrict__ 
     const int half = W >> (J + 1);
 #pragma unroll
     for (int i = 0; i < (1 << J); ++i) {
-      const uint4 w = __ldg(tw + (1 << (C::SL + J)) + (g << J) + i);
+      const uint4 w = __ldg(tw + (root << (C::SL + J)) + (g << J) + i);
 #pragma unroll
       for (int r = 0; r < half; ++r) ct_split(u[i * 2 * half + r], u[i * 2 * half + r + half], w, f);
     }
@@ -476,7 +469,7 @@ __device__ __forceinline__ void fold_last_fwd(u64* u, const uint4* __restrict__ 
 // The first inverse round's KL stages (inverse steps 0 .. KL - 1) on one group.
 template <int LOGN, int LOGE>
 __device__ __forceinline__ void fold_first_inv(u64 (&u)[1 << FCfg<LOGN, LOGE>::KL],
-                                               const uint4* __restrict__ tw, int g, const FoldC& f) {
+                                               const uint4* __restrict__ tw, int g, const FoldC& f, int root) {
   using C = FCfg<LOGN, LOGE>;
   constexpr int W = 1 << C::KL;
 #pragma unroll
@@ -485,7 +478,7 @@ __device__ __forceinline__ void fold_first_inv(u64 (&u)[1 << FCfg<LOGN, LOGE>::K
     const bool odd = ((LOGN - 1 - (C::SL + J)) & 1) != 0;
 #pragma unroll
     for (int i = 0; i < (1 << J); ++i) {
-      const uint4 w = __ldg(tw + (1 << (C::SL + J)) + (g << J) + i);
+      const uint4 w = __ldg(tw + (root << (C::SL + J)) + (g << J) + i);
 #pragma unroll
       for (int r = 0; r < half; ++r) {
         u64& x = u[i * 2 * half + r];
@@ -528,13 +521,83 @@ __device__ __forceinline__ void fold_sparse_head(const DevCtx& ctx, const typena
   const u64* b = sm + ph(tau & (D1 - 1));
 #pragma unroll
   for (int l = 0; l < C::E; ++l) v[l] = b[ph(D1 * (l & m))];
-  R1::fwd_from(j, v, tw, tau, f);
+  R1::fwd_from(j, v, tw, tau, f, 1);
 #pragma unroll
   for (int l = 0; l < C::E; ++l) v[l] = fold_s(v[l], f);
   __syncthreads();   // every thread has read the prologue values
   R1::store(v, sm, tau);
   phase_sync<R1::kLocal>();
-  if constexpr (2 * LOGE < C::SL) FFwdRounds<LOGN, LOGE, 2 * LOGE>::run(v, sm, tw, tau, f);
+  if constexpr (2 * LOGE < C::SL) FFwdRounds<LOGN, LOGE, 2 * LOGE>::run(v, sm, tw, tau, f, 1);
+}
+
+// Last round and epilogue of a (sub)transform of 2^LOGN words whose slots are e0, e0 + 1,
+// ... of a polynomial of 2^LOGP.
+template <int LOGN, int LOGE, int LOGP, class Mode>
+__device__ __forceinline__ void fold_tail(const DevCtx& ctx, const typename Mode::Params& P, const LimbConst& lc,
+                                          int poly, int limb, u64 (&v)[1 << LOGE], u64* sm, const uint4* tw, int tau,
+                                          const FoldC& f, int root, int e0) {
+  using C = FCfg<LOGN, LOGE>;
+  constexpr int NFULL = 1 << LOGP;
+  const u64 q = lc.q;
+  if constexpr (C::FUSE) {
+    // groups of GW consecutive slots per iteration: the last round's groups of
+    // W = 2^KL, gathered in fours for modes that store four coefficients at a time
+    constexpr int W = 1 << C::KL;
+    constexpr int GW = (Mode::kQuad && W < 4) ? 4 : W;
+    // group k = 32 (E / GW) w + 32 j + lane: warp w's own positions [32 E w, 32 E (w + 1))
+    const int kbase = (tau >> 5) * (32 * C::E / GW) + (tau & 31);
+#pragma unroll(Mode::kEpilogueUnroll)
+    for (int j = 0; j < C::E / GW; ++j) {
+      const int k = kbase + 32 * j;
+      u64 u[GW];
+      const ulonglong2* b = reinterpret_cast<const ulonglong2*>(sm + ph(k * GW));
+#pragma unroll
+      for (int i = 0; i < GW / 2; ++i) {
+        const ulonglong2 x = b[i];
+        u[2 * i] = x.x;
+        u[2 * i + 1] = x.y;
+      }
+#pragma unroll
+      for (int s = 0; s < GW / W; ++s) fold_last_fwd<LOGN, LOGE>(u + s * W, tw, k * (GW / W) + s, f, q, 4 * q, root);
+      if constexpr (Mode::kQuad) {
+#pragma unroll
+        for (int i = 0; i < GW / 4; ++i) Mode::template store4<NFULL, true>(ctx, P, lc, poly, limb, e0 + k * GW + 4 * i, u + 4 * i);
+      } else {
+#pragma unroll
+        for (int i = 0; i < GW / 2; ++i)
+          Mode::template store2<NFULL, true>(ctx, P, lc, poly, limb, e0 + k * GW + 2 * i, u[2 * i], u[2 * i + 1]);
+      }
+    }
+  } else {
+    using Rd = FRound<LOGN, LOGE, C::SL>;
+    Rd::load(v, sm, tau);
+    Rd::fwd(v, tw, tau, f, root);
+#pragma unroll
+    for (int l = 0; l < C::E; ++l) v[l] = csub(fold_u(v[l] + 8 * q, f), q);
+    static_assert(Rd::kLocal, "the last round is warp-local");
+    __syncwarp();
+    Rd::store(v, sm, tau);
+    __syncwarp();
+    // the epilogue's groups are warp w's own positions [32 E w, 32 E (w + 1))
+    const int wbase = (tau >> 5) * 32 * C::E, lane = tau & 31;
+    if constexpr (Mode::kQuad) {
+#pragma unroll(Mode::kEpilogueUnroll)
+      for (int l = 0; l < C::E / 4; ++l) {
+        const int e = wbase + 4 * (lane + 32 * l);
+        const ulonglong2* b = reinterpret_cast<const ulonglong2*>(sm + ph(e));
+        const ulonglong2 x01 = b[0], x23 = b[1];
+        u64 x[4] = {x01.x, x01.y, x23.x, x23.y};
+        Mode::template store4<NFULL, true>(ctx, P, lc, poly, limb, e0 + e, x);
+      }
+    } else {
+#pragma unroll(Mode::kEpilogueUnroll)
+      for (int l = 0; l < C::E / 2; ++l) {
+        const int e = wbase + 2 * (lane + 32 * l);
+        const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(sm + ph(e));
+        Mode::template store2<NFULL, true>(ctx, P, lc, poly, limb, e0 + e, x.x, x.y);
+      }
+    }
+  }
 }
 
 template <int LOGN, int LOGE, class Mode>
@@ -544,7 +607,6 @@ __device__ __forceinline__ void ntt_fwd_run_fold(const DevCtx& ctx, const typena
   const int tau = threadIdx.x;
   const LimbConst& lc = ctx.limb[limb];
   const typename Mode::Pre pre(ctx, P, poly);
-  const u64 q = lc.q;
   const FoldC f(lc);
   const uint4* tw = ctx.tw_fwd_f + (size_t)limb * C::N;
   u64 v[C::E];
@@ -570,81 +632,20 @@ __device__ __forceinline__ void ntt_fwd_run_fold(const DevCtx& ctx, const typena
       for (int l = 0; l < C::E; ++l) v[l] = Mode::template load<C::N, true>(ctx, P, pre, lc, poly, limb, tau + l * C::T);
     }
     // (round 0 stores each thread's words at the slots it read them from: no barrier needed here)
-    FFwdRounds<LOGN, LOGE, 0>::run(v, sm, tw, tau, f);
+    FFwdRounds<LOGN, LOGE, 0>::run(v, sm, tw, tau, f, 1);
   }
-  if constexpr (C::FUSE) {
-    // groups of GW consecutive slots per iteration: the last round's groups of
-    // W = 2^KL, gathered in fours for modes that store four coefficients at a time
-    constexpr int W = 1 << C::KL;
-    constexpr int GW = (Mode::kQuad && W < 4) ? 4 : W;
-    // group k = 32 (E / GW) w + 32 j + lane: warp w's own positions [32 E w, 32 E (w + 1))
-    const int kbase = (tau >> 5) * (32 * C::E / GW) + (tau & 31);
-#pragma unroll(Mode::kEpilogueUnroll)
-    for (int j = 0; j < C::E / GW; ++j) {
-      const int k = kbase + 32 * j;
-      u64 u[GW];
-      const ulonglong2* b = reinterpret_cast<const ulonglong2*>(sm + ph(k * GW));
-#pragma unroll
-      for (int i = 0; i < GW / 2; ++i) {
-        const ulonglong2 x = b[i];
-        u[2 * i] = x.x;
-        u[2 * i + 1] = x.y;
-      }
-#pragma unroll
-      for (int s = 0; s < GW / W; ++s) fold_last_fwd<LOGN, LOGE>(u + s * W, tw, k * (GW / W) + s, f, q, 4 * q);
-      if constexpr (Mode::kQuad) {
-#pragma unroll
-        for (int i = 0; i < GW / 4; ++i) Mode::template store4<C::N, true>(ctx, P, lc, poly, limb, k * GW + 4 * i, u + 4 * i);
-      } else {
-#pragma unroll
-        for (int i = 0; i < GW / 2; ++i)
-          Mode::template store2<C::N, true>(ctx, P, lc, poly, limb, k * GW + 2 * i, u[2 * i], u[2 * i + 1]);
-      }
-    }
-  } else {
-    using Rd = FRound<LOGN, LOGE, C::SL>;
-    Rd::load(v, sm, tau);
-    Rd::fwd(v, tw, tau, f);
-#pragma unroll
-    for (int l = 0; l < C::E; ++l) v[l] = csub(fold_u(v[l] + 8 * q, f), q);
-    static_assert(Rd::kLocal, "the last round is warp-local");
-    __syncwarp();
-    Rd::store(v, sm, tau);
-    __syncwarp();
-    // the epilogue's groups are warp w's own positions [32 E w, 32 E (w + 1))
-    const int wbase = (tau >> 5) * 32 * C::E, lane = tau & 31;
-    if constexpr (Mode::kQuad) {
-#pragma unroll(Mode::kEpilogueUnroll)
-      for (int l = 0; l < C::E / 4; ++l) {
-        const int e = wbase + 4 * (lane + 32 * l);
-        const ulonglong2* b = reinterpret_cast<const ulonglong2*>(sm + ph(e));
-        const ulonglong2 x01 = b[0], x23 = b[1];
-        u64 x[4] = {x01.x, x01.y, x23.x, x23.y};
-        Mode::template store4<C::N, true>(ctx, P, lc, poly, limb, e, x);
-      }
-    } else {
-#pragma unroll(Mode::kEpilogueUnroll)
-      for (int l = 0; l < C::E / 2; ++l) {
-        const int e = wbase + 2 * (lane + 32 * l);
-        const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(sm + ph(e));
-        Mode::template store2<C::N, true>(ctx, P, lc, poly, limb, e, x.x, x.y);
-      }
-    }
-  }
+  fold_tail<LOGN, LOGE, LOGN, Mode>(ctx, P, lc, poly, limb, v, sm, tw, tau, f, 1, 0);
 }
 
-template <int LOGN, int LOGE, class Mode>
-__device__ __forceinline__ void ntt_inv_run_fold(const DevCtx& ctx, const typename Mode::Params& P, int poly,
-                                                 int limb, u64* sm) {
+// Prologue and rounds of an inverse (sub)transform of 2^LOGN words (slots e0, e0 + 1, ...
+// of a polynomial of 2^LOGP); on return v holds the coefficients tau + l T.
+template <int LOGN, int LOGE, int LOGP, class Mode, bool SCALED>
+__device__ __forceinline__ void fold_inv_rounds(const DevCtx& ctx, const typename Mode::Params& P,
+                                                const typename Mode::Pre& pre, const LimbConst& lc, int poly, int limb,
+                                                u64 (&v)[1 << LOGE], u64* sm, const uint4* tw, int tau, const FoldC& f,
+                                                u64 q2, const uint4* sc, int root, int e0) {
   using C = FCfg<LOGN, LOGE>;
-  const int tau = threadIdx.x;
-  const LimbConst& lc = ctx.limb[limb];
-  const typename Mode::Pre pre(ctx, P, poly);
-  const u64 q = lc.q, q2 = 2 * q;
-  const FoldC f(lc);
-  const uint4* tw = ctx.tw_inv_f + (size_t)limb * C::N;
-  const uint4* sc = Mode::kInvScale == InvScale::kNinv ? lc.sc_ninv : lc.sc_nqtil;
-  u64 v[C::E];
+  constexpr int NFULL = 1 << LOGP;
   if constexpr (C::FUSE) {
     constexpr int W = 1 << C::KL;
     // group g = 32 (E / W) w + 32 j + lane: warp w's own positions [32 E w, 32 E (w + 1))
@@ -654,15 +655,16 @@ __device__ __forceinline__ void ntt_inv_run_fold(const DevCtx& ctx, const typena
       const int g = gbase + 32 * j;
       u64 u[W];
 #pragma unroll
-      for (int i = 0; i < W; ++i) u[i] = Mode::template load<C::N, true>(ctx, P, pre, lc, poly, limb, g * W + i);
-      fold_first_inv<LOGN, LOGE>(u, tw, g, f);
+      for (int i = 0; i < W; i += 2)
+        Mode::template load2<NFULL>(ctx, P, lc, poly, limb, e0 + g * W + i, u[i], u[i + 1]);
+      fold_first_inv<LOGN, LOGE>(u, tw, g, f, root);
       ulonglong2* b = reinterpret_cast<ulonglong2*>(sm + ph(g * W));
 #pragma unroll
       for (int i = 0; i < W / 2; ++i) b[i] = make_ulonglong2(u[2 * i], u[2 * i + 1]);
     }
     if constexpr (C::SL > 0) {
       phase_sync<FRound<LOGN, LOGE, C::SL - LOGE>::kLocal>();
-      FInvRounds<LOGN, LOGE, C::SL - LOGE>::run(v, sm, tw, tau, f, q2, sc);
+      FInvRounds<LOGN, LOGE, C::SL - LOGE, SCALED>::run(v, sm, tw, tau, f, q2, sc, root);
     } else {
       __syncthreads();
     }
@@ -673,17 +675,135 @@ __device__ __forceinline__ void ntt_inv_run_fold(const DevCtx& ctx, const typena
 #pragma unroll(Mode::kLoadUnroll)
     for (int l = 0; l < C::E; ++l) {
       const int e = wbase + 32 * l;
-      sm[ph(e)] = Mode::template load<C::N, true>(ctx, P, pre, lc, poly, limb, e);
+      sm[ph(e)] = Mode::template load<NFULL, true>(ctx, P, pre, lc, poly, limb, e0 + e);
     }
     static_assert(FRound<LOGN, LOGE, C::SL>::kLocal, "the last round is warp-local");
     __syncwarp();
-    FInvRounds<LOGN, LOGE, C::SL>::run(v, sm, tw, tau, f, q2, sc);
+    FInvRounds<LOGN, LOGE, C::SL, SCALED>::run(v, sm, tw, tau, f, q2, sc, root);
   }
+}
+
+template <int LOGN, int LOGE, class Mode>
+__device__ __forceinline__ void ntt_inv_run_fold(const DevCtx& ctx, const typename Mode::Params& P, int poly,
+                                                 int limb, u64* sm) {
+  using C = FCfg<LOGN, LOGE>;
+  const int tau = threadIdx.x;
+  const LimbConst& lc = ctx.limb[limb];
+  const typename Mode::Pre pre(ctx, P, poly);
+  const u64 q = lc.q;
+  const FoldC f(lc);
+  const uint4* tw = ctx.tw_inv_f + (size_t)limb * C::N;
+  const uint4* sc = Mode::kInvScale == InvScale::kNinv ? lc.sc_ninv : lc.sc_nqtil;
+  u64 v[C::E];
+  fold_inv_rounds<LOGN, LOGE, LOGN, Mode, true>(ctx, P, pre, lc, poly, limb, v, sm, tw, tau, f, 2 * q, sc, 1, 0);
   // v in (0.9 q, 4.1 q), already scaled by the mode's kappa in the last stage
-  if constexpr (ClusterLimbs<Mode>::value) __syncthreads();   // the last round's reads are done
 #pragma unroll
   for (int l = 0; l < C::E; ++l)
     Mode::template store<C::N>(ctx, P, lc, poly, limb, tau + l * C::T, csub(fold_u(v[l], f), q));
+}
+
+// One transform on a cluster of four CTAs, for launches too small to fill the GPU: after
+// two Cooley-Tukey stages block r of N / 4 words is a transform of its own, with the
+// twiddles of the subtree under node 4 + r.  CTA r evaluates the prologue of the r-th
+// quarter of the coefficients into its shared memory, combines the four quarters for its
+// block (three products a word, reading the others' through distributed shared memory)
+// and transforms the block alone; the inverse runs its block's stages first and then the
+// last two on a quarter of the block positions.  Radix 2^3: N / 32 threads a CTA, so a
+// lone transform runs on 4 SMs with a quarter of the words each.
+template <int LOGN>
+struct Quad {
+  static constexpr int LOGM = LOGN - 2, LOGE = 3, M = 1 << LOGM;
+  using C = FCfg<LOGM, LOGE>;
+};
+
+template <int LOGN, class Mode>
+__device__ __forceinline__ void quad_fwd(const DevCtx& ctx, const typename Mode::Params& P, int poly, int limb,
+                                         u64* sm) {
+  namespace cg = cooperative_groups;
+  using Q = Quad<LOGN>;
+  using C = typename Q::C;
+  cg::cluster_group cl = cg::this_cluster();
+  const int tau = threadIdx.x, rank = (int)cl.block_rank(), root = 4 + rank;
+  const LimbConst& lc = ctx.limb[limb];
+  const typename Mode::Pre pre(ctx, P, poly);
+  const FoldC f(lc);
+  const uint4* tw = ctx.tw_fwd_f + (size_t)limb * (1 << LOGN);
+  u64 v[C::E];
+  bool copied = false;
+  if constexpr (SparseInput<Mode>::value) {
+    const int sup = Mode::support(P);
+    if (sup <= Q::M) {   // the first two stages only copy: every block starts from the same words
+      copied = true;
+#pragma unroll
+      for (int l = 0; l < C::E; ++l) {
+        const int p = tau + l * C::T;
+        v[l] = p < sup ? Mode::template load<1 << LOGN, true>(ctx, P, pre, lc, poly, limb, p) : 0ull;
+      }
+    }
+  }
+  if (!copied) {
+#pragma unroll
+    for (int l = 0; l < C::E; ++l) {
+      const int p = tau + l * C::T;
+      sm[ph(p)] = Mode::template load<1 << LOGN, true>(ctx, P, pre, lc, poly, limb, rank * Q::M + p);
+    }
+    const uint4 w1 = __ldg(tw + 1), w2 = __ldg(tw + 2 + (rank >> 1));
+    const u64* x[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) x[k] = cl.map_shared_rank(sm, k);
+    cl.sync();
+#pragma unroll
+    for (int l = 0; l < C::E; ++l) {
+      const int at = ph(tau + l * C::T);
+      const u64 a = mul_split(0, x[2][at], w1, f), b = mul_split(0, x[3][at], w1, f);
+      const u64 c = rank & 2 ? x[0][at] - a : x[0][at] + a, d = rank & 2 ? x[1][at] - b : x[1][at] + b;
+      const u64 t = mul_split(0, d, w2, f);
+      v[l] = fold_s(rank & 1 ? c - t : c + t, f);
+    }
+    cl.sync();   // every quarter has been read: the rounds may write shared memory
+  }
+  FFwdRounds<Q::LOGM, Q::LOGE, 0>::run(v, sm, tw, tau, f, root);
+  fold_tail<Q::LOGM, Q::LOGE, LOGN, Mode>(ctx, P, lc, poly, limb, v, sm, tw, tau, f, root, rank * Q::M);
+}
+
+template <int LOGN, class Mode>
+__device__ __forceinline__ void quad_inv(const DevCtx& ctx, const typename Mode::Params& P, int poly, int limb,
+                                         u64* sm) {
+  namespace cg = cooperative_groups;
+  using Q = Quad<LOGN>;
+  using C = typename Q::C;
+  cg::cluster_group cl = cg::this_cluster();
+  const int tau = threadIdx.x, rank = (int)cl.block_rank(), root = 4 + rank;
+  const LimbConst& lc = ctx.limb[limb];
+  const typename Mode::Pre pre(ctx, P, poly);
+  const u64 q = lc.q;
+  const FoldC f(lc);
+  const uint4* tw = ctx.tw_inv_f + (size_t)limb * (1 << LOGN);
+  const uint4* sc = Mode::kInvScale == InvScale::kNinv ? lc.sc_ninv : lc.sc_nqtil;
+  u64 v[C::E];
+  fold_inv_rounds<Q::LOGM, Q::LOGE, LOGN, Mode, false>(ctx, P, pre, lc, poly, limb, v, sm, tw, tau, f, 2 * q, sc, root,
+                                                       rank * Q::M);
+  __syncthreads();   // the last round's reads are done
+#pragma unroll
+  for (int l = 0; l < C::E; ++l) sm[ph(tau + l * C::T)] = fold_s(v[l], f);
+  const uint4 w2 = __ldg(tw + 2), w3 = __ldg(tw + 3), k = sc[0], wk = sc[1];
+  const u64* y[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) y[i] = cl.map_shared_rank(sm, i);
+  cl.sync();
+#pragma unroll
+  for (int l = 0; l < C::E / 4; ++l) {
+    const int p = rank * (Q::M / 4) + tau + l * C::T, at = ph(p);
+    const u64 y0 = y[0][at], y1 = y[1][at], y2 = y[2][at], y3 = y[3][at];
+    const u64 a0 = y0 + y1, a1 = mul_split(0, y0 - y1, w2, f);
+    const u64 a2 = y2 + y3, a3 = mul_split(0, y2 - y3, w3, f);
+    const u64 x[4] = {mul_split(2 * q, a0 + a2, k, f), mul_split(2 * q, a1 + a3, k, f),
+                      mul_split(2 * q, a0 - a2, wk, f), mul_split(2 * q, a1 - a3, wk, f)};
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      Mode::template store<1 << LOGN>(ctx, P, lc, poly, limb, p + i * Q::M, csub(fold_u(x[i], f), q));
+  }
+  cl.sync();   // the other CTAs have finished reading this one's shared memory
 }
 
 // Launch shape of either engine.
@@ -746,7 +866,18 @@ __global__ void __launch_bounds__(KCfg<LOGN, LOGE, FOLD>::T, KCfg<LOGN, LOGE, FO
   extern __shared__ __align__(16) u64 sm[];
   prefetch_ahead<1 << LOGN, Mode>(ctx, P, first);
   inv_any<LOGN, LOGE, Mode, FOLD>(ctx, P, first + (int)blockIdx.x, blockIdx.y, sm);
-  if constexpr (ClusterLimbs<Mode>::value) Mode::template finish<1 << LOGN>(ctx, P, first + (int)blockIdx.x, sm);
+}
+
+// Cluster (x / 4, limb) of four CTAs transforms polynomial first + x / 4.
+template <int LOGN, class Mode, bool INV>
+__global__ void __launch_bounds__((1 << LOGN) / 32) k_ntt_quad(const __grid_constant__ DevCtx ctx,
+                                                               const __grid_constant__ typename Mode::Params P,
+                                                               int first) {
+  extern __shared__ __align__(16) u64 sm[];
+  if constexpr (INV)
+    quad_inv<LOGN, Mode>(ctx, P, first + (int)(blockIdx.x >> 2), blockIdx.y, sm);
+  else
+    quad_fwd<LOGN, Mode>(ctx, P, first + (int)(blockIdx.x >> 2), blockIdx.y, sm);
 }
 
 // Multi-plan variants: CTA (blockIdx.x, limb) transforms polynomial items[x].y
@@ -810,6 +941,14 @@ struct ModeRaw {
   };
   using Pre = NoPre;
   static __device__ __forceinline__ void rebase(Params&, u64) {}
+  // two consecutive slots of an inverse transform (split engine)
+  template <int N>
+  static __device__ __forceinline__ void load2(const DevCtx& c, const Params& P, const LimbConst&, int poly, int limb,
+                                               int e, u64& x0, u64& x1) {
+    const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(P.polys + limb_off(poly, limb, c.L, N) + e);
+    x0 = x.x;
+    x1 = x.y;
+  }
   template <int N, bool SPLIT>
   static __device__ __forceinline__ u64 load(const DevCtx& c, const Params& P, const Pre& pre, const LimbConst&, int poly, int limb,
                                              int e) {
@@ -1173,6 +1312,22 @@ struct ModeDecrypt {
   };
   using Pre = NoPre;
   static __device__ __forceinline__ void rebase(Params&, u64) {}
+  template <int N>
+  static __device__ __forceinline__ void load2(const DevCtx& c, const Params& P, const LimbConst& lc, int poly,
+                                               int limb, int e, u64& x0, u64& x1) {
+    const FoldC f(lc);
+    const ulonglong2 c1 = __ldg(reinterpret_cast<const ulonglong2*>(P.ct + ct_off(poly, 1, limb, c.L, N) + e));
+    const uint4* key = reinterpret_cast<const uint4*>(P.sk) + (size_t)(c.L + limb) * N + e;
+    const uint4 s0 = __ldg(key), s1 = __ldg(key + 1);
+    if (P.skip_c0) {
+      x0 = mul_split(0, c1.x, s0, f);
+      x1 = mul_split(0, c1.y, s1, f);
+    } else {
+      const ulonglong2 c0 = __ldg(reinterpret_cast<const ulonglong2*>(P.ct + ct_off(poly, 0, limb, c.L, N) + e));
+      x0 = fold_s(mul_split(c0.x, c1.x, s0, f), f);
+      x1 = fold_s(mul_split(c0.y, c1.y, s1, f), f);
+    }
+  }
   template <int N, bool SPLIT>
   static __device__ __forceinline__ u64 load(const DevCtx& c, const Params& P, const Pre& pre, const LimbConst& lc, int poly,
                                              int limb, int e) {
@@ -1195,74 +1350,6 @@ struct ModeDecrypt {
   }
 };
 
-// DO decryption with the CRT step fused (launched as one cluster of the L limb
-// CTAs per ciphertext): each CTA leaves its residues y_j = N^{-1} qtil INTT(c0 +
-// c1 s) in its own shared memory (word e at slot e); after a cluster barrier CTA j
-// takes coefficient pairs j T + tau + i L T, reads the L residues of each through
-// distributed shared memory and writes round(t x / q) mod t to the output
-// element the coefficient carries; a second barrier keeps every CTA's shared
-// memory alive until the others have read it.  Saves the [count][L][N] residue
-// array's write and read and a launch.
-struct ModeDecryptFused {
-  static constexpr InvScale kInvScale = InvScale::kNqtil;
-  static constexpr bool kHeavyLoad = true;
-  static constexpr bool kQuad = false;
-  static constexpr bool kClusterLimbs = true;
-  static constexpr int kLoadUnroll = 8;
-  static constexpr int kEpilogueUnroll = 16;
-  struct Params {
-    ModeDecrypt::Params d;   // d.out unused
-    Packing pk;              // output packing
-    Accessor ac;             // output layout
-    u64* y1;
-    int check;
-  };
-  using Pre = NoPre;
-  static __device__ __forceinline__ void rebase(Params&, u64) {}
-  template <int N, bool SPLIT>
-  static __device__ __forceinline__ u64 load(const DevCtx& c, const Params& P, const Pre& pre, const LimbConst& lc, int poly,
-                                             int limb, int e) {
-    return ModeDecrypt::template load<N, SPLIT>(c, P.d, pre, lc, poly, limb, e);
-  }
-  template <int N>
-  static __device__ __forceinline__ void store(const DevCtx&, const Params&, const LimbConst& lc, int, int, int e,
-                                               u64 x) {
-    extern __shared__ __align__(16) u64 sm_res[];
-    sm_res[e] = x;   // x = N^{-1} qtil INTT, canonical
-  }
-  template <int N>
-  static __device__ __forceinline__ void finish(const DevCtx& c, const Params& P, int poly, u64* sm) {
-    namespace cg = cooperative_groups;
-    cg::cluster_group cl = cg::this_cluster();
-    cl.sync();   // every limb's residues are in its CTA's shared memory
-    const int T = (int)blockDim.x;
-    const int L = c.L;
-    const Window win(P.pk, P.ac, poly, P.y1);
-    const ulonglong2* res[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-      res[j] = reinterpret_cast<const ulonglong2*>(j < L ? cl.map_shared_rank(sm, j) : sm);
-    // coefficient pairs (2 p, 2 p + 1): 16-byte remote loads
-#pragma unroll 2
-    for (int p = (int)blockIdx.y * T + (int)threadIdx.x; p < N / 2; p += L * T) {
-      const ulonglong2 e0 = __ldg(P.pk.tab + 2 * p), e1 = __ldg(P.pk.tab + 2 * p + 1);
-      const bool h0 = win.has(e0), h1 = win.has(e1);
-      if (!h0 && !h1) continue;
-      CrtSum s0{0, 0}, s1{0, 0};
-#pragma unroll
-      for (int j = 0; j < 8; ++j)
-        if (j < L) {
-          const ulonglong2 y = res[j][p];
-          crt_add(s0, y.x, c.limb[j]);
-          crt_add(s1, y.y, c.limb[j]);
-        }
-      if (h0) *reinterpret_cast<u64*>(const_cast<char*>(win.at(e0))) = crt_round(s0, c.t_mask, P.check, c.status);
-      if (h1) *reinterpret_cast<u64*>(const_cast<char*>(win.at(e1))) = crt_round(s1, c.t_mask, P.check, c.status);
-    }
-    cl.sync();   // the other CTAs have finished reading this one's shared memory
-  }
-};
-
 // MO, compact send form of returned ciphertexts: INTT(c0) and, at the
 // coefficients carrying output element flat, c0c[limb][flat] = that coefficient
 // (the rest is dropped).
@@ -1281,6 +1368,13 @@ struct ModeCompact {
   };
   using Pre = NoPre;
   static __device__ __forceinline__ void rebase(Params&, u64) {}
+  template <int N>
+  static __device__ __forceinline__ void load2(const DevCtx& c, const Params& P, const LimbConst&, int poly, int limb,
+                                               int e, u64& x0, u64& x1) {
+    const ulonglong2 x = __ldg(reinterpret_cast<const ulonglong2*>(P.ct + ct_off(poly, 0, limb, c.L, N) + e));
+    x0 = x.x;
+    x1 = x.y;
+  }
   template <int N, bool SPLIT>
   static __device__ __forceinline__ u64 load(const DevCtx& c, const Params& P, const Pre& pre, const LimbConst&, int poly, int limb,
                                              int e) {
@@ -1294,6 +1388,16 @@ struct ModeCompact {
   }
 };
 
+// Whether a launch of `count` polynomials runs on clusters of four CTAs: forward while
+// every CTA has an SM of its own (its first two stages cost three products a word instead
+// of one), inverse, which does no more work, up to two per SM.  Measured (us, clusters /
+// one CTA each; N = 8192): forward 8 transforms 9.8 / 12.2, 38 12.1 / 12.1, 76 15.3 /
+// 12.2; inverse 8 7.4 / 12.8, 76 11.6 / 12.9, 120 14.3 / 12.9.  N = 16384: forward 8 12.9
+// / 21.8, 38 19.9 / 22.0, 76 27.5 / 22.4; inverse 76 22.4 / 24.1, 152 35.4 / 24.5.
+inline bool quad_wins(const DevCtx& ctx, long long count, bool inverse) {
+  return ctx.ntt_arith && ctx.ntt_loge == 4 && 4 * count * ctx.L <= (inverse ? 2 : 1) * ctx.sms;
+}
+
 // Host-side launcher; explicitly instantiated per LOGN and engine in ntt12.cu /
 // ntt13.cu / ntt14.cu (Shoup) and ntt12f.cu / ntt13f.cu / ntt14f.cu (folds).
 template <int LOGN, int LOGE, class Mode, bool INV, bool FOLD>
@@ -1302,29 +1406,28 @@ cudaError_t launch_ntt(const DevCtx& ctx, const typename Mode::Params& P, int fi
   if (count <= 0) return cudaSuccess;
   cudaError_t err;
   dim3 grid((unsigned)count, (unsigned)ctx.L);
+  if constexpr (FOLD && LOGE == 4) {
+    if (quad_wins(ctx, count, INV)) {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(4 * (unsigned)count, (unsigned)ctx.L);
+      cfg.blockDim = dim3((1 << LOGN) / 32);
+      cfg.dynamicSmemBytes = Quad<LOGN>::C::SMEM;
+      cfg.stream = s;
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = 4;
+      at[0].val.clusterDim.y = 1;
+      at[0].val.clusterDim.z = 1;
+      cfg.attrs = at;
+      cfg.numAttrs = 1;
+      return cudaLaunchKernelEx(&cfg, k_ntt_quad<LOGN, Mode, INV>, ctx, P, first);
+    }
+  }
   if constexpr (INV) {
     err = cudaFuncSetAttribute(k_ntt_inv<LOGN, LOGE, Mode, FOLD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)C::SMEM);
     if (err != cudaSuccess) return err;
-    if constexpr (ClusterLimbs<Mode>::value) {
-      // the L limb CTAs of a polynomial form one cluster (portable size <= 8)
-      if (ctx.L > 8) return cudaErrorInvalidValue;
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = grid;
-      cfg.blockDim = dim3((unsigned)C::T);
-      cfg.dynamicSmemBytes = C::SMEM;
-      cfg.stream = s;
-      cudaLaunchAttribute at[1];
-      at[0].id = cudaLaunchAttributeClusterDimension;
-      at[0].val.clusterDim.x = 1;
-      at[0].val.clusterDim.y = (unsigned)ctx.L;
-      at[0].val.clusterDim.z = 1;
-      cfg.attrs = at;
-      cfg.numAttrs = 1;
-      return cudaLaunchKernelEx(&cfg, k_ntt_inv<LOGN, LOGE, Mode, FOLD>, ctx, P, first);
-    } else {
-      k_ntt_inv<LOGN, LOGE, Mode, FOLD><<<grid, C::T, C::SMEM, s>>>(ctx, P, first);
-    }
+    k_ntt_inv<LOGN, LOGE, Mode, FOLD><<<grid, C::T, C::SMEM, s>>>(ctx, P, first);
   } else {
     err = cudaFuncSetAttribute(k_ntt_fwd<LOGN, LOGE, Mode, FOLD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)C::SMEM);
@@ -1338,7 +1441,6 @@ template <int LOGN, int LOGE, class Mode, bool INV, bool FOLD>
 cudaError_t launch_ntt_multi(const DevCtx& ctx, const typename Mode::Params* Ps, const int2* items, long long count,
                              const u64* step, cudaStream_t s) {
   using C = KCfg<LOGN, LOGE, FOLD>;
-  if constexpr (ClusterLimbs<Mode>::value) return cudaErrorNotSupported;   // single-plan launches only
   if (count <= 0) return cudaSuccess;
   if (count > 2147483647ll) return cudaErrorInvalidValue;
   cudaError_t err;
@@ -1374,8 +1476,7 @@ cudaError_t launch_ntt_multi(const DevCtx& ctx, const typename Mode::Params* Ps,
   PENCIL_NTT_INST1(SPEC, LOGN, LOGE, ModePkU, false, FOLD)       \
   PENCIL_NTT_INST1(SPEC, LOGN, LOGE, ModeEncryptPk, false, FOLD) \
   PENCIL_NTT_INST1(SPEC, LOGN, LOGE, ModeCompact, true, FOLD)    \
-  PENCIL_NTT_INST1(SPEC, LOGN, LOGE, ModeDecrypt, true, FOLD)     \
-  PENCIL_NTT_INST1(SPEC, LOGN, LOGE, ModeDecryptFused, true, FOLD)
+  PENCIL_NTT_INST1(SPEC, LOGN, LOGE, ModeDecrypt, true, FOLD)
 // Radix 2^4 and 2^5 register blocks for one N and one engine.
 #define PENCIL_NTT_INSTANTIATE(SPEC, LOGN, FOLD) \
   PENCIL_NTT_INST_E(SPEC, LOGN, 4, FOLD)         \
