@@ -484,6 +484,126 @@ __global__ void __launch_bounds__(MAC_BT + 32) k_mac_bulk(DevCtx ctx, MacParams 
   }
 }
 
+// ------------------------------------------------------------------ MAC, few input blocks
+// Alg. 1 with K <= MAC_SHORT_K input blocks.  What is left per output then is its own
+// traffic (a re-mask word in, two words out), so the kernel streams: a thread = one slot of
+// MAC_SHORT_M output rows m keeps A[m, 0 .. K-1] (both components, split) in registers and
+// walks a strip of output columns n, loading a column's K words of B and its re-mask words
+// one column ahead; B is read once for both rows, A once per strip, nothing goes through
+// shared memory and no CTA waits for a producer.  Four rows gained nothing over two
+// (registers), one row reads B twice as often.  L N = 24576, us, k_mac_bulk / this:
+// M = 30, NC = 64: K = 1 383 / 216, 3 510 / 301 (the least traffic, 1.13 GB, is 170), 6 767 / 465
+// (tensor cores 656); M = 10, NC = 16: K = 1 40 / 26, 3 51 / 34, 6 72 / 49; M = 64, NC = 10:
+// K = 3 198 / 110; M = 4, NC = 4: 13 to 15 either way.
+// 2 K <= 12 products per accumulator: no fold before the last.
+#define MAC_SHORT_K 6
+#define MAC_SHORT_M 2
+template <int K>
+__global__ void __launch_bounds__(MAC_BT) k_mac_short(const __grid_constant__ DevCtx ctx,
+                                                      const __grid_constant__ MacParams P, int strip, int strips) {
+  constexpr int MT = MAC_SHORT_M;
+  const int m0 = P.m_base + (int)(blockIdx.x / strips) * MT;
+  const int n0 = (int)(blockIdx.x % strips) * strip, n1 = min(n0 + strip, P.NC);
+  const int lane = blockIdx.y * MAC_BT + threadIdx.x;
+  const LimbConst& lc = ctx.limb[lane >> ctx.log_n];
+  constexpr u32 M30 = (1u << 30) - 1;
+  const size_t ln = (size_t)P.lanes;
+  u32 aL[MT][K][2], aH[MT][K][2];
+#pragma unroll
+  for (int i = 0; i < MT; ++i) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      const size_t mk = (size_t)min(m0 + i, P.M - 1) * K + k;
+      u64 a0 = __ldg(P.a0 + mk * P.a0_stride + lane);
+      const u64 a1 = __ldg(P.a1 + mk * P.a1_stride + lane);
+      if (P.p0) a0 = add_mod(a0, __ldg(P.p0 + mk * P.p0_stride + lane), lc.q);   // Alg. 1 step 2
+      aL[i][k][0] = (u32)a0 & M30;
+      aH[i][k][0] = (u32)(a0 >> 30);
+      aL[i][k][1] = (u32)a1 & M30;
+      aH[i][k][1] = (u32)(a1 >> 30);
+    }
+  }
+  u64 b[K], s[MT];
+  auto load = [&](int n) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) b[k] = __ldg(P.b + ((size_t)k * P.NC + n) * P.b_stride + lane);
+    if (P.mask) {
+#pragma unroll
+      for (int i = 0; i < MT; ++i)
+        s[i] = __ldg(P.mask + ((size_t)min(m0 + i, P.M - 1) * P.NC + n) * ln + lane);
+    }
+  };
+#pragma unroll
+  for (int i = 0; i < MT; ++i) s[i] = 0;
+  load(n0);
+#pragma unroll 1
+  for (int n = n0; n < n1; ++n) {
+    u32 bL[K], bH[K];
+    u64 sub[MT];
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      bL[k] = (u32)b[k] & M30;
+      bH[k] = (u32)(b[k] >> 30);
+    }
+#pragma unroll
+    for (int i = 0; i < MT; ++i) sub[i] = s[i];
+    if (n + 1 < n1) load(n + 1);
+#pragma unroll
+    for (int i = 0; i < MT; ++i) {
+      Acc3 acc[2] = {{0, 0, 0, 0, 0, 0}, {0, 0, 0, 0, 0, 0}};
+#pragma unroll
+      for (int k = 0; k < K; ++k)
+#pragma unroll
+        for (int c = 0; c < 2; ++c) mac_split(acc[c], aL[i][k][c], aH[i][k][c], bL[k], bH[k]);
+      if (m0 + i < P.M) {
+        u64* o = P.out + ((size_t)(m0 + i) * P.NC + n) * 2 * ln + lane;
+        o[0] = sub_mod(acc3_value(acc[0], lc), sub[i], lc.q);
+        o[ln] = acc3_value(acc[1], lc);
+      }
+    }
+  }
+}
+
+template <int K>
+static cudaError_t launch_mac_short_k(const DevCtx& ctx, const MacParams& P0, cudaStream_t s) {
+  if (P0.lanes % MAC_BT) return cudaErrorInvalidValue;   // L N is a multiple of 4096
+  MacParams P = P0;
+  const unsigned gy = (unsigned)(P.lanes / MAC_BT);
+  // Columns per strip: 16, or 8 where that leaves fewer than 16 CTAs per SM (us, 8 / 16:
+  // M = 30, NC = 64, K = 3, 76 per SM 311 / 301; M = 10, NC = 16, K = 3, 6 per SM 34.0 / 36.5;
+  // M = 2, NC = 64, K = 6, 5 per SM 42.1 / 45.0); strips of even width.
+  const long long mtiles = ((long long)P0.M - P0.m_base + MAC_SHORT_M - 1) / MAC_SHORT_M;
+  const int most = mtiles * ((P.NC + 15) / 16) * gy >= 16ll * ctx.sms ? 16 : 8;
+  const int strips = (P.NC + most - 1) / most, strip = (P.NC + strips - 1) / strips;
+  const long long mchunk = (long long)max(1, 2147483647 / strips) * MAC_SHORT_M;
+  for (long long base = P0.m_base; base < P0.M; base += mchunk) {   // output rows m in [m_base, M)
+    P.m_base = (int)base;
+    const long long mc = (std::min<long long>(mchunk, P0.M - base) + MAC_SHORT_M - 1) / MAC_SHORT_M;
+    k_mac_short<K><<<dim3((unsigned)(mc * strips), gy), MAC_BT, 0, s>>>(ctx, P, strip, strips);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+static cudaError_t launch_mac_short(const DevCtx& ctx, const MacParams& P, cudaStream_t s) {
+  switch (P.K) {
+    case 1:
+      return launch_mac_short_k<1>(ctx, P, s);
+    case 2:
+      return launch_mac_short_k<2>(ctx, P, s);
+    case 3:
+      return launch_mac_short_k<3>(ctx, P, s);
+    case 4:
+      return launch_mac_short_k<4>(ctx, P, s);
+    case 5:
+      return launch_mac_short_k<5>(ctx, P, s);
+    case 6:
+      return launch_mac_short_k<6>(ctx, P, s);
+  }
+  return cudaErrorInvalidValue;
+}
+
 // ------------------------------------------------------------------ MAC, shared-memory staged
 // CTA = 32 slots x 8 warps.  The CTA owns an output block of MB x NB (m, n)
 // pairs (MB * NB = 64) for its 32 slots; warp w owns pairs 8w .. 8w + 7
@@ -725,7 +845,8 @@ static cudaError_t launch_mac_bulk(const DevCtx& ctx, const MacParams& P0, bool 
 // 5 657 / 651, 6 657 / 768, 16 875 / 1542, 32 1582 / 2871; M = 10, NC = 16: K = 6
 // 74 / 72, 8 75 / 84, 16 91 / 138; M = 4, NC = 4: K = 16 36 / 25, 32 65 / 42; M = 2,
 // NC = 64: K = 16 150 / 114.  Two 54-bit primes at N = 4096 (k_mac): M = 10, NC = 16:
-// K = 1 24 / 22, 2 24 / 28, 16 38 / 129.
+// K = 1 24 / 22, 2 24 / 28, 16 38 / 129.  (Single launches with split-form primes take
+// k_mac_short up to K = 6; there the rule decides for the batch engine's items only.)
 bool mac_mma_wins(const DevCtx& ctx, const MacParams& P, bool dual) {
   if (!ctx.mac_mma || ctx.mac_nt == 0 || ctx.mac_staging != 1) return false;   // not available, or tuned away
   const double rows = P.M - P.m_base, K = P.K, nt = (P.NC + 15) / 16, pairs = rows * P.NC / 64.0;
@@ -737,6 +858,8 @@ bool mac_mma_wins(const DevCtx& ctx, const MacParams& P, bool dual) {
 }
 
 cudaError_t launch_mac(const DevCtx& ctx, const MacParams& P0, bool dual, cudaStream_t s) {
+  if (!dual && ctx.mac_split && ctx.mac_nt != 0 && ctx.mac_staging == 1 && P0.K >= 1 && P0.K <= MAC_SHORT_K)
+    return launch_mac_short(ctx, P0, s);   // faster than both at every size measured
   if (mac_mma_wins(ctx, P0, dual)) return launch_mac_mma(ctx, P0, dual, s);
   if (ctx.mac_split && ctx.mac_nt == 0) return launch_mac_smem(ctx, P0, dual, s);
   if (ctx.mac_split && ctx.mac_staging == 1) {
