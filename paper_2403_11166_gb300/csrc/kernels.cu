@@ -966,35 +966,82 @@ cudaError_t launch_sample_pk(u64 seed, int first, int count, int n, int8_t* e1, 
 // Mask polynomial of each output ciphertext: at coefficients carrying output
 // element `flat`, Philox(key (seed, 4), counter (flat/4, 0, 0, 0)) word flat%4;
 // elsewhere Philox(key (seed, 5), counter (i/4, ct, 0, 0)) word i%4; mod t.
-// Coefficients 4 blk .. 4 blk + 3 of output polynomial ct.  The padding stream's block is
-// drawn where some coefficient carries no output; then each pass evaluates one block of
-// the element stream for every coefficient that draws from it, so a warp takes as many
-// passes as its worst thread has different blocks: one or two, where one per coefficient
-// took four (rows of outputs start at any flat % 4; 1920 polynomials of 28 x 19 tiles at
-// N = 8192: 239 us with four).
+// A CTA of 256 threads does 1024 consecutive coefficients of output polynomial ct, four
+// per thread (blk: this thread's).  Bound by the Philox blocks it draws: neighbours carry
+// neighbouring elements, rows starting at any flat % 4, so a thread alone meets one to
+// three blocks and a warp pays for its worst thread (a padding pass and two element passes;
+// one per coefficient before that).  Here the CTA lists its different blocks once, draws
+// them one per thread and hands the words out through shared memory: about 1.3 blocks per
+// thread where rows are 28 elements and a gap of 2 (1920 polynomials of 28 x 19 tiles at
+// N = 8192: 163 -> 112 us; 160 of 32 x 32 tiles 20 -> 16; polynomials that are nearly all
+// padding, whose blocks no two threads share, pay for the list: three launches of a 128 to
+// 128 channel layer's forward and gradients 338 -> 369).
+#define MASK_POLY_LIST 512   // blocks drawn at a time (of at most 256 + 1024): 20 KB, eight CTAs per SM
 __device__ __forceinline__ void mask_poly_block(const DevCtx& ctx, const Packing& pk, const Window& win, u64 seed,
                                                 int ct, int blk, u64* out_ct) {
-  i64 flat[4];
-  u32 todo = 0;
+  __shared__ i64 src[MASK_POLY_LIST];   // element block, or -1 - (block of the padding stream)
+  __shared__ __align__(16) u64 word[MASK_POLY_LIST][4];
+  __shared__ int warp_total[8];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  i64 key[4];
+  u32 sub = 0, lead = 0;   // flat % 4 (two bits each); first coefficient of a run on one block
+  bool pad = false;
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    flat[i] = win.index(pk, 4 * blk + i);
-    todo |= flat[i] >= 0 ? 1u << i : 0u;
+    const i64 flat = win.index(pk, 4 * blk + i);
+    key[i] = flat >> 2;   // (-1: no output)
+    sub |= (u32)(flat & 3) << (2 * i);
+    pad = pad || flat < 0;
+  }
+  // a run (at most four coefficients: elements of a polynomial differ) may continue the
+  // previous lane's; its first lane lists it
+  const i64 before = __shfl_up_sync(0xffffffffu, key[3], 1);
+  if (key[0] >= 0 && (lane == 0 || before != key[0])) lead |= 1u;
+#pragma unroll
+  for (int i = 1; i < 4; ++i)
+    if (key[i] >= 0 && key[i] != key[i - 1]) lead |= 1u << i;
+  const int mine = __popc(lead) + (pad ? 1 : 0);
+  int upto = mine;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const int o = __shfl_up_sync(0xffffffffu, upto, d);
+    if (lane >= d) upto += o;
+  }
+  if (lane == 31) warp_total[warp] = upto;
+  __syncthreads();
+  int base = upto - mine, total = 0;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) {
+    base += w < warp ? warp_total[w] : 0;
+    total += warp_total[w];
+  }
+  // coefficient i's entry in the list: padding at `base`, then this thread's runs; a run
+  // continued from the previous lane is the last entry before `base`
+  int at[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int n = __popc(lead & ((2u << i) - 1u));
+    at[i] = key[i] < 0 ? base : n ? base + (pad ? 1 : 0) + n - 1 : base - 1;
   }
   Philox4 r = {{0, 0, 0, 0}};
-  if (todo != 15u) r = philox4x64((u64)blk, (u64)ct, 0ull, 0ull, seed, PENCIL_DOM_MASK_PAD);
-  while (todo) {
-    i64 src = 0;
-#pragma unroll
-    for (int i = 3; i >= 0; --i)
-      if (todo >> i & 1u) src = flat[i] >> 2;
-    const Philox4 w = philox4x64((u64)src, 0ull, 0ull, 0ull, seed, PENCIL_DOM_MASK);
+  for (int c0 = 0; c0 < total; c0 += MASK_POLY_LIST) {   // (once, but for widely strided outputs)
+    if (pad && (unsigned)(base - c0) < MASK_POLY_LIST) src[base - c0] = -1 - (i64)blk;
 #pragma unroll
     for (int i = 0; i < 4; ++i)
-      if ((todo >> i & 1u) && flat[i] >> 2 == src) {
-        r.v[i] = philox_word(w, (int)(flat[i] & 3));
-        todo &= ~(1u << i);
-      }
+      if ((lead >> i & 1u) && (unsigned)(at[i] - c0) < MASK_POLY_LIST) src[at[i] - c0] = key[i];
+    __syncthreads();
+    for (int e = tid; e < min(total - c0, MASK_POLY_LIST); e += 256) {
+      const i64 b = src[e];
+      const Philox4 w = philox4x64((u64)(b >= 0 ? b : -1 - b), b >= 0 ? 0ull : (u64)ct, 0ull, 0ull, seed,
+                                   b >= 0 ? PENCIL_DOM_MASK : PENCIL_DOM_MASK_PAD);
+      reinterpret_cast<ulonglong2*>(word[e])[0] = make_ulonglong2(w.v[0], w.v[1]);
+      reinterpret_cast<ulonglong2*>(word[e])[1] = make_ulonglong2(w.v[2], w.v[3]);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if ((unsigned)(at[i] - c0) < MASK_POLY_LIST)
+        r.v[i] = word[at[i] - c0][key[i] < 0 ? (u32)i : sub >> (2 * i) & 3u];
   }
   ulonglong2* o = reinterpret_cast<ulonglong2*>(out_ct + 4 * blk);
   o[0] = make_ulonglong2(r.v[0] & ctx.t_mask, r.v[1] & ctx.t_mask);
