@@ -90,8 +90,10 @@ int pencil_ctx_primes(const PencilCtx* ctx, uint64_t* primes, uint64_t* psis);
  * thread copies its own operand words a few input blocks ahead (cp.async ring);
  * 1 (default) = exact base-256 digit products on the tensor cores where they are
  * the faster form for the product's sizes and the primes allow them (2^b - c with
- * c < 2^(b-32)), else integer multiply-adds with one producer warp per CTA copying
- * whole 1 KB operand rows (cp.async.bulk + mbarrier).
+ * c < 2^(b-32)); integer multiply-adds that keep the ciphertext rows in registers
+ * for Alg. 1 products of at most six input blocks; else integer multiply-adds with
+ * one producer warp per CTA copying whole 1 KB operand rows (cp.async.bulk +
+ * mbarrier).  (The columns then apply to the last form and to batches.)
  * PENCIL_TUNE_NTT_ARITH: butterfly arithmetic of the NTT kernels: 0 = Shoup
  * products with Harvey's lazy butterflies (any prime); 1 = pseudo-Mersenne
  * products of signed lazily growing values (q = 2^b - c: the high word of a split

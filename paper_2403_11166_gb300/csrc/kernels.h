@@ -153,7 +153,7 @@ PENCIL_NTT_INSTANTIATE(extern, 13, true)
 PENCIL_NTT_INSTANTIATE(extern, 14, true)
 
 // Dispatch on log2(N), the context's radix (log2 of coefficients per thread) and
-// its butterfly arithmetic (Shoup / Harvey, or pseudo-Mersenne folds).
+// its butterfly arithmetic (Shoup / Harvey, or signed split products).
 template <class Mode, bool INV>
 cudaError_t ntt_multi(const DevCtx& ctx, const typename Mode::Params* Ps, const int2* items, long long count,
                       const u64* step, cudaStream_t s) {

@@ -1449,7 +1449,7 @@ inline bool quad_wins(const DevCtx& ctx, long long count, bool inverse) {
 }
 
 // Host-side launcher; explicitly instantiated per LOGN and engine in ntt12.cu /
-// ntt13.cu / ntt14.cu (Shoup) and ntt12f.cu / ntt13f.cu / ntt14f.cu (folds).
+// ntt13.cu / ntt14.cu (Shoup) and ntt12f.cu / ntt13f.cu / ntt14f.cu (split products).
 template <int LOGN, int LOGE, class Mode, bool INV, bool FOLD>
 cudaError_t launch_ntt(const DevCtx& ctx, const typename Mode::Params& P, int first, int count, cudaStream_t s) {
   using C = KCfg<LOGN, LOGE, FOLD>;
