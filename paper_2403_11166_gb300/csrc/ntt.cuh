@@ -883,17 +883,17 @@ __device__ __forceinline__ void prefetch_ahead(const DevCtx& ctx, const typename
   }
 }
 
-// CTA (x, limb) transforms polynomial first + x.
-template <int LOGN, int LOGE, class Mode, bool FOLD>
-__global__ void __launch_bounds__(KCfg<LOGN, LOGE, FOLD>::T, KCfg<LOGN, LOGE, FOLD>::MIN_BLOCKS)
+// CTA (x, limb) transforms polynomial first + x; MB CTAs per SM.
+template <int LOGN, int LOGE, class Mode, bool FOLD, int MB = KCfg<LOGN, LOGE, FOLD>::MIN_BLOCKS>
+__global__ void __launch_bounds__(KCfg<LOGN, LOGE, FOLD>::T, MB)
     k_ntt_fwd(DevCtx ctx, typename Mode::Params P, int first) {
   extern __shared__ __align__(16) u64 sm[];
   prefetch_ahead<1 << LOGN, Mode>(ctx, P, first);
   fwd_any<LOGN, LOGE, Mode, FOLD>(ctx, P, first + (int)blockIdx.x, blockIdx.y, sm);
 }
 
-template <int LOGN, int LOGE, class Mode, bool FOLD>
-__global__ void __launch_bounds__(KCfg<LOGN, LOGE, FOLD>::T, KCfg<LOGN, LOGE, FOLD>::MIN_BLOCKS)
+template <int LOGN, int LOGE, class Mode, bool FOLD, int MB = KCfg<LOGN, LOGE, FOLD>::MIN_BLOCKS>
+__global__ void __launch_bounds__(KCfg<LOGN, LOGE, FOLD>::T, MB)
     k_ntt_inv(DevCtx ctx, typename Mode::Params P, int first) {
   extern __shared__ __align__(16) u64 sm[];
   prefetch_ahead<1 << LOGN, Mode>(ctx, P, first);
@@ -1448,14 +1448,25 @@ inline bool quad_wins(const DevCtx& ctx, long long count, bool inverse) {
   return ctx.ntt_arith && ctx.ntt_loge == 4 && 4 * count * ctx.L <= (inverse ? 2 : 1) * ctx.sms;
 }
 
+// Whether a launch of 256-thread transforms (N = 4096, radix 2^4) runs four to an SM with 64
+// registers a thread (some spill a word or two) instead of two with up to 120: once there are
+// enough of them, issue is what bounds it and 32 warps hide more than 16; a launch that fits
+// the SMs in one go is each transform's latency, which the registers shorten.  Measured (us, two /
+// four per SM): raw forward 2.6 transforms per SM 26.1 / 26.2, 3.9 30.7 / 30.3, 5.1 39.1 /
+// 38.2, 13.8 75.1 / 68.2, 59 279 / 247; raw inverse 3.9 33.9 / 34.9, 5.1 43.2 / 42.8, 7.9
+// 52.5 / 52.9, 59 310 / 289; encoding 3.4 27.8 / 26.4, 13.5 63.5 / 55.1; MO preparation 18.5
+// 180 / 154; decryption 4.6 65.7 / 58.5, 9.3 122 / 101.
+inline bool many_small(const DevCtx& ctx, long long count, bool inverse) {
+  return count * ctx.L > (inverse ? 4ll : 3ll) * ctx.sms;
+}
+
 // Host-side launcher; explicitly instantiated per LOGN and engine in ntt12.cu /
 // ntt13.cu / ntt14.cu (Shoup) and ntt12f.cu / ntt13f.cu / ntt14f.cu (split products).
 template <int LOGN, int LOGE, class Mode, bool INV, bool FOLD>
 cudaError_t launch_ntt(const DevCtx& ctx, const typename Mode::Params& P, int first, int count, cudaStream_t s) {
   using C = KCfg<LOGN, LOGE, FOLD>;
   if (count <= 0) return cudaSuccess;
-  cudaError_t err;
-  dim3 grid((unsigned)count, (unsigned)ctx.L);
+  const dim3 grid((unsigned)count, (unsigned)ctx.L);
   if constexpr (FOLD && LOGE == 4) {
     if (quad_wins(ctx, count, INV)) {
       cudaLaunchConfig_t cfg = {};
@@ -1473,18 +1484,24 @@ cudaError_t launch_ntt(const DevCtx& ctx, const typename Mode::Params& P, int fi
       return cudaLaunchKernelEx(&cfg, k_ntt_quad<LOGN, Mode, INV>, ctx, P, first);
     }
   }
-  if constexpr (INV) {
-    err = cudaFuncSetAttribute(k_ntt_inv<LOGN, LOGE, Mode, FOLD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)C::SMEM);
+  auto launch = [&](auto kernel) {
+    const cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
     if (err != cudaSuccess) return err;
-    k_ntt_inv<LOGN, LOGE, Mode, FOLD><<<grid, C::T, C::SMEM, s>>>(ctx, P, first);
-  } else {
-    err = cudaFuncSetAttribute(k_ntt_fwd<LOGN, LOGE, Mode, FOLD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)C::SMEM);
-    if (err != cudaSuccess) return err;
-    k_ntt_fwd<LOGN, LOGE, Mode, FOLD><<<grid, C::T, C::SMEM, s>>>(ctx, P, first);
+    kernel<<<grid, C::T, C::SMEM, s>>>(ctx, P, first);
+    return cudaGetLastError();
+  };
+  if constexpr (FOLD && LOGN == 12 && LOGE == 4) {
+    if (many_small(ctx, count, INV)) {
+      if constexpr (INV)
+        return launch(k_ntt_inv<LOGN, LOGE, Mode, FOLD, 4>);
+      else
+        return launch(k_ntt_fwd<LOGN, LOGE, Mode, FOLD, 4>);
+    }
   }
-  return cudaGetLastError();
+  if constexpr (INV)
+    return launch(k_ntt_inv<LOGN, LOGE, Mode, FOLD>);
+  else
+    return launch(k_ntt_fwd<LOGN, LOGE, Mode, FOLD>);
 }
 
 template <int LOGN, int LOGE, class Mode, bool INV, bool FOLD>
