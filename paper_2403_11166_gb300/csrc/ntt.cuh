@@ -1444,6 +1444,9 @@ struct ModeCompact {
 // one CTA each; N = 8192): forward 8 transforms 9.8 / 12.2, 38 12.1 / 12.1, 76 15.3 /
 // 12.2; inverse 8 7.4 / 12.8, 76 11.6 / 12.9, 120 14.3 / 12.9.  N = 16384: forward 8 12.9
 // / 21.8, 38 19.9 / 22.0, 76 27.5 / 22.4; inverse 76 22.4 / 24.1, 152 35.4 / 24.5.
+// N = 4096 (L = 2): inverse 3 transforms 5.5 / 7.2; encryption 10.3 / 13.6, encoding 6.7 / 7.3,
+// preparation 13.9 / 15.5; the bare forward transform, whose prologue and epilogue leave the
+// CTAs nothing else to share, 7.5 / 6.3: it alone stays in one CTA.
 inline bool quad_wins(const DevCtx& ctx, long long count, bool inverse) {
   return ctx.ntt_arith && ctx.ntt_loge == 4 && 4 * count * ctx.L <= (inverse ? 2 : 1) * ctx.sms;
 }
@@ -1468,7 +1471,7 @@ cudaError_t launch_ntt(const DevCtx& ctx, const typename Mode::Params& P, int fi
   if (count <= 0) return cudaSuccess;
   const dim3 grid((unsigned)count, (unsigned)ctx.L);
   if constexpr (FOLD && LOGE == 4) {
-    if (quad_wins(ctx, count, INV)) {
+    if (quad_wins(ctx, count, INV) && !(LOGN == 12 && std::is_same_v<Mode, ModeRaw> && !INV)) {
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(4 * (unsigned)count, (unsigned)ctx.L);
       cfg.blockDim = dim3((1 << LOGN) / 32);
