@@ -21,8 +21,11 @@ static cudaError_t launch(const DevCtx& ctx, const MacParams& P0, cudaStream_t s
   using T = MmaTile<DUAL, MT, NT>;
   const int stages = P0.K > T::KC ? 2 : 1;
   const size_t smem = T::bytes(stages);
+  // The attribute belongs to the function, not to this launch: every caller sets the same
+  // (two-stage) value, so that a thread with one stage cannot lower it between another
+  // thread's call here and its launch with two.
   const cudaError_t e =
-      cudaFuncSetAttribute(k_mac_mma<DUAL, MT, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      cudaFuncSetAttribute(k_mac_mma<DUAL, MT, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::bytes(2));
   if (e != cudaSuccess) return e;
   MacParams P = P0;
   const int ntiles = (P0.NC + NT - 1) / NT;
