@@ -23,10 +23,11 @@
 
 #include "digits.cuh"
 #include "kernels.h"
+#include "rules.h"
 
 namespace pencil {
 
-#define RM_KC 16
+#define RM_KC 16           // (ring_split's chunks)
 #define RM_PITCH 18        // words of a row of 16 k: 144 bytes, LDS.128 of 8 rows x 4 threads conflict-free
 #define RM_STAGES 3
 #define RM_THREADS 128
@@ -34,9 +35,8 @@ namespace pencil {
 struct RingMma {
   long long npos;          // B * Ho * Wo
   long long K;             // reduction length
-  int chunks, per;         // chunks of 16, chunks of one part
+  RingSplit r;             // its parts; parts > 1: atomics
   int v_rows, w_rows;      // lanes along rows (1) or along k (0)
-  int split;               // parts > 1: atomics
 };
 
 struct RmRow {   // one output column (position) of V: offset of its window, window origin
@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(RM_THREADS, MI == 2 ? 2 : 3) k_ring_mma(const 
   const long long pos0 = (long long)blockIdx.x * BN;
   const int o0 = blockIdx.y * BM;
   const int Co = P.kbound.x, KH = P.kbound.z, KW = P.kbound.w;
-  const int c0 = blockIdx.z * R.per, c1 = min(R.chunks, c0 + R.per);
+  const unsigned c0 = blockIdx.z * R.r.per, c1 = c0 + min(R.r.per, R.r.chunks - c0);
   constexpr int FAR = -(1 << 30);
   if (tid < BN) {
     const long long pos = pos0 + tid;
@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(RM_THREADS, MI == 2 ? 2 : 3) k_ring_mma(const 
     }
     rows[tid] = r;
   }
-  auto make_k = [&](int ch) {   // threads 0 .. 15
+  auto make_k = [&](unsigned ch) {   // threads 0 .. 15
     const long long k = (long long)ch * RM_KC + tid;
     RmK e{0, FAR, 0};
     i64 w = 0;
@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(RM_THREADS, MI == 2 ? 2 : 3) k_ring_mma(const 
     ktab[ch & 1][tid] = e;
     kw[ch & 1][tid] = w;
   };
-  auto issue = [&](int ch) {
+  auto issue = [&](unsigned ch) {
     u64* st = sm + (ch % RM_STAGES) * ((BM + BN) * RM_PITCH);
     const RmK* kt = ktab[ch & 1];
     // in row order a thread's row, in k order its k, is the same in every pass
@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(RM_THREADS, MI == 2 ? 2 : 3) k_ring_mma(const 
 #pragma unroll
       for (int o = 0; o < 4; ++o) sum[mi][ni][o] = 0;
 
-  for (int ch = c0; ch < c1; ++ch) {
+  for (unsigned ch = c0; ch < c1; ++ch) {
     asm volatile("cp.async.wait_group 1;\n" ::: "memory");
     __syncthreads();   // chunk ch is here; chunk ch - 1 has been read; the table of ch + 2 is written
     if (ch + 2 < c1) issue(ch + 2);
@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(RM_THREADS, MI == 2 ? 2 : 3) k_ring_mma(const 
           if (o >= Co) continue;
           const i64 flat = base + o * P.y.s1;
           u64 v = sum[mi][ni][2 * h + w] - bias;
-          if (R.split) {
+          if (R.r.parts > 1) {
             atomicAdd(reinterpret_cast<unsigned long long*>(P.out + flat), (unsigned long long)v);
           } else {
             if (P.addend) v += P.addend[flat];
@@ -314,20 +314,15 @@ static cudaError_t launch(const RingParams& P, RingMma R, int sms, cudaStream_t 
       cudaFuncSetAttribute(k_ring_mma<D, MI, WM, WN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const long long gx = (R.npos + BN - 1) / BN, gy = (P.kbound.x + BM - 1) / BM;
-  // parts: up to three CTAs per SM, at least four chunks each
-  long long parts = std::max<long long>(1, 3ll * sms / std::max<long long>(1, gx * gy));
-  parts = std::min<long long>(parts, std::max(1, R.chunks / 4));
-  R.per = (int)((R.chunks + parts - 1) / parts);
-  parts = (R.chunks + R.per - 1) / R.per;
-  R.split = parts > 1;
+  if (!ring_split(R.K, gx * gy, sms, &R.r)) return cudaErrorInvalidValue;
   const unsigned eb = (unsigned)((P.outs + 255) / 256);
-  if (R.split) {
+  if (R.r.parts > 1) {
     k_ring_edge<<<eb, 256, 0, s>>>(P, 1);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
-  k_ring_mma<D, MI, WM, WN><<<dim3((unsigned)gx, (unsigned)gy, (unsigned)parts), RM_THREADS, smem, s>>>(P, R);
+  k_ring_mma<D, MI, WM, WN><<<dim3((unsigned)gx, (unsigned)gy, R.r.parts), RM_THREADS, smem, s>>>(P, R);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if (R.split) {
+  if (R.r.parts > 1) {
     k_ring_edge<<<eb, 256, 0, s>>>(P, 0);
     e = cudaGetLastError();
   }
@@ -346,8 +341,6 @@ cudaError_t launch_ring_mma(const RingParams& P, int sms, cudaStream_t s) {
   RingMma R{};
   R.npos = P.outs / Co;
   R.K = (long long)Ci * KH * KW;
-  if (R.K > (1ll << 34)) return cudaErrorInvalidValue;
-  R.chunks = (int)((R.K + RM_KC - 1) / RM_KC);
   const long long B = R.npos / ((long long)P.Ho * P.Wo);
   R.v_rows = run(P.Wo, P.v.s3, P.Ho == 1 ? B : 1, P.v.s0) >= run(KW, P.v.s3, KH == 1 ? Ci : 1, P.v.s1);
   R.w_rows = (P.w.s0 == 1 ? std::min(Co, 32) : 1) > run(KW, P.w.s3, KH == 1 ? Ci : 1, P.w.s1);
