@@ -34,9 +34,11 @@ namespace pencil {
 
 struct RingMma {
   long long npos;          // B * Ho * Wo
-  long long K;             // reduction length
-  RingSplit r;             // its parts; parts > 1: atomics
+  long long K;             // reduction length of this launch, from element k0 on
+  long long k0;
+  int chunks, per;         // chunks of 16, chunks of one part
   int v_rows, w_rows;      // lanes along rows (1) or along k (0)
+  int split;               // several parts or launches: atomics
 };
 
 struct RmRow {   // one output column (position) of V: offset of its window, window origin
@@ -103,7 +105,7 @@ __global__ void __launch_bounds__(RM_THREADS, MI == 2 ? 2 : 3) k_ring_mma(const 
   const long long pos0 = (long long)blockIdx.x * BN;
   const int o0 = blockIdx.y * BM;
   const int Co = P.kbound.x, KH = P.kbound.z, KW = P.kbound.w;
-  const unsigned c0 = blockIdx.z * R.r.per, c1 = c0 + min(R.r.per, R.r.chunks - c0);
+  const int c0 = blockIdx.z * R.per, c1 = min(R.chunks, c0 + R.per);
   constexpr int FAR = -(1 << 30);
   if (tid < BN) {
     const long long pos = pos0 + tid;
@@ -118,13 +120,13 @@ __global__ void __launch_bounds__(RM_THREADS, MI == 2 ? 2 : 3) k_ring_mma(const 
     }
     rows[tid] = r;
   }
-  auto make_k = [&](unsigned ch) {   // threads 0 .. 15
+  auto make_k = [&](int ch) {   // threads 0 .. 15
     const long long k = (long long)ch * RM_KC + tid;
     RmK e{0, FAR, 0};
     i64 w = 0;
     if (k < R.K) {
-      const long long uv = (long long)KH * KW, c = k / uv;
-      const int q = (int)(k - c * uv);
+      const long long uv = (long long)KH * KW, e0 = R.k0 + k, c = e0 / uv;
+      const int q = (int)(e0 - c * uv);
       e.u = q / KW;
       e.x = q - e.u * KW;
       e.v = c * P.v.s1 + e.u * P.v.s2 + e.x * P.v.s3;
@@ -133,7 +135,7 @@ __global__ void __launch_bounds__(RM_THREADS, MI == 2 ? 2 : 3) k_ring_mma(const 
     ktab[ch & 1][tid] = e;
     kw[ch & 1][tid] = w;
   };
-  auto issue = [&](unsigned ch) {
+  auto issue = [&](int ch) {
     u64* st = sm + (ch % RM_STAGES) * ((BM + BN) * RM_PITCH);
     const RmK* kt = ktab[ch & 1];
     // in row order a thread's row, in k order its k, is the same in every pass
@@ -206,7 +208,7 @@ __global__ void __launch_bounds__(RM_THREADS, MI == 2 ? 2 : 3) k_ring_mma(const 
 #pragma unroll
       for (int o = 0; o < 4; ++o) sum[mi][ni][o] = 0;
 
-  for (unsigned ch = c0; ch < c1; ++ch) {
+  for (int ch = c0; ch < c1; ++ch) {
     asm volatile("cp.async.wait_group 1;\n" ::: "memory");
     __syncthreads();   // chunk ch is here; chunk ch - 1 has been read; the table of ch + 2 is written
     if (ch + 2 < c1) issue(ch + 2);
@@ -281,7 +283,7 @@ __global__ void __launch_bounds__(RM_THREADS, MI == 2 ? 2 : 3) k_ring_mma(const 
           if (o >= Co) continue;
           const i64 flat = base + o * P.y.s1;
           u64 v = sum[mi][ni][2 * h + w] - bias;
-          if (R.r.parts > 1) {
+          if (R.split) {
             atomicAdd(reinterpret_cast<unsigned long long*>(P.out + flat), (unsigned long long)v);
           } else {
             if (P.addend) v += P.addend[flat];
@@ -314,15 +316,22 @@ static cudaError_t launch(const RingParams& P, RingMma R, int sms, cudaStream_t 
       cudaFuncSetAttribute(k_ring_mma<D, MI, WM, WN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const long long gx = (R.npos + BN - 1) / BN, gy = (P.kbound.x + BM - 1) / BM;
-  if (!ring_split(R.K, gx * gy, sms, &R.r)) return cudaErrorInvalidValue;
+  const long long K = R.K;
+  R.split = K > kRingLaunchK || ring_split(K, gx * gy, sms).parts > 1;
   const unsigned eb = (unsigned)((P.outs + 255) / 256);
-  if (R.r.parts > 1) {
+  if (R.split) {
     k_ring_edge<<<eb, 256, 0, s>>>(P, 1);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
-  k_ring_mma<D, MI, WM, WN><<<dim3((unsigned)gx, (unsigned)gy, R.r.parts), RM_THREADS, smem, s>>>(P, R);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if (R.r.parts > 1) {
+  for (R.k0 = 0; R.k0 < K; R.k0 += kRingLaunchK) {
+    R.K = std::min(K - R.k0, kRingLaunchK);
+    const RingSplit r = ring_split(R.K, gx * gy, sms);
+    R.chunks = r.chunks;
+    R.per = r.per;
+    k_ring_mma<D, MI, WM, WN><<<dim3((unsigned)gx, (unsigned)gy, (unsigned)r.parts), RM_THREADS, smem, s>>>(P, R);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  if (R.split) {
     k_ring_edge<<<eb, 256, 0, s>>>(P, 0);
     e = cudaGetLastError();
   }

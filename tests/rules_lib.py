@@ -11,14 +11,13 @@ CSRC = os.path.join(ROOT, "paper_2403_11166_gb300", "csrc")
 SHIM = r"""
 #include "rules.h"
 using namespace pencil;
-extern "C" int ring_split_(long long K, long long tiles, int sms, unsigned* out) {
-  RingSplit r;
-  if (!ring_split(K, tiles, sms, &r)) return 0;
+extern "C" void ring_split_(long long K, long long tiles, int sms, int* out) {
+  const RingSplit r = ring_split(K, tiles, sms);
   out[0] = r.chunks;
   out[1] = r.per;
   out[2] = r.parts;
-  return 1;
 }
+extern "C" long long ring_launch_k() { return kRingLaunchK; }
 """
 
 
@@ -34,7 +33,12 @@ def load() -> ctypes.CDLL:
 
 
 def ring_split(k: int, tiles: int, sms: int = 152):
-    """(chunks, chunks of a part, parts), or None where the length is refused."""
-    out = (ctypes.c_uint * 3)()
-    ok = load().ring_split_(ctypes.c_longlong(k), ctypes.c_longlong(tiles), sms, out)
-    return tuple(out) if ok else None
+    """(chunks, chunks of a part, parts) of one launch"""
+    out = (ctypes.c_int * 3)()
+    load().ring_split_(ctypes.c_longlong(k), ctypes.c_longlong(tiles), sms, out)
+    return tuple(out)
+
+
+def ring_launch_k() -> int:
+    load().ring_launch_k.restype = ctypes.c_longlong
+    return load().ring_launch_k()

@@ -7,21 +7,19 @@ from tests import rules_lib
 MOST_WORDS = 284208 * (1 << 20) // 8
 
 
-@pytest.mark.parametrize("k", [1, 16, 17, 784, 6272, (1 << 31) + 5, (1 << 34) - 1, (1 << 34) + 1, 1 << 35, (1 << 35) + 16,
+@pytest.mark.parametrize("k", [1, 16, 17, 784, 6272, (1 << 31) + 5, (1 << 34) - 1, 1 << 34, (1 << 34) + 1, 1 << 35,
                                MOST_WORDS])
 @pytest.mark.parametrize("tiles", [1, 3, 100, 457, 100000])
 def test_ring_parts_cover_every_reduction_that_fits_the_device(k, tiles):
-    """Every reduction whose operand fits the device is taken; its parts cover the chunks
-    once, none is empty, and no chunk number (the kernel looks three ahead) leaves 32 bits."""
-    split = rules_lib.ring_split(k, tiles)
-    assert split is not None
-    chunks, per, parts = split
-    assert chunks == -(-k // 16)
-    assert (parts - 1) * per < chunks <= parts * per
-    assert parts <= 65535 and (parts == 1 or per >= 4)
-    assert chunks + 3 < 1 << 32
-
-
-def test_ring_refuses_what_cannot_exist():
-    assert rules_lib.ring_split(0, 1) is None
-    assert rules_lib.ring_split(3 << 34, 1) is None
+    """Every reduction whose operand fits the device is taken, in launches of at most
+    ring_launch_k elements: a launch's parts cover its chunks once, none is empty, and no
+    chunk number (the kernel looks three ahead) leaves 32 bits."""
+    most, start = rules_lib.ring_launch_k(), 0
+    assert most % 16 == 0
+    while start < k:
+        part = min(k - start, most)
+        chunks, per, parts = rules_lib.ring_split(part, tiles)
+        assert chunks == -(-part // 16) and chunks + 3 < 1 << 31
+        assert (parts - 1) * per < chunks <= parts * per
+        assert 1 <= parts <= 65535 and (parts == 1 or per >= 4)
+        start += part
