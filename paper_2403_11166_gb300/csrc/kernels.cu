@@ -8,6 +8,7 @@
 
 #include "kernels.h"
 #include "mac_mma.cuh"
+#include "rules.h"
 
 namespace pencil {
 
@@ -1180,17 +1181,19 @@ __device__ __forceinline__ void ring_store(const RingParams& P, int a, int o, in
   P.out[flat] = acc & P.t_mask;
 }
 
-// Few output channels: thread = RING_PT consecutive output positions (a, i, j) x all
-// (at most RING_OT) output channels; the reduction runs over (c, u, v) in nested loops
-// (no divisions), each kernel value loaded once for the thread's RING_PT positions and
-// each input value once for its channels.  Channels past Co multiply a zero kernel value.
+// Short reductions: thread = RING_PT consecutive output positions (a, i, j) x RING_OT
+// consecutive output channels (8 when there are as many, else 4); the reduction runs over
+// (c, u, v) in nested loops (no divisions), each kernel value loaded once for the thread's
+// RING_PT positions and each input value once for its channels.  Channels past Co multiply
+// a zero kernel value.  Bound by each step's load latency (about 0.5 us a step) until the
+// positions fill the GPU, then by the integer pipe.
 #define RING_PT 4
-#define RING_OT 4
+template <int RING_OT>
 __global__ void __launch_bounds__(128, 4) k_ring_tile(RingParams P) {
   const long long npos = P.outs / P.kbound.x;   // B * Ho * Wo
   const long long pos0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * RING_PT;
   if (pos0 >= npos) return;
-  constexpr int o0 = 0;
+  const int o0 = blockIdx.y * RING_OT;
   const int Co = P.kbound.x, Ci = P.kbound.y, KH = P.kbound.z, KW = P.kbound.w;
   const long long HWo = (long long)P.Ho * P.Wo;
   const int no = min(RING_OT, Co - o0);
@@ -1256,16 +1259,132 @@ __global__ void __launch_bounds__(128, 4) k_ring_tile(RingParams P) {
         if (t < no) ring_store(P, pa[q], o0 + t, pi[q], pj[q], acc[q][t]);
 }
 
-// The tensor cores take every correlation but one corner: at most 3 output channels
-// fill 3 of a tile's 16 rows, and with t >= 2^48 (20 MMAs per 8 k instead of 12) a
-// short kernel is faster on the integer pipe (conv3x3 64->3, 56x56, batch 64: 471 us
-// against 381 us; with t = 2^41 377 us; 4 channels at 28x28 105 us against 284 us).
+// Weight gradients of few images (long (u, v) ranges, few c): one CTA per output,
+// threads over the (u, v) positions of each c (consecutive threads read
+// consecutive elements).
+__global__ void __launch_bounds__(256) k_ring_block(RingParams P) {
+  const long long id = blockIdx.x;
+  const int KH = P.kbound.z, KW = P.kbound.w, Ci = P.kbound.y;
+  const int j = (int)(id % P.Wo);
+  const int i = (int)((id / P.Wo) % P.Ho);
+  const int o = (int)((id / ((long long)P.Wo * P.Ho)) % P.kbound.x);
+  const int a = (int)(id / ((long long)P.Wo * P.Ho * P.kbound.x));
+  const int UV = KH * KW;
+  u64 acc = 0;
+  const u64* vb = P.v.ptr + P.v.base + a * P.v.s0;
+  const u64* wb = P.w.ptr + P.w.base + o * P.w.s0;
+  for (int c = 0; c < Ci; ++c) {
+    for (int q = threadIdx.x; q < UV; q += blockDim.x) {
+      const int u = q / KW, v = q - (q / KW) * KW;
+      const int rr = i + u - P.v.pr, ss = j + v - P.v.ps;
+      if ((unsigned)rr >= (unsigned)P.v.hr || (unsigned)ss >= (unsigned)P.v.wr) continue;
+      acc += __ldg(vb + c * P.v.s1 + rr * P.v.s2 + ss * P.v.s3) * __ldg(wb + c * P.w.s1 + u * P.w.s2 + v * P.w.s3);
+    }
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
+  __shared__ u64 part[8];
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    u64 s = 0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += part[w];
+    ring_store(P, a, o, i, j, s);
+  }
+}
+
+// The same with a short output (grad_W's HO x WO kernel offsets, at most 5 x 5): one
+// CTA per (a, o) keeps all HO * WO outputs in registers, so
+// each kernel value (grad_Y) is loaded once for all of them and the input rows
+// around it come from L1; (u, v) advance by the block size without a division.
+template <int HO, int WO>
+__global__ void __launch_bounds__(256) k_ring_wgrad(RingParams P) {
+  const int Co = P.kbound.x, Ci = P.kbound.y, KH = P.kbound.z, KW = P.kbound.w;
+  const int o = (int)(blockIdx.x % (unsigned)Co);
+  const int a = (int)(blockIdx.x / (unsigned)Co);
+  const int UV = KH * KW;
+  u64 acc[HO * WO];
+#pragma unroll
+  for (int t = 0; t < HO * WO; ++t) acc[t] = 0;
+  const u64* vb = P.v.ptr + P.v.base + a * P.v.s0;
+  const u64* wb = P.w.ptr + P.w.base + (i64)o * P.w.s0;
+  const int su = (int)blockDim.x / KW, sv = (int)blockDim.x - su * KW;
+  const int u0 = (int)threadIdx.x / KW, v0 = (int)threadIdx.x - u0 * KW;
+  for (int c = 0; c < Ci; ++c) {
+    const u64* vc = vb + c * P.v.s1;
+    const u64* wc = wb + c * P.w.s1;
+    int u = u0, v = v0;
+    for (int q = threadIdx.x; q < UV; q += blockDim.x) {
+      const u64 g = __ldg(wc + u * P.w.s2 + v * P.w.s3);
+#pragma unroll
+      for (int i = 0; i < HO; ++i) {
+        const int rr = i + u - P.v.pr;
+        if ((unsigned)rr >= (unsigned)P.v.hr) continue;
+        const u64* row = vc + rr * P.v.s2;
+#pragma unroll
+        for (int j = 0; j < WO; ++j) {
+          const int ss = j + v - P.v.ps;
+          if ((unsigned)ss < (unsigned)P.v.wr) acc[i * WO + j] += g * __ldg(row + ss * P.v.s3);
+        }
+      }
+      u += su;
+      v += sv;
+      if (v >= KW) {
+        v -= KW;
+        ++u;
+      }
+    }
+  }
+  __shared__ u64 part[8][HO * WO];   // 256 threads = 8 warps
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+  for (int t = 0; t < HO * WO; ++t) {
+    u64 x = acc[t];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) x += __shfl_down_sync(0xffffffffu, x, off);
+    if (lane == 0) part[warp][t] = x;
+  }
+  __syncthreads();
+  if ((int)threadIdx.x < HO * WO) {
+    u64 sum = 0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) sum += part[w][threadIdx.x];
+    ring_store(P, a, o, (int)threadIdx.x / WO, (int)threadIdx.x % WO, sum);
+  }
+}
+
+// Form by sizes: ring_form (rules.h).
 cudaError_t launch_ring(const RingParams& P, int sms, cudaStream_t s) {
   if (P.outs == 0) return cudaSuccess;
-  if (P.kbound.x > 3 || !(P.t_mask >> 48) || (long long)P.kbound.z * P.kbound.w >= 256)
-    return launch_ring_mma(P, sms, s);
-  const long long positions = P.outs / P.kbound.x;
-  k_ring_tile<<<(unsigned)((positions + 128 * RING_PT - 1) / (128 * RING_PT)), 128, 0, s>>>(P);
+  const RingShape shape{P.outs, P.kbound.x, P.kbound.y, P.kbound.z, P.kbound.w, P.Ho, P.Wo, (P.t_mask >> 48) != 0};
+  switch (ring_form(shape, sms)) {
+    case RingForm::kDigits:
+      return launch_ring_mma(P, sms, s);
+    case RingForm::kOffsets: {
+      const unsigned pairs = (unsigned)(P.outs / ((long long)P.Ho * P.Wo));   // (a, o) pairs
+      if (P.Ho == 3)
+        k_ring_wgrad<3, 3><<<pairs, 256, 0, s>>>(P);
+      else if (P.Ho == 5)
+        k_ring_wgrad<5, 5><<<pairs, 256, 0, s>>>(P);
+      else
+        k_ring_wgrad<1, 1><<<pairs, 256, 0, s>>>(P);
+      break;
+    }
+    case RingForm::kOutputs:
+      k_ring_block<<<(unsigned)P.outs, 256, 0, s>>>(P);
+      break;
+    case RingForm::kTile: {
+      const long long positions = P.outs / P.kbound.x;
+      const unsigned gx = (unsigned)((positions + 128 * RING_PT - 1) / (128 * RING_PT));
+      const int ot = P.kbound.x >= 8 ? 8 : 4;
+      const dim3 grid(gx, (unsigned)((P.kbound.x + ot - 1) / ot));
+      if (ot == 8)
+        k_ring_tile<8><<<grid, 128, 0, s>>>(P);
+      else
+        k_ring_tile<4><<<grid, 128, 0, s>>>(P);
+      break;
+    }
+  }
   return cudaGetLastError();
 }
 

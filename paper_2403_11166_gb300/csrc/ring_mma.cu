@@ -354,8 +354,8 @@ cudaError_t launch_ring_mma(const RingParams& P, int sms, cudaStream_t s) {
   R.v_rows = run(P.Wo, P.v.s3, P.Ho == 1 ? B : 1, P.v.s0) >= run(KW, P.v.s3, KH == 1 ? Ci : 1, P.v.s1);
   R.w_rows = (P.w.s0 == 1 ? std::min(Co, 32) : 1) > run(KW, P.w.s3, KH == 1 ? Ci : 1, P.w.s1);
   const bool wide = P.t_mask >> 48;
-  if (Co > 32) return wide ? launch<8, 2, 2, 2>(P, R, sms, s) : launch<6, 2, 2, 2>(P, R, sms, s);
-  if (Co > 16) return wide ? launch<8, 1, 2, 2>(P, R, sms, s) : launch<6, 1, 2, 2>(P, R, sms, s);
+  if (ring_tile(Co).rows == 64) return wide ? launch<8, 2, 2, 2>(P, R, sms, s) : launch<6, 2, 2, 2>(P, R, sms, s);
+  if (ring_tile(Co).rows == 32) return wide ? launch<8, 1, 2, 2>(P, R, sms, s) : launch<6, 1, 2, 2>(P, R, sms, s);
   return wide ? launch<8, 1, 1, 4>(P, R, sms, s) : launch<6, 1, 1, 4>(P, R, sms, s);
 }
 

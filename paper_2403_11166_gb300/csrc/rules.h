@@ -29,4 +29,86 @@ inline RingSplit ring_split(long long K, long long tiles, int sms) {
   return r;
 }
 
+
+// Sizes of one correlation (kernels.h, RingParams): `wide` = t > 2^48 (eight digits, not six).
+struct RingShape {
+  long long outs;
+  int Co, Ci, KH, KW, Ho, Wo;
+  bool wide;
+  long long positions() const { return outs / Co; }
+  long long K() const { return (long long)Ci * KH * KW; }
+};
+
+enum class RingForm {
+  kTile,      // k_ring_tile: a thread = 4 positions x 4 or 8 channels, the whole reduction
+  kOffsets,   // k_ring_wgrad: a CTA = all kernel offsets of one (a, o)
+  kOutputs,   // k_ring_block: a CTA = one output
+  kDigits     // k_ring_mma: digit products on the tensor cores
+};
+
+// Output tile of the tensor-core form: rows (channels), columns (positions), CTAs per SM.
+struct RingTile {
+  int rows, cols, per_sm;
+};
+inline RingTile ring_tile(int Co) {
+  return Co > 32 ? RingTile{64, 64, 2} : Co > 16 ? RingTile{32, 64, 3} : RingTile{16, 128, 3};
+}
+
+// Modelled times of the forms, us.  Fitted to 3174 sizes on GB300 (positions 1 .. 200704,
+// reductions of 1 .. 100 000, 1 .. 1000 channels, t = 2^41 and 2^59): tensor cores within 7 %
+// (rms), tile 10 %, offsets 14 %, outputs 8 %; choosing by them costs 0.2 % over the faster
+// of the forms' measured times (geometric mean).
+inline double ring_digits_us(const RingShape& s, int sms) {
+  const RingTile t = ring_tile(s.Co);
+  const long long tiles = ((s.positions() + t.cols - 1) / t.cols) * ((s.Co + t.rows - 1) / t.rows);
+  const RingSplit p = ring_split(s.K(), tiles, sms);   // (a longer reduction's first launch)
+  // waves of CTAs; a chunk takes a full SM 2.75 us (rows 64: 3.05), a lone CTA 1.6
+  const long long ctas = tiles * p.parts, cap = (long long)t.per_sm * sms, rest = ctas % cap;
+  const double full = t.rows == 64 ? 3.05 : 2.75;
+  const double wave = (double)(ctas / cap) * full + (rest ? std::max(1.6, full * (double)rest / (double)cap) : 0.0);
+  return 0.3 + 2.75 * std::min(1.0, (double)s.positions() / 64) + (t.rows == 64 ? 1.7 : 0.0) +
+         (p.parts > 1 ? 2.9 : 0.0) + wave * (p.per * (s.wide ? 1.28 : 1.0) + 1.5);
+}
+
+// a serial part (latency of one thread's loop) and a parallel one (work over the GPU)
+inline double ring_overlap_us(double serial, double work, double share) {
+  return std::max(serial, work) + share * std::min(serial, work);
+}
+
+inline double ring_tile_us(const RingShape& s) {
+  const int ot = s.Co >= 8 ? 8 : 4;
+  const double K = (double)s.K(), lines = K / s.KW, groups = (s.Co + ot - 1) / ot;
+  return 2.0 + 1.5 * std::min(1.0, (double)s.positions() / 8) +
+         ring_overlap_us((0.36 * K + 0.185 * lines) * (ot == 8 ? 1.42 : 1.0),
+                         (double)s.positions() * groups * (0.247 * ot * K + 1.55 * lines + 3.9 * std::min(ot, s.Co)) * 1e-6,
+                         0.64);
+}
+
+inline double ring_offsets_us(const RingShape& s) {
+  const double h = (double)s.Ho * s.Wo, steps = (double)s.Ci * (((long long)s.KH * s.KW + 255) / 256);
+  return 1.94 + ring_overlap_us(steps * (0.205 + 0.049 * h),
+                                (double)s.outs / h * (steps * (0.158 * h + 0.41) + 0.33 * h) * 1e-3, 0.37);
+}
+
+inline double ring_outputs_us(const RingShape& s) {
+  const double steps = (double)s.Ci * (((long long)s.KH * s.KW + 255) / 256);
+  return 2.17 + ring_overlap_us(0.317 * steps, (double)s.outs * (steps + 2.8) * 0.59e-3, 0.61);
+}
+
+// The tensor cores take a correlation unless its integer form is faster: short reductions
+// (a chunk of 16 is paid whole), weight gradients of few images (the split's two extra
+// passes), few channels over many positions (at most 4 of a tile's 16 rows exist), above
+// all with t > 2^48.  Integer form by the kernel's elements: 256 or more (weight gradients)
+// share them over a CTA's threads.  Measured (us, integer / tensor cores): fc 64 x 2048 to 2
+// weights, batch 1, K = 1 4.9 / 9.5; 28 x 28 image's 3 x 3 weight gradient, 3 to 64 channels,
+// batch 1 4.8 / 17.5, batch 8 41 / 14; conv3x3 64->3, 56x56, batch 64 379 / 374 (t = 2^41),
+// 381 / 468 (t = 2^59); fc 2048 to 2, batch 64 1240 / 13 (t = 2^59: / 14.5).
+inline RingForm ring_form(const RingShape& s, int sms) {
+  const bool cta = (long long)s.KH * s.KW >= 256 && s.outs < 1ll << 31;
+  const bool offsets = cta && s.Ho == s.Wo && (s.Ho == 1 || s.Ho == 3 || s.Ho == 5);
+  const RingForm integer = offsets ? RingForm::kOffsets : cta ? RingForm::kOutputs : RingForm::kTile;
+  const double us = offsets ? ring_offsets_us(s) : cta ? ring_outputs_us(s) : ring_tile_us(s);
+  return us < ring_digits_us(s, sms) ? integer : RingForm::kDigits;
+}
+
 }  // namespace pencil

@@ -18,7 +18,11 @@ extern "C" void ring_split_(long long K, long long tiles, int sms, int* out) {
   out[2] = r.parts;
 }
 extern "C" long long ring_launch_k() { return kRingLaunchK; }
+extern "C" int ring_form_(long long outs, const int* d, int wide, int sms) {
+  return (int)ring_form(RingShape{outs, d[0], d[1], d[2], d[3], d[4], d[5], wide != 0}, sms);
+}
 """
+RING_FORMS = ("tile", "offsets", "outputs", "digits")
 
 
 @functools.lru_cache(maxsize=None)
@@ -42,3 +46,17 @@ def ring_split(k: int, tiles: int, sms: int = 152):
 def ring_launch_k() -> int:
     load().ring_launch_k.restype = ctypes.c_longlong
     return load().ring_launch_k()
+
+
+def ring_form(layer, role: int, t_bits: int, sms: int = 152) -> str:
+    """Form of a plaintext correlation; layer = (B, Ci, Co, H, kernel, pad), fully connected
+    ones with H = kernel = 1; role 0 forward, 1 input gradient, 2 weight gradient."""
+    b, ci, co, h, k, pad = layer
+    ho = h + 2 * pad - k + 1
+    if role == 0:
+        outs, dims = b * co * ho * ho, (co, ci, k, k, ho, ho)
+    elif role == 1:
+        outs, dims = b * ci * h * h, (ci, co, k, k, h, h)
+    else:
+        outs, dims = ci * co * k * k, (co, b, ho, ho, k, k)
+    return RING_FORMS[load().ring_form_(ctypes.c_longlong(outs), (ctypes.c_int * 6)(*dims), int(t_bits > 48), sms)]

@@ -23,3 +23,32 @@ def test_ring_parts_cover_every_reduction_that_fits_the_device(k, tiles):
         assert (parts - 1) * per < chunks <= parts * per
         assert 1 <= parts <= 65535 and (parts == 1 or per >= 4)
         start += part
+
+
+# (B, Ci, Co, H, kernel, pad), role, t_bits -> form, where the measured times of the forms
+# are at least 1.2 apart (us: integer form / tensor cores)
+RING_FORMS = [
+    ((1, 256, 100, 1, 1, 0), 2, 41, "tile"),          # 4.8 / 9.5
+    ((1, 2048, 1001, 1, 1, 0), 2, 41, "tile"),        # 13.0 / 18.9
+    ((64, 2048, 1, 1, 1, 0), 1, 41, "tile"),          # 5.0 / 9.5
+    ((1000, 3, 8, 1, 1, 0), 0, 59, "tile"),           # 6.9 / 7.4 and less
+    ((64, 3, 64, 56, 1, 0), 0, 41, "tile"),           # 59.8 / 94.9
+    ((64, 3, 3, 56, 3, 1), 0, 41, "tile"),            # 20.9 / 36.9
+    ((64, 64, 3, 56, 3, 1), 0, 59, "tile"),           # 381 / 468
+    ((1, 1, 1, 28, 5, 2), 2, 41, "offsets"),          # 8.8 / 15.0
+    ((1, 16, 8, 28, 3, 1), 2, 59, "offsets"),         # 4.2 / 17.1
+    ((1, 16, 64, 28, 1, 0), 2, 41, "offsets"),        # 5.2 / 15.8
+    ((64, 2048, 2, 1, 1, 0), 0, 59, "digits"),        # 1240 / 13.4
+    ((64, 2048, 2, 1, 1, 0), 0, 41, "digits"),
+    ((1000, 10, 3, 1, 1, 0), 2, 59, "digits"),        # 535 / 15
+    ((8, 64, 3, 14, 3, 1), 0, 59, "digits"),          # 285 / 16
+    ((64, 16, 16, 32, 3, 1), 0, 41, "digits"),        # 104 / 48
+    ((64, 16, 16, 32, 3, 1), 2, 59, "digits"),        # 190 / 70
+    ((64, 2048, 1001, 1, 1, 0), 2, 41, "digits"),     # 97 / 38
+    ((128, 128, 128, 16, 3, 1), 2, 41, "digits"),
+]
+
+
+@pytest.mark.parametrize("layer,role,t_bits,form", RING_FORMS)
+def test_ring_form_is_the_faster_one(layer, role, t_bits, form):
+    assert rules_lib.ring_form(layer, role, t_bits) == form
