@@ -111,4 +111,8 @@ inline RingForm ring_form(const RingShape& s, int sms) {
   return us < ring_digits_us(s, sms) ? integer : RingForm::kDigits;
 }
 
+// CTAs (one cluster) per channel of a bias gradient over `elements` each: one takes 16
+// elements a thread; a cluster's launch costs as much.
+inline int bias_parts(long long elements) { return elements > 4096 ? 8 : 1; }
+
 }  // namespace pencil

@@ -21,6 +21,7 @@ extern "C" long long ring_launch_k() { return kRingLaunchK; }
 extern "C" int ring_form_(long long outs, const int* d, int wide, int sms) {
   return (int)ring_form(RingShape{outs, d[0], d[1], d[2], d[3], d[4], d[5], wide != 0}, sms);
 }
+extern "C" int bias_parts_(long long elements) { return bias_parts(elements); }
 """
 RING_FORMS = ("tile", "offsets", "outputs", "digits")
 

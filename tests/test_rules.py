@@ -1,4 +1,6 @@
 """Launch rules (csrc/rules.h) on the host."""
+import ctypes
+
 import pytest
 
 from tests import rules_lib
@@ -52,3 +54,8 @@ RING_FORMS = [
 @pytest.mark.parametrize("layer,role,t_bits,form", RING_FORMS)
 def test_ring_form_is_the_faster_one(layer, role, t_bits, form):
     assert rules_lib.ring_form(layer, role, t_bits) == form
+
+
+def test_a_small_bias_gradient_is_no_cluster_launch():
+    parts = rules_lib.load().bias_parts_
+    assert [parts(ctypes.c_longlong(n)) for n in (1, 4096, 4097, 1 << 40)] == [1, 1, 8, 8]
