@@ -1465,8 +1465,10 @@ cudaError_t launch_bias_grad(const u64* g, int B, int Co, long long hw, u64 t_ma
 // exact mod t):  out[e] = addend[e] (+ or -) sum_{i2, i} k[i2 terms + i]
 // src[off + (e / inner) outer + e % inner + i tstride + i2 tstride2].
 // Bound by memory (64 terms: 64 words read per word written); a thread takes V
-// consecutive elements (V = 2, 16-byte accesses, when every offset and stride is even
-// and the tensors are 16-byte aligned) with eight terms' loads in flight.
+// consecutive elements (V = 2, 16-byte accesses, for launches that fill the GPU with them
+// when every offset and stride is even and the tensors are 16-byte aligned) with eight
+// terms' loads in flight (four terms, 1000 elements: 1.9 us; with the last terms one by one
+// 2.5; 2^22 elements 31 / 35).
 template <int V>
 __global__ void __launch_bounds__(256) k_lincomb(const __grid_constant__ LincombP P, u64 t_mask) {
   const long long stride = (long long)gridDim.x * blockDim.x * V;
@@ -1484,16 +1486,31 @@ __global__ void __launch_bounds__(256) k_lincomb(const __grid_constant__ Lincomb
     for (int i2 = 0; i2 < P.terms2; ++i2) {
       const u64* src = base + i2 * P.tstride2;
       const u64* k = P.k + i2 * P.terms;
-#pragma unroll 8
-      for (int i = 0; i < P.terms; ++i) {
-        if constexpr (V == 2) {
-          const ulonglong2 x = __ldg(reinterpret_cast<const ulonglong2*>(src + i * P.tstride));
-          acc0 += k[i] * x.x;
-          acc1 += k[i] * x.y;
-        } else {
-          acc0 += k[i] * __ldg(src + i * P.tstride);
+      // groups of eight terms, then of four, two and one: every load of a group is in flight at once
+      int i = 0;
+      auto group = [&](auto size) {
+        constexpr int G = decltype(size)::value;
+        ulonglong2 x[G];
+#pragma unroll
+        for (int j = 0; j < G; ++j) {
+          const u64* at = src + (i + j) * P.tstride;
+          if constexpr (V == 2)
+            x[j] = __ldg(reinterpret_cast<const ulonglong2*>(at));
+          else
+            x[j].x = __ldg(at);
         }
-      }
+#pragma unroll
+        for (int j = 0; j < G; ++j) {
+          acc0 += k[i + j] * x[j].x;
+          if constexpr (V == 2) acc1 += k[i + j] * x[j].y;
+        }
+        i += G;
+      };
+#pragma unroll 1
+      while (i + 8 <= P.terms) group(std::integral_constant<int, 8>{});
+      if (P.terms & 4) group(std::integral_constant<int, 4>{});
+      if (P.terms & 2) group(std::integral_constant<int, 2>{});
+      if (P.terms & 1) group(std::integral_constant<int, 1>{});
     }
     if (P.negate) {
       acc0 = 0 - acc0;
@@ -1518,7 +1535,7 @@ cudaError_t launch_lincomb(const LincombP& P, u64 t_mask, cudaStream_t s) {
   const long long all = P.off | P.inner | P.outer | P.count | P.tstride | P.tstride2;
   const uintptr_t ptrs = reinterpret_cast<uintptr_t>(P.src) | reinterpret_cast<uintptr_t>(P.out) |
                          reinterpret_cast<uintptr_t>(P.addend);
-  const bool pairs = !(all & 1) && !(ptrs & 15);
+  const bool pairs = lincomb_pairs(P.count) && !(all & 1) && !(ptrs & 15);
   const long long blocks = std::min<long long>((P.count + (pairs ? 511 : 255)) / (pairs ? 512 : 256), 152LL * 16);
   if (pairs)
     k_lincomb<2><<<(unsigned)blocks, 256, 0, s>>>(P, t_mask);

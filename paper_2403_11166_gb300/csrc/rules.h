@@ -115,4 +115,10 @@ inline RingForm ring_form(const RingShape& s, int sms) {
 // elements a thread; a cluster's launch costs as much.
 inline int bias_parts(long long elements) { return elements > 4096 ? 8 : 1; }
 
+// Whether a linear combination's threads take two elements each (where everything is
+// aligned for it): below, twice the threads hide more latency (us, one / two: 65536 elements
+// of 64 terms 5.2 / 5.7, of 4 2.2 / 2.2; 150 000 6.8 / 6.7 and 2.5 / 2.4; 2^20 81.2 / 80.3 and
+// 6.6 / 5.1).
+inline bool lincomb_pairs(long long count) { return count >= 1 << 17; }
+
 }  // namespace pencil

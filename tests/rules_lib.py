@@ -22,6 +22,7 @@ extern "C" int ring_form_(long long outs, const int* d, int wide, int sms) {
   return (int)ring_form(RingShape{outs, d[0], d[1], d[2], d[3], d[4], d[5], wide != 0}, sms);
 }
 extern "C" int bias_parts_(long long elements) { return bias_parts(elements); }
+extern "C" int lincomb_pairs_(long long count) { return lincomb_pairs(count); }
 """
 RING_FORMS = ("tile", "offsets", "outputs", "digits")
 
@@ -61,3 +62,7 @@ def ring_form(layer, role: int, t_bits: int, sms: int = 152) -> str:
     else:
         outs, dims = ci * co * k * k, (co, b, ho, ho, k, k)
     return RING_FORMS[load().ring_form_(ctypes.c_longlong(outs), (ctypes.c_int * 6)(*dims), int(t_bits > 48), sms)]
+
+
+def lincomb_pairs(count: int) -> bool:
+    return bool(load().lincomb_pairs_(ctypes.c_longlong(count)))

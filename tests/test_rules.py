@@ -59,3 +59,7 @@ def test_ring_form_is_the_faster_one(layer, role, t_bits, form):
 def test_a_small_bias_gradient_is_no_cluster_launch():
     parts = rules_lib.load().bias_parts_
     assert [parts(ctypes.c_longlong(n)) for n in (1, 4096, 4097, 1 << 40)] == [1, 1, 8, 8]
+
+
+def test_small_linear_combinations_take_one_element_a_thread():
+    assert not rules_lib.lincomb_pairs(100000) and rules_lib.lincomb_pairs(1 << 17)
