@@ -405,10 +405,8 @@ struct Window {
     return has(ent) ? __ldg(reinterpret_cast<const u64*>(at(ent))) : 0ull;
   }
   // element index of coefficient e in the operand's tensor (null ptr), or -1
-  __device__ __forceinline__ i64 index(const Packing& pk, int e) const {
-    const ulonglong2 ent = __ldg(pk.tab + e);
-    return has(ent) ? (i64)at(ent) >> 3 : -1;
-  }
+  __device__ __forceinline__ i64 index(const ulonglong2& ent) const { return has(ent) ? (i64)at(ent) >> 3 : -1; }
+  __device__ __forceinline__ i64 index(const Packing& pk, int e) const { return index(__ldg(pk.tab + e)); }
 };
 
 // Decryption's CRT step: with y_j = x_j (q/q_j)^{-1} mod q_j,

@@ -974,25 +974,43 @@ cudaError_t launch_sample_pk(u64 seed, int first, int count, int n, int8_t* e1, 
 // one per coefficient before that).  Here the CTA lists its different blocks once, draws
 // them one per thread and hands the words out through shared memory: about 1.3 blocks per
 // thread where rows are 28 elements and a gap of 2 (1920 polynomials of 28 x 19 tiles at
-// N = 8192: 163 -> 112 us; 160 of 32 x 32 tiles 20 -> 16; polynomials that are nearly all
-// padding, whose blocks no two threads share, pay for the list: three launches of a 128 to
-// 128 channel layer's forward and gradients 338 -> 369).
+// N = 8192: 241 -> 120 us; 160 of 32 x 32 tiles 21 -> 17).  A warp without outputs lists
+// nothing and needs no window: each thread draws its padding block.  Three launches of a 128
+// to 128 channel layer's forward and gradients, whose polynomials are 75 to 99 % padding: 344
+// us drawn by each thread, 376 with every block listed, 330.  What still loses to drawing by
+// each thread: outputs at stride (no two neighbours share a block; 513 polynomials of a fully
+// connected layer's weight gradient 47 -> 57 us) and dense aligned rows (13 -> 14).  At least
+// five or six CTAs per SM (48 or 40 registers instead of 56): spills, 1.1 to 1.4x.
 #define MASK_POLY_LIST 512   // blocks drawn at a time (of at most 256 + 1024): 20 KB, eight CTAs per SM
-__device__ __forceinline__ void mask_poly_block(const DevCtx& ctx, const Packing& pk, const Window& win, u64 seed,
+__device__ __forceinline__ void mask_poly_block(const DevCtx& ctx, const Packing& pk, const Accessor& ac, u64 seed,
                                                 int ct, int blk, u64* out_ct) {
   __shared__ i64 src[MASK_POLY_LIST];   // element block, or -1 - (block of the padding stream)
   __shared__ __align__(16) u64 word[MASK_POLY_LIST][4];
   __shared__ int warp_total[8];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  i64 key[4];
+  i64 key[4] = {-1, -1, -1, -1};
   u32 sub = 0, lead = 0;   // flat % 4 (two bits each); first coefficient of a run on one block
   bool pad = false;
+  ulonglong2 ent[4];
+  bool none = true;
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const i64 flat = win.index(pk, 4 * blk + i);
-    key[i] = flat >> 2;   // (-1: no output)
-    sub |= (u32)(flat & 3) << (2 * i);
-    pad = pad || flat < 0;
+    ent[i] = __ldg(pk.tab + 4 * blk + i);
+    none = none && ent[i].x == PENCIL_TAB_NONE;
+  }
+  const bool empty = __all_sync(0xffffffffu, none);   // no outputs in the warp: nothing to list
+  Philox4 r = {{0, 0, 0, 0}};
+  if (empty) {
+    r = philox4x64((u64)blk, (u64)ct, 0ull, 0ull, seed, PENCIL_DOM_MASK_PAD);
+  } else {
+    const Window win(pk, ac, ct, nullptr);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const i64 flat = win.index(ent[i]);
+      key[i] = flat >> 2;   // (-1: no output)
+      sub |= (u32)(flat & 3) << (2 * i);
+      pad = pad || flat < 0;
+    }
   }
   // a run (at most four coefficients: elements of a polynomial differ) may continue the
   // previous lane's; its first lane lists it
@@ -1024,7 +1042,6 @@ __device__ __forceinline__ void mask_poly_block(const DevCtx& ctx, const Packing
     const int n = __popc(lead & ((2u << i) - 1u));
     at[i] = key[i] < 0 ? base : n ? base + (pad ? 1 : 0) + n - 1 : base - 1;
   }
-  Philox4 r = {{0, 0, 0, 0}};
   for (int c0 = 0; c0 < total; c0 += MASK_POLY_LIST) {   // (once, but for widely strided outputs)
     if (pad && (unsigned)(base - c0) < MASK_POLY_LIST) src[base - c0] = -1 - (i64)blk;
 #pragma unroll
@@ -1041,7 +1058,7 @@ __device__ __forceinline__ void mask_poly_block(const DevCtx& ctx, const Packing
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < 4; ++i)
-      if ((unsigned)(at[i] - c0) < MASK_POLY_LIST)
+      if (!empty && (unsigned)(at[i] - c0) < MASK_POLY_LIST)
         r.v[i] = word[at[i] - c0][key[i] < 0 ? (u32)i : sub >> (2 * i) & 3u];
   }
   ulonglong2* o = reinterpret_cast<ulonglong2*>(out_ct + 4 * blk);
@@ -1054,7 +1071,7 @@ __global__ void __launch_bounds__(256) k_mask_poly(const __grid_constant__ DevCt
                                                    const __grid_constant__ Accessor ac, u64 seed, u64* out) {
   const int lg = ctx.log_n - 10, ct = blockIdx.x >> lg;
   const int blk = ((int)(blockIdx.x & ((1u << lg) - 1u)) << 8) + threadIdx.x;
-  mask_poly_block(ctx, pk, Window(pk, ac, ct, nullptr), seed, ct, blk, out + ((size_t)ct << ctx.log_n));
+  mask_poly_block(ctx, pk, ac, seed, ct, blk, out + ((size_t)ct << ctx.log_n));
 }
 
 cudaError_t launch_mask_poly(const DevCtx& ctx, const Packing& pk, const Accessor& ac, u64 seed, int count, u64* out,
@@ -1577,7 +1594,7 @@ __global__ void __launch_bounds__(256) k_mask_poly_multi(const __grid_constant__
   const int blk = ((int)(blockIdx.x & ((1u << lg) - 1u)) << 8) + threadIdx.x;
   const MaskPolyP& P = Ps[it.x];
   const u64 seed = P.seed + ((step ? *step : 0ull) << 32);
-  mask_poly_block(ctx, P.pk, Window(P.pk, P.ac, it.y, nullptr), seed, it.y, blk, P.out + ((size_t)it.y << ctx.log_n));
+  mask_poly_block(ctx, P.pk, P.ac, seed, it.y, blk, P.out + ((size_t)it.y << ctx.log_n));
 }
 
 __global__ void k_mo_share_multi(const MoShareP* __restrict__ Ps, const int2* __restrict__ items, long long n_items,
