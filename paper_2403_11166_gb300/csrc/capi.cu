@@ -211,7 +211,7 @@ struct PencilPlan {
   Accessor acc_v, acc_w, acc_y;  // ptr filled per call
   long long hw;                  // output spatial size (bias broadcast)
   int co_out;                    // output channel count seen by the bias
-  ulonglong2* d_tab = nullptr;   // [3][N]: v, w, y tables (Packing)
+  ulonglong2* d_tab = nullptr;   // [3][N]: v, w, y tables, then their [3][N / 32] groups (Packing)
   int4* d_org = nullptr;         // origins: v [ct_in], w [pt], y [ct_out]
   Packing pk_v, pk_w, pk_y;
   long long ws_encrypt, ws_forward, ws_backward, ws_decrypt, ws_encrypt_pk;
@@ -863,8 +863,10 @@ extern "C" int pencil_plan_linear(PencilCtx* ctx, const PencilLayerDesc* layer, 
   }
   DeviceGuard guard(ctx->device);
   // beside the coordinates, the byte offset they give in the operand's tensor
-  std::vector<ulonglong2> tab2(tab.size());
+  std::vector<ulonglong2> tab2(tab.size() + tab.size() / 32 / sizeof(ulonglong2), make_ulonglong2(0, 0));
+  unsigned char* groups = reinterpret_cast<unsigned char*>(tab2.data() + tab.size());
   for (size_t i = 0; i < tab.size(); ++i) {
+    if (tab[i] != PENCIL_TAB_NONE) groups[i / 32] = 1;
     const Accessor& ac = i < (size_t)n ? P->acc_v : i < 2 * (size_t)n ? P->acc_w : P->acc_y;
     const u64 x = tab[i];
     const i64 off = x == PENCIL_TAB_NONE ? 0
@@ -886,10 +888,12 @@ extern "C" int pencil_plan_linear(PencilCtx* ctx, const PencilLayerDesc* layer, 
         support[sgm] = e + 1;
         break;
       }
-  P->pk_v = Packing{P->d_tab, P->d_org, make_int4(g.B, g.Ci, g.H, g.W), support[0]};
-  P->pk_w = Packing{P->d_tab + n, P->d_org + P->ct_in, make_int4(g.Co, g.Ci, g.KH, g.KW), support[1]};
+  const unsigned char* d_groups = reinterpret_cast<const unsigned char*>(P->d_tab + 3 * (size_t)n);
+  P->pk_v = Packing{P->d_tab, P->d_org, make_int4(g.B, g.Ci, g.H, g.W), support[0], d_groups};
+  P->pk_w = Packing{P->d_tab + n, P->d_org + P->ct_in, make_int4(g.Co, g.Ci, g.KH, g.KW), support[1],
+                    d_groups + n / 32};
   P->pk_y = Packing{P->d_tab + 2 * (size_t)n, P->d_org + P->ct_in + P->pt, make_int4(g.B, g.Co, g.Ho(), g.Wo()),
-                    support[2]};
+                    support[2], d_groups + 2 * (n / 32)};
 
   // --- workspace sizes (bytes, each region 256-byte aligned)
   auto al = [](long long b) { return (b + 255) / 256 * 256; };

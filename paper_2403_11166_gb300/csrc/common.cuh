@@ -82,6 +82,7 @@ struct Packing {
   const int4* org;
   int4 bound;
   int support;
+  const unsigned char* groups;   // [N / 32]: whether any of 32 consecutive coefficients has an entry
 };
 
 #define PENCIL_TAB_NONE 0x7FFF7FFF7FFF7FFFull
