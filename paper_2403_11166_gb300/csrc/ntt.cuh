@@ -1491,6 +1491,14 @@ inline bool many_small(const DevCtx& ctx, long long count, bool inverse) {
   return count * ctx.L > (inverse ? 4ll : 3ll) * ctx.sms;
 }
 
+// Whether a launch of 512-thread transforms (N = 8192, radix 2^4) that gives no SM two of them
+// is compiled for one CTA per SM, with up to 128 registers a thread instead of 64: there is
+// no second CTA whose warps hide a transform's latency (us, two per SM / one: raw forward 75
+// transforms 11.7 / 10.9, 120 11.8 / 10.9; raw inverse 120 12.4 / 12.0; encryption 96 23.5 /
+// 22.7; decryption 120 18.7 / 18.1; compact form 120 14.6 / 13.5; 240 transforms, two on an
+// SM, forward 19.9 / 20.6).
+inline bool lone(const DevCtx& ctx, long long count) { return count * ctx.L <= ctx.sms; }
+
 // Host-side launcher; explicitly instantiated per LOGN and engine in ntt12.cu /
 // ntt13.cu / ntt14.cu (Shoup) and ntt12f.cu / ntt13f.cu / ntt14f.cu (split products).
 template <int LOGN, int LOGE, class Mode, bool INV, bool FOLD>
@@ -1527,6 +1535,14 @@ cudaError_t launch_ntt(const DevCtx& ctx, const typename Mode::Params& P, int fi
         return launch(k_ntt_inv<LOGN, LOGE, Mode, FOLD, 4>);
       else
         return launch(k_ntt_fwd<LOGN, LOGE, Mode, FOLD, 4>);
+    }
+  }
+  if constexpr (FOLD && LOGN == 13 && LOGE == 4) {
+    if (lone(ctx, count)) {
+      if constexpr (INV)
+        return launch(k_ntt_inv<LOGN, LOGE, Mode, FOLD, 1>);
+      else
+        return launch(k_ntt_fwd<LOGN, LOGE, Mode, FOLD, 1>);
     }
   }
   if constexpr (INV)
