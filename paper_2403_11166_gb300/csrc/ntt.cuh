@@ -1409,11 +1409,13 @@ struct ModeDecrypt {
   static __device__ __forceinline__ u64 load(const DevCtx& c, const Params& P, const Pre& pre, const LimbConst& lc, int poly,
                                              int limb, int e) {
     const u64 c1 = __ldg(P.ct + ct_off(poly, 1, limb, c.L, N) + e);
-    if constexpr (SPLIT) {   // c0 + c1 s in [-0.6, 2.6], folded; c1 s alone is in range
+    if constexpr (SPLIT) {   // c0 + c1 s in [-0.6, 2.6], folded
       const FoldC f(lc);
       const uint4 s = __ldg(reinterpret_cast<const uint4*>(P.sk) + (size_t)(c.L + limb) * N + e);
-      if (P.skip_c0) return mul_split(0, c1, s, f);
-      return fold_s(mul_split(__ldg(P.ct + ct_off(poly, 0, limb, c.L, N) + e), c1, s, f), f);
+      // one product for both forms: a branch around a second one kept the loads of different
+      // words apart (256 polynomials at N = 8192 with radix 2^5: 125 us, 89 like this)
+      const u64 c0 = P.skip_c0 ? 0 : __ldg(P.ct + ct_off(poly, 0, limb, c.L, N) + e);
+      return fold_s(mul_split(c0, c1, s, f), f);
     }
     const ulonglong2 s = __ldg(P.sk + (size_t)limb * N + e);
     const u64 c1s = mul_shoup(c1, s.x, s.y, lc.q);
