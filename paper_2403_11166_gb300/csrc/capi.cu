@@ -15,6 +15,7 @@
 
 #include "../../include/pencil_he.h"
 #include "kernels.h"
+#include "rules.h"
 
 using namespace pencil;
 typedef unsigned __int128 u128;
@@ -94,18 +95,9 @@ static u64 min_root_2n(u64 q, u64 two_n) {
 
 static u64 shoup(u64 w, u64 q) { return (u64)(((u128)w << 64) / q); }
 
-// Split twiddle of mul_split (common.cuh), q = 2^b - c with b = bit length of q: the
-// centred representatives of w and w 2^32 mod q, each as (low b - 32 bits, signed rest).
 static uint4 split_twiddle(u64 w, u64 q) {
-  const int sh = 32 - __builtin_clzll(q);
-  u32 out[4];
-  const u64 v[2] = {w, (u64)(((u128)w << 32) % q)};
-  for (int i = 0; i < 2; ++i) {
-    const i64 x = v[i] > q / 2 ? (i64)v[i] - (i64)q : (i64)v[i];
-    out[2 * i] = (u32)((u64)x & ((1ull << sh) - 1));
-    out[2 * i + 1] = (u32)(int32_t)(x >> sh);
-  }
-  return make_uint4(out[0], out[1], out[2], out[3]);
+  const SplitWords s = split_words(w, q);
+  return make_uint4(s.v[0], s.v[1], s.v[2], s.v[3]);
 }
 
 static unsigned brv(unsigned x, int bits) {
@@ -180,12 +172,12 @@ struct PencilCtx {
 
 struct PencilSecretKey {
   PencilCtx* ctx;
-  ulonglong2* sk = nullptr;   // [L][N] (value, Shoup companion), then [L][N] split twiddles (uint4)
+  ulonglong2* sk = nullptr;   // [L][N] (value, Shoup companion), then (key_forms) [L][N] split twiddles (uint4)
 };
 
 struct PencilPublicKey {
   PencilCtx* ctx;
-  ulonglong2* key = nullptr;   // [2][L][N] (value, Shoup companion), [2][L][N] split twiddles, N bytes of scratch
+  ulonglong2* key = nullptr;   // [2][L][N] (value, Shoup companion), (key_forms) [2][L][N] split twiddles, N bytes of scratch
 };
 
 struct Geom {
@@ -316,14 +308,12 @@ extern "C" int pencil_ctx_create(const PencilParams* params, int device, PencilC
   d.t_bits = p.t_bits;
   d.t_mask = (1ull << p.t_bits) - 1;
   std::vector<ulonglong2> tf((size_t)d.L * n), ti((size_t)d.L * n);
-  // split butterflies (mul_split) need q_j = 2^b - c with c < 2^24 (b = 59, 60) or
-  // c < 2^(b-33) for every limb; the arithmetic knob is open for b = 60 only
+  // split butterflies need a split_prime for every limb; the arithmetic knob is open for
+  // 60-bit ones only
   bool fold_ok = true, fold60 = true;
   for (u64 q : qs) {
-    const int b = 64 - __builtin_clzll(q);
-    const u64 c = (1ull << b) - q;
-    fold_ok = fold_ok && b >= 40 && c < (b >= 59 ? 1ull << 24 : 1ull << (b - 33));
-    fold60 = fold60 && b == 60 && c < (1ull << 24);
+    fold_ok = fold_ok && split_prime(q);
+    fold60 = fold60 && split_prime(q) && bit_length(q) == 60;
   }
   ctx->arith_knob = fold60;
   std::vector<uint4> tff(fold_ok ? (size_t)d.L * n : 0), tif(fold_ok ? (size_t)d.L * n : 0);
@@ -351,7 +341,7 @@ extern "C" int pencil_ctx_create(const PencilParams* params, int device, PencilC
     lc.ninvs = shoup(lc.ninv, q);
     lc.delta = delta_mod(qs, p.t_bits, q);
     lc.deltas = shoup(lc.delta, q);
-    lc.delta_sp = split_twiddle(lc.delta, q);
+    lc.delta_sp = fold_ok ? split_twiddle(lc.delta, q) : make_uint4(0, 0, 0, 0);
     u64 qt = 1;
     for (int i = 0; i < d.L; ++i)
       if (i != j) qt = mulmod(qt, qs[i] % q, q);
@@ -365,8 +355,8 @@ extern "C" int pencil_ctx_create(const PencilParams* params, int device, PencilC
     lc.nqtil = mulmod(lc.ninv, lc.qtil, q);
     lc.nqtils = shoup(lc.nqtil, q);
     lc.a_max = (u64)((((u128)1) << 64) / q * q - 1);
-    lc.sb = 32 - (u32)__builtin_clzll(q);
-    lc.cb = (1ull << (64 - __builtin_clzll(q))) - q;
+    lc.sb = (u32)std::max(0, bit_length(q) - 32);   // (shorter primes take neither form)
+    lc.cb = (1ull << bit_length(q)) - q;
     {   // bias of one combination of diagonals (digits.cuh): 0x33000000 sum_{j < 7} 2^(16 j)
       u64 bias = 0, w = 0x33000000ull % q;
       for (int i = 0; i < 7; ++i) {
@@ -531,6 +521,10 @@ extern "C" int pencil_sync_status(PencilCtx* ctx, int32_t* status) {
 }
 
 // ================================================================== keys
+// Forms a key's values are kept in: with Shoup companions, and as split twiddles in
+// contexts that have the split butterflies (whatever the arithmetic knob says at the time).
+static size_t key_forms(const PencilCtx* ctx) { return ctx->dev.tw_fwd_f ? 2 : 1; }
+
 extern "C" int pencil_keygen(PencilCtx* ctx, uint64_t seed, PencilSecretKey** out, void* stream) {
   if (!ctx || !out) return PENCIL_E_ARG;
   *out = nullptr;
@@ -538,7 +532,7 @@ extern "C" int pencil_keygen(PencilCtx* ctx, uint64_t seed, PencilSecretKey** ou
   PencilSecretKey* sk = new (std::nothrow) PencilSecretKey();
   if (!sk) return PENCIL_E_CUDA;
   sk->ctx = ctx;
-  if (cudaMalloc(&sk->sk, 2ull * ctx->dev.L * ctx->n * sizeof(ulonglong2)) != cudaSuccess) {
+  if (cudaMalloc(&sk->sk, key_forms(ctx) * ctx->dev.L * ctx->n * sizeof(ulonglong2)) != cudaSuccess) {
     delete sk;
     return PENCIL_E_CUDA;
   }
@@ -569,7 +563,7 @@ extern "C" int pencil_pk_keygen(PencilCtx* ctx, const PencilSecretKey* sk, uint6
   PencilPublicKey* pk = new (std::nothrow) PencilPublicKey();
   if (!pk) return PENCIL_E_CUDA;
   pk->ctx = ctx;
-  const size_t key_bytes = 4ull * ctx->dev.L * ctx->n * sizeof(ulonglong2);
+  const size_t key_bytes = 2 * key_forms(ctx) * ctx->dev.L * ctx->n * sizeof(ulonglong2);
   if (cudaMalloc(&pk->key, key_bytes + ctx->n) != cudaSuccess) {
     delete pk;
     return PENCIL_E_CUDA;

@@ -1207,10 +1207,12 @@ __device__ __forceinline__ u64 shoup_companion(u64 w, u64 q) {
   return (u64)((((unsigned __int128)w) << 64) / q);
 }
 
-// Word `at` of a key of `rows` x n values in both product forms: with its Shoup
-// companion, and as a split twiddle behind all of those (mul_split).
-__device__ __forceinline__ void put_key(ulonglong2* key, int rows, size_t at, int n, u64 x, const LimbConst& lc) {
+// Word `at` of a key of `rows` x n values: with its Shoup companion and, in contexts that
+// have the split butterflies, as a split twiddle behind all of those (mul_split).
+__device__ __forceinline__ void put_key(const DevCtx& c, ulonglong2* key, int rows, size_t at, int n, u64 x,
+                                        const LimbConst& lc) {
   key[at] = make_ulonglong2(x, shoup_companion(x, lc.q));
+  if (!c.tw_fwd_f) return;
   const u64 half = lc.q >> 1, y = reduce128(x >> 32, x << 32, lc);
   const i64 a = x > half ? (i64)(x - lc.q) : (i64)x, b = y > half ? (i64)(y - lc.q) : (i64)y;
   const u64 m = (1ull << lc.sb) - 1ull;
@@ -1239,8 +1241,8 @@ struct ModeKeygen {
   template <int N, bool SPLIT>
   static __device__ __forceinline__ void store2(const DevCtx& c, const Params& P, const LimbConst& lc, int, int limb,
                                                 int e, u64 x0, u64 x1) {
-    put_key(P.sk, c.L, limb * N + e, N, x0, lc);
-    put_key(P.sk, c.L, limb * N + e + 1, N, x1, lc);
+    put_key(c, P.sk, c.L, limb * N + e, N, x0, lc);
+    put_key(c, P.sk, c.L, limb * N + e + 1, N, x1, lc);
   }
 };
 
@@ -1277,8 +1279,8 @@ struct ModePkKeygen {
       const u64 a = reduce64(uniform_word(w.v[i], e + i, 0, limb, P.seed, PENCIL_DOM_PK_A, lc), lc);
       const ulonglong2 s = __ldg(P.sk + (size_t)limb * N + e + i);
       const u64 p0 = neg_mod(add_mod(mul_shoup(a, s.x, s.y, lc.q), x[i], lc.q), lc.q);
-      put_key(P.key, 2 * c.L, (size_t)limb * N + e + i, N, p0, lc);
-      put_key(P.key, 2 * c.L, (size_t)(c.L + limb) * N + e + i, N, a, lc);
+      put_key(c, P.key, 2 * c.L, (size_t)limb * N + e + i, N, p0, lc);
+      put_key(c, P.key, 2 * c.L, (size_t)(c.L + limb) * N + e + i, N, a, lc);
     }
   }
 };

@@ -5,6 +5,34 @@
 
 namespace pencil {
 
+// ------------------------------------------------------------------ split products
+inline int bit_length(unsigned long long q) { return 64 - __builtin_clzll(q); }
+
+// Whether mul_split (common.cuh) takes the prime q = 2^b - c: c < 2^24 for b = 59, 60 and
+// c < 2^(b-33) below; b >= 40.
+inline bool split_prime(unsigned long long q) {
+  const int b = bit_length(q);
+  if (b < 40 || b > 60) return false;
+  return (1ull << b) - q < (b >= 59 ? 1ull << 24 : 1ull << (b - 33));
+}
+
+// Split twiddle of mul_split for a split_prime q of b bits: the centred representatives of
+// w < q and of w 2^32 mod q, each as (low b - 32 bits, signed rest).
+struct SplitWords {
+  unsigned v[4];
+};
+inline SplitWords split_words(unsigned long long w, unsigned long long q) {
+  const int sh = bit_length(q) - 32;
+  const unsigned long long v[2] = {w, (unsigned long long)(((unsigned __int128)w << 32) % q)};
+  SplitWords out;
+  for (int i = 0; i < 2; ++i) {
+    const long long x = v[i] > q / 2 ? (long long)(v[i] - q) : (long long)v[i];
+    out.v[2 * i] = (unsigned)((unsigned long long)x & ((1ull << sh) - 1));
+    out.v[2 * i + 1] = (unsigned)(int)(x >> sh);
+  }
+  return out;
+}
+
 // ------------------------------------------------------------------ plaintext correlations
 // Reduction of one tensor-core launch in parts of whole 16-element chunks.
 struct RingSplit {

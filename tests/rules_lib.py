@@ -23,6 +23,11 @@ extern "C" int ring_form_(long long outs, const int* d, int wide, int sms) {
 }
 extern "C" int bias_parts_(long long elements) { return bias_parts(elements); }
 extern "C" int lincomb_pairs_(long long count) { return lincomb_pairs(count); }
+extern "C" int split_prime_(unsigned long long q) { return split_prime(q); }
+extern "C" void split_words_(unsigned long long w, unsigned long long q, unsigned* out) {
+  const SplitWords s = split_words(w, q);
+  for (int i = 0; i < 4; ++i) out[i] = s.v[i];
+}
 """
 RING_FORMS = ("tile", "offsets", "outputs", "digits")
 
@@ -66,3 +71,15 @@ def ring_form(layer, role: int, t_bits: int, sms: int = 152) -> str:
 
 def lincomb_pairs(count: int) -> bool:
     return bool(load().lincomb_pairs_(ctypes.c_longlong(count)))
+
+
+def split_prime(q: int) -> bool:
+    return bool(load().split_prime_(ctypes.c_ulonglong(q)))
+
+
+def split_words(w: int, q: int):
+    """(low, rest) of w and of w 2^32 mod q, the rests signed."""
+    out = (ctypes.c_uint * 4)()
+    load().split_words_(ctypes.c_ulonglong(w), ctypes.c_ulonglong(q), out)
+    signed = [v - (1 << 32) if v >> 31 else v for v in out]
+    return (out[0], signed[1]), (out[2], signed[3])

@@ -1,8 +1,10 @@
 """Launch rules (csrc/rules.h) on the host."""
 import ctypes
+import random
 
 import pytest
 
+from oracle.params import BfvParams
 from tests import rules_lib
 
 # words that fit a 284 208 MiB device beside nothing else
@@ -63,3 +65,29 @@ def test_a_small_bias_gradient_is_no_cluster_launch():
 
 def test_small_linear_combinations_take_one_element_a_thread():
     assert not rules_lib.lincomb_pairs(100000) and rules_lib.lincomb_pairs(1 << 17)
+
+
+# (log2 N, primes, bits): every ring the repository's tests and benchmark use, and the
+# shortest and longest primes a context takes
+PRIMES = [q for ring in ((12, 2, 54), (12, 2, 60), (13, 3, 60), (14, 4, 60), (13, 4, 59), (12, 2, 48))
+          for q in BfvParams(log_n=ring[0], num_primes=ring[1], prime_bits=ring[2]).primes]
+
+
+@pytest.mark.parametrize("q", sorted(set(PRIMES)))
+def test_split_words_are_the_centred_residues(q):
+    """(compiled with undefined behaviour trapped: no shift leaves its type)"""
+    if not rules_lib.split_prime(q):
+        pytest.skip("not of the split products' form")
+    sh, r = q.bit_length() - 32, random.Random(q)
+    for w in [0, 1, 2, q // 2, q // 2 + 1, q - 2, q - 1] + [r.randrange(q) for _ in range(200)]:
+        for (low, rest), v in zip(rules_lib.split_words(w, q), (w, (w << 32) % q)):
+            x = (rest << sh) + low
+            assert x % q == v and -q // 2 <= x <= q // 2
+            assert 0 <= low < 1 << sh and -(1 << 31) <= rest < 1 << 31
+
+
+def test_short_primes_take_no_split_products():
+    for bits in (30, 31, 32, 36, 39):
+        for q in BfvParams(log_n=12, num_primes=2, prime_bits=bits).primes:
+            assert not rules_lib.split_prime(q)
+    assert not rules_lib.split_prime((1 << 61) - 1)
