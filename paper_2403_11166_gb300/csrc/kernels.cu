@@ -486,7 +486,7 @@ __global__ void __launch_bounds__(MAC_BT + 32) k_mac_bulk(DevCtx ctx, MacParams 
 }
 
 // ------------------------------------------------------------------ MAC, few input blocks
-// Alg. 1 with K <= MAC_SHORT_K input blocks.  What is left per output then is its own
+// Alg. 1 with K <= kMacShortK input blocks.  What is left per output then is its own
 // traffic (a re-mask word in, two words out), so the kernel streams: a thread = one slot of
 // MAC_SHORT_M output rows m keeps A[m, 0 .. K-1] (both components, split) in registers and
 // walks a strip of output columns n, loading a column's K words of B and its re-mask words
@@ -497,7 +497,6 @@ __global__ void __launch_bounds__(MAC_BT + 32) k_mac_bulk(DevCtx ctx, MacParams 
 // (tensor cores 656); M = 10, NC = 16: K = 1 40 / 26, 3 51 / 34, 6 72 / 49; M = 64, NC = 10:
 // K = 3 198 / 110; M = 4, NC = 4: 13 to 15 either way.
 // 2 K <= 12 products per accumulator: no fold before the last.
-#define MAC_SHORT_K 6
 #define MAC_SHORT_M 2
 template <int K>
 __global__ void __launch_bounds__(MAC_BT) k_mac_short(const __grid_constant__ DevCtx ctx,
@@ -837,51 +836,32 @@ static cudaError_t launch_mac_bulk(const DevCtx& ctx, const MacParams& P0, bool 
   return cudaSuccess;
 }
 
-// Digit products on the tensor cores (mac_mma.cu) against the integer multiply-add
-// kernels, by modelled time of one slot's block in common units.  A tensor-core tile
-// is 16 columns n x 4 rows m (Alg. 2: 8 rows of one component) whatever part of it
-// exists and pays its combination once per chunk of 16 (8) input blocks; the integer
-// kernels pay per existing (m, n) pair and input block.  Fitted to launches on GB300
-// at L N = 24576 (us; tensor cores / k_mac_bulk): M = 30, NC = 64: K = 3 605 / 510,
-// 5 657 / 651, 6 657 / 768, 16 875 / 1542, 32 1582 / 2871; M = 10, NC = 16: K = 6
-// 74 / 72, 8 75 / 84, 16 91 / 138; M = 4, NC = 4: K = 16 36 / 25, 32 65 / 42; M = 2,
-// NC = 64: K = 16 150 / 114.  Two 54-bit primes at N = 4096 (k_mac): M = 10, NC = 16:
-// K = 1 24 / 22, 2 24 / 28, 16 38 / 129.  (Single launches with split-form primes take
-// k_mac_short up to K = 6; there the rule decides for the batch engine's items only.)
+static MacKnobs mac_knobs(const DevCtx& ctx) {
+  return MacKnobs{ctx.mac_mma != 0, ctx.mac_split != 0, ctx.mac_nt, ctx.mac_staging};
+}
+
 bool mac_mma_wins(const DevCtx& ctx, const MacParams& P, bool dual) {
-  if (!ctx.mac_mma || ctx.mac_nt == 0 || ctx.mac_staging != 1) return false;   // not available, or tuned away
-  const double rows = P.M - P.m_base, K = P.K, nt = (P.NC + 15) / 16, pairs = rows * P.NC / 64.0;
-  if (dual)
-    return 2.0 * ((P.M - P.m_base + 7) / 8) * nt * 22.0 * ((P.K + 7) / 8) <
-           pairs * (ctx.mac_split ? 11.0 + 6.0 * K : 15.0 + 13.0 * K);
-  const double unit = P.K <= 16 ? 19.0 + 0.7 * K : 26.0 * ((P.K + 15) / 16);
-  return ((P.M - P.m_base + 3) / 4) * nt * unit < pairs * (ctx.mac_split ? 11.0 + 2.65 * K : 15.0 + 6.6 * K);
+  return mac_digits_win(mac_knobs(ctx), P.M - P.m_base, P.K, P.NC, dual);
 }
 
 cudaError_t launch_mac(const DevCtx& ctx, const MacParams& P0, bool dual, cudaStream_t s) {
-  if (!dual && ctx.mac_split && ctx.mac_nt != 0 && ctx.mac_staging == 1 && P0.K >= 1 && P0.K <= MAC_SHORT_K)
-    return launch_mac_short(ctx, P0, s);   // faster than both at every size measured
-  if (mac_mma_wins(ctx, P0, dual)) return launch_mac_mma(ctx, P0, dual, s);
-  if (ctx.mac_split && ctx.mac_nt == 0) return launch_mac_smem(ctx, P0, dual, s);
-  if (ctx.mac_split && ctx.mac_staging == 1) {
-    switch (ctx.mac_nt) {
-      case 2:
-        return launch_mac_bulk<2>(ctx, P0, dual, s);
-      case 8:
-        return launch_mac_bulk<8>(ctx, P0, dual, s);
-      default:
-        return launch_mac_bulk<4>(ctx, P0, dual, s);
-    }
-  }
-  if (ctx.mac_split) {
-    switch (ctx.mac_nt) {
-      case 2:
-        return launch_mac_ring<2>(ctx, P0, dual, s);
-      case 8:
-        return launch_mac_ring<8>(ctx, P0, dual, s);
-      default:
-        return launch_mac_ring<4>(ctx, P0, dual, s);
-    }
+  switch (mac_form(mac_knobs(ctx), P0.M - P0.m_base, P0.K, P0.NC, dual)) {
+    case MacForm::kShort:
+      return launch_mac_short(ctx, P0, s);
+    case MacForm::kDigits:
+      return launch_mac_mma(ctx, P0, dual, s);
+    case MacForm::kSmem:
+      return launch_mac_smem(ctx, P0, dual, s);
+    case MacForm::kBulk:
+      return ctx.mac_nt == 2   ? launch_mac_bulk<2>(ctx, P0, dual, s)
+             : ctx.mac_nt == 8 ? launch_mac_bulk<8>(ctx, P0, dual, s)
+                               : launch_mac_bulk<4>(ctx, P0, dual, s);
+    case MacForm::kRing:
+      return ctx.mac_nt == 2   ? launch_mac_ring<2>(ctx, P0, dual, s)
+             : ctx.mac_nt == 8 ? launch_mac_ring<8>(ctx, P0, dual, s)
+                               : launch_mac_ring<4>(ctx, P0, dual, s);
+    case MacForm::kGeneric:
+      break;
   }
   constexpr int NT = 8;
   const int threads = 256;

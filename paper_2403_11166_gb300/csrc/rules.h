@@ -33,6 +33,51 @@ inline SplitWords split_words(unsigned long long w, unsigned long long q) {
   return out;
 }
 
+// ------------------------------------------------------------------ multiply-accumulate
+// What a context allows and asks for (DevCtx: mac_mma, mac_split, mac_nt, mac_staging).
+struct MacKnobs {
+  bool digits, split;
+  int columns, staging;
+};
+
+enum class MacForm {
+  kGeneric,   // k_mac: any prime
+  kSmem,      // k_mac_smem: columns 0
+  kRing,      // k_mac_ring: staging 0
+  kBulk,      // k_mac_bulk
+  kShort,     // k_mac_short: Alg. 1 with at most kMacShortK input blocks
+  kDigits     // k_mac_mma: digit products on the tensor cores
+};
+constexpr int kMacShortK = 6;
+
+// Digit products on the tensor cores (mac_mma.cu) against the integer multiply-add
+// kernels, by modelled time of one slot's block in common units.  A tensor-core tile
+// is 16 columns n x 4 rows m (Alg. 2: 8 rows of one component) whatever part of it
+// exists and pays its combination once per chunk of 16 (8) input blocks; the integer
+// kernels pay per existing (m, n) pair and input block.  Fitted to launches on GB300
+// at L N = 24576 (us; tensor cores / k_mac_bulk): M = 30, NC = 64: K = 3 605 / 510,
+// 5 657 / 651, 6 657 / 768, 16 875 / 1542, 32 1582 / 2871; M = 10, NC = 16: K = 6
+// 74 / 72, 8 75 / 84, 16 91 / 138; M = 4, NC = 4: K = 16 36 / 25, 32 65 / 42; M = 2,
+// NC = 64: K = 16 150 / 114.  Two 54-bit primes at N = 4096 (k_mac): M = 10, NC = 16:
+// K = 1 24 / 22, 2 24 / 28, 16 38 / 129.  (Single launches with split-form primes take
+// k_mac_short up to K = 6; there the rule decides for the batch engine's items only.)
+inline bool mac_digits_win(const MacKnobs& c, int rows, int K, int NC, bool dual) {
+  if (!c.digits || c.columns == 0 || c.staging != 1) return false;   // not available, or tuned away
+  const double k = K, nt = (NC + 15) / 16, pairs = (double)rows * NC / 64.0;
+  if (dual) return 2.0 * ((rows + 7) / 8) * nt * 22.0 * ((K + 7) / 8) < pairs * (c.split ? 11.0 + 6.0 * k : 15.0 + 13.0 * k);
+  const double unit = K <= 16 ? 19.0 + 0.7 * k : 26.0 * ((K + 15) / 16);
+  return ((rows + 3) / 4) * nt * unit < pairs * (c.split ? 11.0 + 2.65 * k : 15.0 + 6.6 * k);
+}
+
+// Form of a single launch of output rows x NC products over K input blocks.
+inline MacForm mac_form(const MacKnobs& c, int rows, int K, int NC, bool dual) {
+  if (!dual && c.split && c.columns != 0 && c.staging == 1 && K >= 1 && K <= kMacShortK)
+    return MacForm::kShort;   // faster than both at every size measured
+  if (mac_digits_win(c, rows, K, NC, dual)) return MacForm::kDigits;
+  if (!c.split) return MacForm::kGeneric;
+  return c.columns == 0 ? MacForm::kSmem : c.staging == 1 ? MacForm::kBulk : MacForm::kRing;
+}
+
 // ------------------------------------------------------------------ plaintext correlations
 // Reduction of one tensor-core launch in parts of whole 16-element chunks.
 struct RingSplit {

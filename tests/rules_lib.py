@@ -28,7 +28,11 @@ extern "C" void split_words_(unsigned long long w, unsigned long long q, unsigne
   const SplitWords s = split_words(w, q);
   for (int i = 0; i < 4; ++i) out[i] = s.v[i];
 }
+extern "C" int mac_form_(int digits, int split, int columns, int staging, int rows, int K, int NC, int dual) {
+  return (int)mac_form(MacKnobs{digits != 0, split != 0, columns, staging}, rows, K, NC, dual != 0);
+}
 """
+MAC_FORMS = ("generic", "smem", "ring", "bulk", "short", "digits")
 RING_FORMS = ("tile", "offsets", "outputs", "digits")
 
 
@@ -83,3 +87,9 @@ def split_words(w: int, q: int):
     load().split_words_(ctypes.c_ulonglong(w), ctypes.c_ulonglong(q), out)
     signed = [v - (1 << 32) if v >> 31 else v for v in out]
     return (out[0], signed[1]), (out[2], signed[3])
+
+
+def mac_form(rows: int, k: int, nc: int, dual: bool = False, split: bool = True, columns: int = 4, staging: int = 1) -> str:
+    """Form of a single multiply-accumulate; split: the context's primes are the 60-bit ones
+    (else other primes that digit products take)."""
+    return MAC_FORMS[load().mac_form_(1, int(split), columns, staging, rows, k, nc, int(dual))]

@@ -91,3 +91,13 @@ def test_short_primes_take_no_split_products():
         for q in BfvParams(log_n=12, num_primes=2, prime_bits=bits).primes:
             assert not rules_lib.split_prime(q)
     assert not rules_lib.split_prime((1 << 61) - 1)
+
+
+def test_multiply_accumulate_forms():
+    """Alg. 1 with few input blocks streams; digit products where a tile's 4 x 16 (weight
+    gradients 8 x 16) outputs mostly exist; the knobs and the primes decide the rest."""
+    form = rules_lib.mac_form
+    assert form(10, 6, 16) == "short" and form(10, 16, 16) == "digits" and form(64, 32, 43, dual=True) == "digits"
+    assert form(2, 16, 64) == "bulk" and form(5, 9, 7) == "bulk" and form(3, 2, 5, dual=True) == "bulk"
+    assert form(10, 16, 16, staging=0) == "ring" and form(10, 16, 16, columns=0) == "smem"
+    assert form(10, 2, 16, split=False) == "digits" and form(10, 16, 16, split=False, columns=0) == "generic"
