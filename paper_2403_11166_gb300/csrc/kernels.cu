@@ -758,8 +758,11 @@ static cudaError_t launch_mac_smem(const DevCtx& ctx, const MacParams& P0, bool 
   const int MB = 64 / NB;
   const int words = dual ? 3 * (MB + NB) : 2 * MB + NB + (P0.p0 ? MB : 0);
   const size_t smem = (size_t)MAC_STAGES * words * MAC_LANES * sizeof(u64);
-  cudaError_t e = dual ? cudaFuncSetAttribute(k_mac_smem<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-                       : cudaFuncSetAttribute(k_mac_smem<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // the most of any launch (64 rows x 1 column): the attribute is the function's, and another
+  // thread may launch with other sizes between the two calls here
+  const int most = (int)(MAC_STAGES * 3 * 65 * MAC_LANES * sizeof(u64));
+  cudaError_t e = dual ? cudaFuncSetAttribute(k_mac_smem<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most)
+                       : cudaFuncSetAttribute(k_mac_smem<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
   if (e != cudaSuccess) return e;
   const int nblocks = (P0.NC + NB - 1) / NB;
   MacParams P = P0;

@@ -65,3 +65,43 @@ def test_threads_launch_products_of_one_and_two_stages(rows):
     assert not codes
     for _, _, out, want, _ in jobs:
         assert torch.equal(out, want)
+
+
+def test_threads_launch_staged_products_of_different_shapes():
+    """The same for the shared-memory staged kernel (columns 0), whose stage depends on the
+    number of output columns: 1 (the largest) and 8 (the smallest)."""
+    from paper_2403_11166_gb300 import he
+    ctx = he.Context(12, 2, 60, 41)
+    ctx.tune(he.TUNE_MAC_COLUMNS, 0)
+    jobs = []
+    for nc in (1, 8) * 2:
+        plan = he.Plan(ctx, he.Layer(he.FC, 8, 2, nc), he.ROLE_FWD, (1, 1, 1, 1, 1, 1, 1))
+        s = plan.sizes
+        ct_in, ct_out, pt = plan.new_ct(s.ct_in).zero_(), plan.new_ct(s.ct_out), plan.new_pt(s.pt).zero_()
+        x0 = torch.zeros(16, dtype=torch.int64, device="cuda")
+        y0 = torch.empty(s.out_elems, dtype=torch.int64, device="cuda")
+        ws, stream = plan.new_ws(s.ws_forward), torch.cuda.Stream()
+        he.he_linear_forward(ctx, plan, ct_in, pt, x0, None, 9, ct_out, y0, ws)
+        torch.cuda.synchronize()
+        args = (ctx.h, plan.h, he._ptr(ct_in), he._ptr(pt), he._ptr(ct_out), he._ptr(ws),
+                ctypes.c_size_t(ws.numel() * 8), he._stream(stream))
+        jobs.append((args, ct_out, ct_out.clone(), (plan, ct_in, pt, ws, stream)))
+    codes = []
+    start = threading.Barrier(len(jobs))
+
+    def run(args):
+        start.wait()
+        for _ in range(CALLS):
+            rc = he.lib.he_linear_forward_apply(*args)
+            if rc:
+                codes.append(rc)
+
+    threads = [threading.Thread(target=run, args=(j[0],)) for j in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not codes
+    for _, out, want, _ in jobs:
+        assert torch.equal(out, want)
