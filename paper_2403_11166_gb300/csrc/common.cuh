@@ -206,8 +206,8 @@ __device__ __forceinline__ void gs_butterfly(u64& x, u64& y, u64 w, u64 ws, u64 
 }
 
 // ------------------------------------------------------------------ pseudo-Mersenne twiddle products
-// For q = 2^b - c (c < 2^24 for b = 59, 60, c < 2^(b-33) below) and signed lazy values
-// |y| < 8 2^b.  A twiddle w is kept as its centred representative and that of
+// For q = 2^b - c (c < 2^24 for b = 59, 60, c < 2^(b-33) below; split_prime) and signed lazy
+// values y in (-7 2^b, 7.97 2^b).  A twiddle w is kept as its centred representative and that of
 // w 2^32 mod q, each split at bit sh = b - 32: w = w1 2^sh + w0 with 0 <= w0 < 2^sh
 // and w1 a signed 32-bit word.  With y = y1 2^32 + y0, y0 the SIGNED low word (y1 takes
 // its carry), and v the split of w 2^32:
@@ -215,8 +215,12 @@ __device__ __forceinline__ void gs_butterfly(u64& x, u64& y, u64 w, u64 ws, u64 
 //   y w = L + H 2^sh = L + lo32(H) 2^sh + hi32(H) 2^b = L + lo32(H) 2^sh + hi32(H) c  (mod q):
 // the high word of H is the quotient and its low word sits at bit sh, so nothing is
 // split by shifts and masks and no quotient is estimated: five wide multiply-adds, two
-// shifts, three additions.  The value is signed, for y in [-A, B] (units of 2^b)
-// between -(1/2 + A/16 + 1/32) and 3/2 + B/16 + 1/32.  (The unsigned form it replaces
+// shifts, three additions.  The value is signed, for y in [-A, B] (units of 2^b) between
+// -(1/2 + A 2^(b-64) + e) and 3/2 + B 2^(b-64) + e with e = max|hi32(H)| c / 2^b <=
+// (2^30 + max(A, B) 2^(b-33)) c / 2^b: 1/64 + max(A, B) / 512 for b = 60, twice the first
+// term for 59, 1/8 + max(A, B) 2^(b-66) below.  (Shorter primes have the larger e and the
+// smaller A and B terms: the ranges of ct_split and gs_split hold for all of them.  Every
+// range here is checked in exact fractions, tests/test_split_ranges.py.)  (The unsigned form it replaces
 // split w at bit 32 and needed fourteen instructions; measured in registers, a forward
 // butterfly with its share of the folds takes 30.0 cycles per warp against 36.7; the low
 // word's shift as a sixth wide multiply-add 32.5.)
@@ -297,11 +301,6 @@ __device__ __forceinline__ void gs_split(u64& x, u64& y, const uint4 w, const Fo
   const u64 d = x - y;
   x = x + y;
   y = mul_split(0, d, w, f);
-}
-
-// [0, 8q) -> [0, q)
-__device__ __forceinline__ u64 canon8(u64 x, u64 q) {
-  return csub(csub_s(csub_s(x, 4 * q), 2 * q), q);
 }
 
 // [0, 4q) -> [0, q)

@@ -261,8 +261,8 @@ __device__ __forceinline__ void ntt_inv_run(const DevCtx& ctx, const typename Mo
 // common.cuh): no correction step inside a butterfly and no added multiple of q;
 // signed values grow lazily and are folded only where the bound requires it
 // (units of 2^b):
-//  * forward: from [0, 1], k = 1 .. 4 stages stay inside -(1.59, 3.27, 5.06, 6.96) ..
-//    (2.59, 4.27, 6.06, 7.96), so the registers are folded once per round of at most
+//  * forward: from [0, 1], k = 1 .. 4 stages stay inside -(1.65, 3.33, 5.06, 6.96) ..
+//    (2.65, 4.33, 6.06, 7.96) for primes of every length, so the registers are folded once per round of at most
 //    four stages (rounds of five fold after their second stage too); before the last
 //    fold 4 q (at most two stages) or 8 q is added, so that it is unsigned and one
 //    conditional subtraction is canonical;
