@@ -503,12 +503,12 @@ int pencil_profile_read(PencilCtx* ctx, PencilProfEntry* out, int32_t max_entrie
  * multiply-accumulate, 4: split-quotient Shoup multiply (mul_shoup3), 5: forward
  * butterfly on [0, 8q), 6: forward butterfly on [0, 4q) (Harvey), 7: inverse
  * butterfly on [0, 4q), 8: inverse butterfly on [0, 2q) (Harvey), 9: 32x32
- * high half (mul.hi.u32), 10: pseudo-Mersenne product (mul_fold, PTX), 11: the
- * same product written in C (mul_fold_c), 12: forward fold butterfly, 13: inverse
- * fold butterfly, 14: fold60 alone, 15: forward butterfly with mul_fold_c; for
- * 5-8 and 12, 13, 15 a step is one butterfly.  Times the launch with CUDA events on `stream` and returns
- * the elapsed milliseconds and the number of chain steps (threads * 8 * iters).
- * Synchronises `stream`. */
+ * high half (mul.hi.u32), 10 or 11: split product (mul_split), 12 or 15: forward
+ * split butterfly and its share of the folds, 13: inverse split butterfly and its
+ * fold, 14: fold of a signed lazy value; for 5-8, 12, 13 and 15 a step is one
+ * butterfly.  Times the launch with CUDA events on `stream` and returns the elapsed
+ * milliseconds and the number of chain steps (threads * 8 * iters).  Synchronises
+ * `stream`. */
 int pencil_mul_probe(PencilCtx* ctx, int32_t which, int64_t iters, int32_t blocks, int32_t threads, double* ms,
                      double* steps, void* stream);
 

@@ -1135,8 +1135,6 @@ static int alg1_prepare(PencilCtx* ctx, const PencilPlan* P, const u64* x0, cons
   return PENCIL_OK;
 }
 
-// Alg. 1 steps 2-3 on the received ciphertexts: ct_out[m, n] = sum_k
-// (ct_in[m, k] + NTT(Delta x0)[m, k]) pt[k, n] - NTT(Delta s)[m, n], one launch.
 // -(bias of all the combinations of diagonals of one output) mod q_j (digits.cuh)
 static void mac_mma_start(const PencilCtx* ctx, MacParams& M, bool dual) {
   const u64 combos = (u64)mac_mma_combinations(M.K, dual);
@@ -1144,6 +1142,8 @@ static void mac_mma_start(const PencilCtx* ctx, MacParams& M, bool dual) {
     M.start[j] = mulmod(combos % ctx->primes[j], ctx->dev.limb[j].digit_bias, ctx->primes[j]);
 }
 
+// Alg. 1 steps 2-3 on the received ciphertexts: ct_out[m, n] = sum_k
+// (ct_in[m, k] + NTT(Delta x0)[m, k]) pt[k, n] - NTT(Delta s)[m, n], one launch.
 static int alg1_apply(PencilCtx* ctx, const PencilPlan* P, const u64* ct_in, const u64* pt, u64* ct_out, char* ws,
                       cudaStream_t s) {
   const Alg1Ws w = alg1_ws(P, ws);

@@ -1032,7 +1032,7 @@ struct ModeRaw {
 
 // DO encryption: prologue round(q m / t) + e (m gathered by the packing), epilogue
 // c0 = slot - a*s_hat, c1 = a with a sampled in the NTT domain, four coefficients
-// per Philox block (one 64-bit word each, uniform_mod_q).
+// per Philox block (one 64-bit word each, uniform_word).
 struct ModeEncrypt {
   static constexpr bool kHeavyLoad = true;
   static constexpr bool kQuad = true;
@@ -1251,8 +1251,8 @@ __device__ __forceinline__ u64 neg_mod(u64 v, u64 q) { return v ? q - v : 0; }
 
 // DO public key (BFV as in Fan-Vercauteren): x = NTT(e) of the sampled error;
 // p1 = a, uniform in the NTT domain from Philox (key (seed, 7), counter
-// (i/4, 0, limb, 0), word i%4; uniform_mod_q); p0 = -(a s) - x.  Both stored
-// with Shoup companions: key[comp][L][N].
+// (i/4, 0, limb, 0), word i%4; uniform_word); p0 = -(a s) - x.  Both stored as
+// put_key stores them: key[comp][L][N].
 struct ModePkKeygen {
   static constexpr bool kHeavyLoad = true;
   static constexpr bool kQuad = true;
