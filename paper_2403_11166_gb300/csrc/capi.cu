@@ -875,7 +875,13 @@ extern "C" int pencil_plan_linear(PencilCtx* ctx, const PencilLayerDesc* layer, 
     pencil_plan_destroy(P);
     return PENCIL_E_CUDA;
   }
-  int support[3] = {0, 0, 0};
+  int support[3] = {0, 0, 0}, warps[3] = {0, 0, 0};
+  for (int sgm = 0; sgm < 3; ++sgm)
+    for (int e = 0; e < n; e += 128) {
+      bool some = false;
+      for (int i = 0; i < 128; ++i) some = some || tab[(size_t)sgm * n + e + i] != PENCIL_TAB_NONE;
+      warps[sgm] += some ? 1 : 0;
+    }
   for (int sgm = 0; sgm < 3; ++sgm)
     for (int e = n - 1; e >= 0; --e)
       if (tab[(size_t)sgm * n + e] != PENCIL_TAB_NONE) {
@@ -883,11 +889,11 @@ extern "C" int pencil_plan_linear(PencilCtx* ctx, const PencilLayerDesc* layer, 
         break;
       }
   const unsigned char* d_groups = reinterpret_cast<const unsigned char*>(P->d_tab + 3 * (size_t)n);
-  P->pk_v = Packing{P->d_tab, P->d_org, make_int4(g.B, g.Ci, g.H, g.W), support[0], d_groups};
+  P->pk_v = Packing{P->d_tab, P->d_org, make_int4(g.B, g.Ci, g.H, g.W), support[0], d_groups, warps[0]};
   P->pk_w = Packing{P->d_tab + n, P->d_org + P->ct_in, make_int4(g.Co, g.Ci, g.KH, g.KW), support[1],
-                    d_groups + n / 32};
+                    d_groups + n / 32, warps[1]};
   P->pk_y = Packing{P->d_tab + 2 * (size_t)n, P->d_org + P->ct_in + P->pt, make_int4(g.B, g.Co, g.Ho(), g.Wo()),
-                    support[2], d_groups + 2 * (n / 32)};
+                    support[2], d_groups + 2 * (n / 32), warps[2]};
 
   // --- workspace sizes (bytes, each region 256-byte aligned)
   auto al = [](long long b) { return (b + 255) / 256 * 256; };

@@ -957,14 +957,16 @@ cudaError_t launch_sample_pk(u64 seed, int first, int count, int n, int8_t* e1, 
 // one per coefficient before that).  Here the CTA lists its different blocks once, draws
 // them one per thread and hands the words out through shared memory: about 1.3 blocks per
 // thread where rows are 28 elements and a gap of 2 (1920 polynomials of 28 x 19 tiles at
-// N = 8192: 241 -> 120 us; 160 of 32 x 32 tiles 21 -> 17).  A warp without outputs lists
-// nothing and needs no window: each thread draws its padding block.  Three launches of a 128
-// to 128 channel layer's forward and gradients, whose polynomials are 75 to 99 % padding: 344
-// us drawn by each thread, 376 with every block listed, 330.  What still loses to drawing by
+// N = 8192: 241 -> 114 us; 160 of 32 x 32 tiles 21 -> 17).  With SKIP (mask_skips) a warp
+// without outputs lists nothing and needs no window: each thread draws its padding block.
+// Three launches of a 128 to 128 channel layer's forward and gradients, whose polynomials are
+// 75 to 99 % padding: 344 us drawn by each thread, 376 with every block listed, 330 skipping;
+// full polynomials pay for the test (the 1920 above: 120 us).  What still loses to drawing by
 // each thread: outputs at stride (no two neighbours share a block; 513 polynomials of a fully
 // connected layer's weight gradient 47 -> 57 us) and dense aligned rows (13 -> 14).  At least
 // five or six CTAs per SM (48 or 40 registers instead of 56): spills, 1.1 to 1.4x.
 #define MASK_POLY_LIST 512   // blocks drawn at a time (of at most 256 + 1024): 20 KB, eight CTAs per SM
+template <bool SKIP>
 __device__ __forceinline__ void mask_poly_block(const DevCtx& ctx, const Packing& pk, const Accessor& ac, u64 seed,
                                                 int ct, int blk, u64* out_ct) {
   __shared__ i64 src[MASK_POLY_LIST];   // element block, or -1 - (block of the padding stream)
@@ -981,7 +983,7 @@ __device__ __forceinline__ void mask_poly_block(const DevCtx& ctx, const Packing
     ent[i] = __ldg(pk.tab + 4 * blk + i);
     none = none && ent[i].x == PENCIL_TAB_NONE;
   }
-  const bool empty = __all_sync(0xffffffffu, none);   // no outputs in the warp: nothing to list
+  const bool empty = SKIP && __all_sync(0xffffffffu, none);   // no outputs in the warp: nothing to list
   Philox4 r = {{0, 0, 0, 0}};
   if (empty) {
     r = philox4x64((u64)blk, (u64)ct, 0ull, 0ull, seed, PENCIL_DOM_MASK_PAD);
@@ -1050,18 +1052,22 @@ __device__ __forceinline__ void mask_poly_block(const DevCtx& ctx, const Packing
 }
 
 // (a CTA of 256 threads stays inside one polynomial: its window is uniform)
+template <bool SKIP>
 __global__ void __launch_bounds__(256) k_mask_poly(const __grid_constant__ DevCtx ctx, const __grid_constant__ Packing pk,
                                                    const __grid_constant__ Accessor ac, u64 seed, u64* out) {
   const int lg = ctx.log_n - 10, ct = blockIdx.x >> lg;
   const int blk = ((int)(blockIdx.x & ((1u << lg) - 1u)) << 8) + threadIdx.x;
-  mask_poly_block(ctx, pk, ac, seed, ct, blk, out + ((size_t)ct << ctx.log_n));
+  mask_poly_block<SKIP>(ctx, pk, ac, seed, ct, blk, out + ((size_t)ct << ctx.log_n));
 }
 
 cudaError_t launch_mask_poly(const DevCtx& ctx, const Packing& pk, const Accessor& ac, u64 seed, int count, u64* out,
                              cudaStream_t s) {
   const long long total = (long long)count * (ctx.n >> 2);
   if (total == 0) return cudaSuccess;
-  k_mask_poly<<<(unsigned)(total / 256), 256, 0, s>>>(ctx, pk, ac, seed, out);
+  if (mask_skips(count, ctx.n, pk.warps, ctx.sms))
+    k_mask_poly<true><<<(unsigned)(total / 256), 256, 0, s>>>(ctx, pk, ac, seed, out);
+  else
+    k_mask_poly<false><<<(unsigned)(total / 256), 256, 0, s>>>(ctx, pk, ac, seed, out);
   return cudaGetLastError();
 }
 
@@ -1577,7 +1583,7 @@ __global__ void __launch_bounds__(256) k_mask_poly_multi(const __grid_constant__
   const int blk = ((int)(blockIdx.x & ((1u << lg) - 1u)) << 8) + threadIdx.x;
   const MaskPolyP& P = Ps[it.x];
   const u64 seed = P.seed + ((step ? *step : 0ull) << 32);
-  mask_poly_block(ctx, P.pk, P.ac, seed, it.y, blk, P.out + ((size_t)it.y << ctx.log_n));
+  mask_poly_block<true>(ctx, P.pk, P.ac, seed, it.y, blk, P.out + ((size_t)it.y << ctx.log_n));
 }
 
 __global__ void k_mo_share_multi(const MoShareP* __restrict__ Ps, const int2* __restrict__ items, long long n_items,

@@ -194,4 +194,12 @@ inline int bias_parts(long long elements) { return elements > 4096 ? 8 : 1; }
 // 6.6 / 5.1).
 inline bool lincomb_pairs(long long count) { return count >= 1 << 17; }
 
+// Whether `count` mask polynomials, of whose n / 128 runs of 128 coefficients `warps` carry
+// outputs, are drawn by the form that skips the others (k_mask_poly): a fifth of them or more
+// are empty and the launch has two CTAs of 1024 coefficients for every SM (a smaller one is
+// one CTA's latency, which the test lengthens: 2 polynomials 3.6 / 3.9 us).
+inline bool mask_skips(long long count, int n, int warps, int sms) {
+  return 5ll * (n / 128 - warps) >= n / 128 && count * (n / 1024) >= 2ll * sms;
+}
+
 }  // namespace pencil

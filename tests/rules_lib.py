@@ -31,6 +31,7 @@ extern "C" void split_words_(unsigned long long w, unsigned long long q, unsigne
 extern "C" int mac_form_(int digits, int split, int columns, int staging, int rows, int K, int NC, int dual) {
   return (int)mac_form(MacKnobs{digits != 0, split != 0, columns, staging}, rows, K, NC, dual != 0);
 }
+extern "C" int mask_skips_(long long count, int n, int warps, int sms) { return mask_skips(count, n, warps, sms); }
 """
 MAC_FORMS = ("generic", "smem", "ring", "bulk", "short", "digits")
 RING_FORMS = ("tile", "offsets", "outputs", "digits")
@@ -93,3 +94,7 @@ def mac_form(rows: int, k: int, nc: int, dual: bool = False, split: bool = True,
     """Form of a single multiply-accumulate; split: the context's primes are the 60-bit ones
     (else other primes that digit products take)."""
     return MAC_FORMS[load().mac_form_(1, int(split), columns, staging, rows, k, nc, int(dual))]
+
+
+def mask_skips(count: int, n: int, warps: int, sms: int = 152) -> bool:
+    return bool(load().mask_skips_(ctypes.c_longlong(count), n, warps, sms))

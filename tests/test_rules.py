@@ -101,3 +101,10 @@ def test_multiply_accumulate_forms():
     assert form(2, 16, 64) == "bulk" and form(5, 9, 7) == "bulk" and form(3, 2, 5, dual=True) == "bulk"
     assert form(10, 16, 16, staging=0) == "ring" and form(10, 16, 16, columns=0) == "smem"
     assert form(10, 2, 16, split=False) == "digits" and form(10, 16, 16, split=False, columns=0) == "generic"
+
+
+def test_mask_polynomials_skip_where_many_warps_are_empty():
+    skips = rules_lib.mask_skips
+    assert skips(2752, 8192, 18) and skips(2048, 8192, 51)
+    assert not skips(2048, 8192, 52) and not skips(1920, 8192, 64)   # nearly full
+    assert not skips(2, 8192, 4) and not skips(37, 8192, 4) and skips(38, 8192, 4)   # one wave
