@@ -875,11 +875,12 @@ extern "C" int pencil_plan_linear(PencilCtx* ctx, const PencilLayerDesc* layer, 
     pencil_plan_destroy(P);
     return PENCIL_E_CUDA;
   }
-  int support[3] = {0, 0, 0}, warps[3] = {0, 0, 0};
+  int support[3] = {0, 0, 0}, filled[3] = {0, 0, 0}, warps[3] = {0, 0, 0};
   for (int sgm = 0; sgm < 3; ++sgm)
-    for (int e = 0; e < n; e += 128) {
-      bool some = false;
-      for (int i = 0; i < 128; ++i) some = some || tab[(size_t)sgm * n + e + i] != PENCIL_TAB_NONE;
+    for (int w = 0; w < n / 128; ++w) {
+      const unsigned char* g4 = groups + sgm * (n / 32) + 4 * w;
+      const int some = g4[0] + g4[1] + g4[2] + g4[3];
+      filled[sgm] += some;
       warps[sgm] += some ? 1 : 0;
     }
   for (int sgm = 0; sgm < 3; ++sgm)
@@ -889,11 +890,11 @@ extern "C" int pencil_plan_linear(PencilCtx* ctx, const PencilLayerDesc* layer, 
         break;
       }
   const unsigned char* d_groups = reinterpret_cast<const unsigned char*>(P->d_tab + 3 * (size_t)n);
-  P->pk_v = Packing{P->d_tab, P->d_org, make_int4(g.B, g.Ci, g.H, g.W), support[0], d_groups, warps[0]};
+  P->pk_v = Packing{P->d_tab, P->d_org, make_int4(g.B, g.Ci, g.H, g.W), support[0], d_groups, filled[0], warps[0]};
   P->pk_w = Packing{P->d_tab + n, P->d_org + P->ct_in, make_int4(g.Co, g.Ci, g.KH, g.KW), support[1],
-                    d_groups + n / 32, warps[1]};
+                    d_groups + n / 32, filled[1], warps[1]};
   P->pk_y = Packing{P->d_tab + 2 * (size_t)n, P->d_org + P->ct_in + P->pt, make_int4(g.B, g.Co, g.Ho(), g.Wo()),
-                    support[2], d_groups + 2 * (n / 32), warps[2]};
+                    support[2], d_groups + 2 * (n / 32), filled[2], warps[2]};
 
   // --- workspace sizes (bytes, each region 256-byte aligned)
   auto al = [](long long b) { return (b + 255) / 256 * 256; };
@@ -1362,7 +1363,10 @@ extern "C" int compact_returned(PencilCtx* ctx, const PencilPlan* P, const uint6
   C.out_elems = P->out_elems;
   {
     PROF(ctx, PENCIL_K_INTT_COMPACT, s);
-    CUDA_TRY((ntt<ModeCompact, true>(ctx->dev, C, (int)P->out_count(), s, (int)P->out_first())));
+    if (compact_skips(ctx->n, P->pk_y.filled))
+      CUDA_TRY((ntt<ModeCompactFew, true>(ctx->dev, C, (int)P->out_count(), s, (int)P->out_first())));
+    else
+      CUDA_TRY((ntt<ModeCompact, true>(ctx->dev, C, (int)P->out_count(), s, (int)P->out_first())));
   }
   return PENCIL_OK;
 }

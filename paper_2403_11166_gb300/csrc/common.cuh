@@ -83,6 +83,7 @@ struct Packing {
   int4 bound;
   int support;
   const unsigned char* groups;   // [N / 32]: whether any of 32 consecutive coefficients has an entry
+  int filled;                    // those groups
   int warps;                     // of the N / 128 runs of 128 coefficients, those with an entry
 };
 

@@ -150,7 +150,7 @@ struct FewOutputs<M, std::void_t<decltype(M::kFewOutputs)>> : std::bool_constant
 // Epilogue of an inverse transform: value(l) of coefficient tau + l T.  A warp's 32
 // coefficients of one l are a group; where half of its groups or more store nothing they are
 // skipped, each lane having looked up one of them.  (Other warps run the plain loop, whose
-// loads the branches would serialise: 160 polynomials of 80 % outputs 49 us, 51 skipping.)
+// loads the branches would serialise.)
 template <class Mode, int N, int E, class Value>
 __device__ __forceinline__ void store_inverse(const DevCtx& ctx, const typename Mode::Params& P, const LimbConst& lc,
                                               int poly, int limb, int tau, Value value) {
@@ -1438,7 +1438,6 @@ struct ModeCompact {
   static constexpr InvScale kInvScale = InvScale::kNinv;
   static constexpr bool kHeavyLoad = false;
   static constexpr bool kQuad = false;
-  static constexpr bool kFewOutputs = true;
   static constexpr int kLoadUnroll = 16;
   static constexpr int kEpilogueUnroll = 16;
   struct Params {
@@ -1462,13 +1461,19 @@ struct ModeCompact {
                                              int e) {
     return __ldg(P.ct + ct_off(poly, 0, limb, c.L, N) + e);
   }
-  static __device__ __forceinline__ bool occupied(const Params& P, int group) { return __ldg(P.pk.groups + group) != 0; }
   template <int N>
   static __device__ __forceinline__ void store(const DevCtx&, const Params& P, const LimbConst& lc, int poly,
                                                int limb, int e, u64 x) {
     const i64 flat = Window(P.pk, P.ac, poly, nullptr).index(P.pk, e);
     if (flat >= 0) P.c0c[(size_t)limb * P.out_elems + flat] = x;   // x = N^{-1} INTT, canonical
   }
+};
+
+// The same for polynomials of which many groups of 32 coefficients carry no output
+// (compact_skips).
+struct ModeCompactFew : ModeCompact {
+  static constexpr bool kFewOutputs = true;
+  static __device__ __forceinline__ bool occupied(const Params& P, int group) { return __ldg(P.pk.groups + group) != 0; }
 };
 
 // Whether a launch of `count` polynomials runs on clusters of four CTAs: forward while
@@ -1595,6 +1600,7 @@ cudaError_t launch_ntt_multi(const DevCtx& ctx, const typename Mode::Params* Ps,
   PENCIL_NTT_INST1(SPEC, LOGN, LOGE, ModePkU, false, FOLD)       \
   PENCIL_NTT_INST1(SPEC, LOGN, LOGE, ModeEncryptPk, false, FOLD) \
   PENCIL_NTT_INST1(SPEC, LOGN, LOGE, ModeCompact, true, FOLD)    \
+  PENCIL_NTT_INST1(SPEC, LOGN, LOGE, ModeCompactFew, true, FOLD) \
   PENCIL_NTT_INST1(SPEC, LOGN, LOGE, ModeDecrypt, true, FOLD)
 // Radix 2^4 and 2^5 register blocks for one N and one engine.
 #define PENCIL_NTT_INSTANTIATE(SPEC, LOGN, FOLD) \

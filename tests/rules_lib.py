@@ -32,6 +32,7 @@ extern "C" int mac_form_(int digits, int split, int columns, int staging, int ro
   return (int)mac_form(MacKnobs{digits != 0, split != 0, columns, staging}, rows, K, NC, dual != 0);
 }
 extern "C" int mask_skips_(long long count, int n, int warps, int sms) { return mask_skips(count, n, warps, sms); }
+extern "C" int compact_skips_(int n, int filled) { return compact_skips(n, filled); }
 """
 MAC_FORMS = ("generic", "smem", "ring", "bulk", "short", "digits")
 RING_FORMS = ("tile", "offsets", "outputs", "digits")

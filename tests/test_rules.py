@@ -108,3 +108,8 @@ def test_mask_polynomials_skip_where_many_warps_are_empty():
     assert skips(2752, 8192, 18) and skips(2048, 8192, 51)
     assert not skips(2048, 8192, 52) and not skips(1920, 8192, 64)   # nearly full
     assert not skips(2, 8192, 4) and not skips(37, 8192, 4) and skips(38, 8192, 4)   # one wave
+
+
+def test_compact_form_skips_where_half_of_the_groups_are_empty():
+    skips = rules_lib.load().compact_skips_
+    assert [bool(skips(8192, f)) for f in (1, 128, 129, 256)] == [True, True, False, False]
