@@ -1324,6 +1324,15 @@ extern "C" int he_linear_backward(PencilCtx* ctx, const PencilPlan* Pd, const Pe
   return PENCIL_OK;
 }
 
+// Decryption's transforms of the plan's outputs.
+static cudaError_t launch_decrypt(PencilCtx* ctx, const PencilPlan* P, ModeDecrypt::Params D, cudaStream_t s) {
+  PROF(ctx, PENCIL_K_INTT_DECRYPT, s);
+  D.groups = P->pk_y.groups;
+  const int count = (int)P->out_count(), first = (int)P->out_first();
+  return compact_skips(ctx->n, P->pk_y.filled) ? ntt<ModeDecryptFew, true>(ctx->dev, D, count, s, first)
+                                               : ntt<ModeDecrypt, true>(ctx->dev, D, count, s, first);
+}
+
 extern "C" int decrypt_to_share(PencilCtx* ctx, const PencilSecretKey* sk, const PencilPlan* P,
                                 const uint64_t* ct_out, uint64_t* y1, int32_t check_noise, void* ws, size_t ws_bytes,
                                 void* stream) {
@@ -1337,10 +1346,7 @@ extern "C" int decrypt_to_share(PencilCtx* ctx, const PencilSecretKey* sk, const
   D.sk = sk->sk;
   D.out = reinterpret_cast<u64*>(ws);
   D.skip_c0 = 0;
-  {
-    PROF(ctx, PENCIL_K_INTT_DECRYPT, s);
-    CUDA_TRY((ntt<ModeDecrypt, true>(ctx->dev, D, (int)P->out_count(), s, (int)P->out_first())));
-  }
+  CUDA_TRY(launch_decrypt(ctx, P, D, s));
   {
     PROF(ctx, PENCIL_K_DECRYPT_COMBINE, s);
     CUDA_TRY(launch_decrypt_combine(ctx->dev, P->pk_y, P->acc_y, D.out, (int)P->out_first(), (int)P->out_count(),
@@ -1384,10 +1390,7 @@ extern "C" int decrypt_compact_to_share(PencilCtx* ctx, const PencilSecretKey* s
   D.sk = sk->sk;
   D.out = reinterpret_cast<u64*>(ws);
   D.skip_c0 = 1;
-  {
-    PROF(ctx, PENCIL_K_INTT_DECRYPT, s);
-    CUDA_TRY((ntt<ModeDecrypt, true>(ctx->dev, D, (int)P->out_count(), s, (int)P->out_first())));
-  }
+  CUDA_TRY(launch_decrypt(ctx, P, D, s));
   {
     PROF(ctx, PENCIL_K_DECRYPT_COMBINE, s);
     CUDA_TRY(launch_decrypt_combine(ctx->dev, P->pk_y, P->acc_y, D.out, (int)P->out_first(), (int)P->out_count(),
@@ -1872,6 +1875,7 @@ extern "C" int pencil_batch_commit(PencilBatch* B, const PencilSecretKey* sk, vo
     dec[l].sk = sk->sk;
     dec[l].out = yres;
     dec[l].skip_c0 = 0;
+    dec[l].groups = P->pk_y.groups;
     comb[l] = CombineP{P->pk_y, P->acc_y, yres, u.y1};
     for (long long i = 0; i < P->ct_out; ++i) it_out.push_back(make_int2(l, (int)i));
     for (long long i = 0; i < prep[l].n_in + P->ct_out; ++i) it_prep.push_back(make_int2(l, (int)i));

@@ -1388,6 +1388,7 @@ struct ModeDecrypt {
     const ulonglong2* sk;   // [L][N] with companions, then [L][N] split
     u64* out;               // [count][L][N]
     int skip_c0;
+    const unsigned char* groups;   // ModeDecryptFew: the output packing's (Packing::groups)
   };
   using Pre = NoPre;
   static __device__ __forceinline__ void rebase(Params&, u64) {}
@@ -1429,6 +1430,13 @@ struct ModeDecrypt {
                                                int limb, int e, u64 x) {
     P.out[limb_off(poly, limb, c.L, N) + e] = x;   // x = N^{-1} qtil INTT, canonical
   }
+};
+
+// The same for polynomials of which many groups of 32 coefficients carry no output
+// (compact_skips): the CRT pass reads no residue of those, and none is written.
+struct ModeDecryptFew : ModeDecrypt {
+  static constexpr bool kFewOutputs = true;
+  static __device__ __forceinline__ bool occupied(const Params& P, int group) { return __ldg(P.groups + group) != 0; }
 };
 
 // MO, compact send form of returned ciphertexts: INTT(c0) and, at the
@@ -1601,7 +1609,8 @@ cudaError_t launch_ntt_multi(const DevCtx& ctx, const typename Mode::Params* Ps,
   PENCIL_NTT_INST1(SPEC, LOGN, LOGE, ModeEncryptPk, false, FOLD) \
   PENCIL_NTT_INST1(SPEC, LOGN, LOGE, ModeCompact, true, FOLD)    \
   PENCIL_NTT_INST1(SPEC, LOGN, LOGE, ModeCompactFew, true, FOLD) \
-  PENCIL_NTT_INST1(SPEC, LOGN, LOGE, ModeDecrypt, true, FOLD)
+  PENCIL_NTT_INST1(SPEC, LOGN, LOGE, ModeDecrypt, true, FOLD)    \
+  PENCIL_NTT_INST1(SPEC, LOGN, LOGE, ModeDecryptFew, true, FOLD)
 // Radix 2^4 and 2^5 register blocks for one N and one engine.
 #define PENCIL_NTT_INSTANTIATE(SPEC, LOGN, FOLD) \
   PENCIL_NTT_INST_E(SPEC, LOGN, 4, FOLD)         \

@@ -45,6 +45,8 @@ def test_compact_form_is_the_output_coefficients(log_n, limbs, bits, radix, arit
         assert torch.equal(row[at.clamp(max=row.numel() - 1)], c0c[j])
         assert torch.unique(c0c[j]).numel() == s.out_elems   # (uniform residues: no two alike)
     ws, y, z = plan.new_ws(s.ws_decrypt), *(torch.empty(s.out_elems, dtype=torch.int64, device="cuda") for _ in range(2))
+    ws.fill_(-1)   # (residues of empty groups are not written, and not read)
     he.decrypt_to_share(ctx, sk, plan, ct, y, False, ws)
+    ws.fill_(7)
     he.decrypt_compact_to_share(ctx, sk, plan, ct, c0c, z, False, ws)
     assert torch.equal(y, z)
